@@ -200,6 +200,11 @@ struct Elem<__nv_bfloat16> {
   __device__ __forceinline__ static uint32_t sign(const void *p, int64_t i) {
     return ((const uint16_t *)p)[i] >> 15;
   }
+  // sign bits of the 8 elements of 16 bytes, element j in bit j
+  __device__ __forceinline__ static uint32_t signs(const uint4 &u) {
+    auto two = [](uint32_t w) { return ((w >> 15) & 1u) | ((w >> 30) & 2u); };
+    return two(u.x) | two(u.y) << 2 | two(u.z) << 4 | two(u.w) << 6;
+  }
   // 16 bytes -> 8 floats as 4 float2 pairs (element 2j in .x, 2j+1 in .y)
   __device__ __forceinline__ static void unpack(const uint4 &u, float2 *f) {
     f[0] = bf16x2_to_float2(u.x);
@@ -221,6 +226,10 @@ struct Elem<float> {
   }
   __device__ __forceinline__ static uint32_t sign(const void *p, int64_t i) {
     return ((const uint32_t *)p)[i] >> 31;
+  }
+  // sign bits of the 4 elements of 16 bytes, element j in bit j
+  __device__ __forceinline__ static uint32_t signs(const uint4 &u) {
+    return u.x >> 31 | (u.y >> 31) << 1 | (u.z >> 31) << 2 | (u.w >> 31) << 3;
   }
   // 16 bytes -> 4 floats as 2 float2 pairs
   __device__ __forceinline__ static void unpack(const uint4 &u, float2 *f) {

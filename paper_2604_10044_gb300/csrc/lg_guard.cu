@@ -32,20 +32,6 @@ __global__ void begin_step_kernel(lg_cache c) {
     c.len[b] = n + 1;
 }
 
-// sketch word w of a row: sign bits of elements [32w, 32w+32) of the row flattened [H_kv][d]
-template <typename T>
-__device__ __forceinline__ uint32_t sketch_word(const void *row_base, int64_t head_stride, int d,
-                                                int w) {
-  uint32_t bits = 0;
-#pragma unroll 4
-  for (int j = 0; j < 32; ++j) {
-    const int e = w * 32 + j;
-    const int h = e / d, x = e % d;
-    bits |= Elem<T>::sign(row_base, (int64_t)h * head_stride + x) << j;
-  }
-  return bits;
-}
-
 // Blocks [0, row_blocks): one thread per 16-byte chunk of a new row, written to slot
 // len[b] - 1.  Blocks [row_blocks, row_blocks + batch) when the guard layer is in the call:
 // the sketch of that layer's new V row (read from v_new [n_layers][b][H_kv][d]), a warp per
@@ -113,31 +99,85 @@ __global__ void append_kernel(lg_cache c, int layer0, int n_layers, const uint4 
   }
 }
 
-// sketches of rows [0, len[b]) of the guard layer, read from the cache
-template <typename T>
-__global__ void sketch_build_kernel(lg_cache c, int guard_layer, int max_len) {
+// Sketches of rows [0, len[b]) of the guard layer, read from the cache.  Bound by HBM: every V
+// row of the layer is read once.  A warp's load covers 512 contiguous bytes of one kv-head
+// (kRows whole rows), 16 bytes a lane, and kSketchLoads such loads are in flight before the
+// first is used; a lane packs the sign bits of its 4 or 8 elements and the kLanes lanes of a
+// 32-element word join theirs by shuffles.  The loads of a warp are consecutive (row block,
+// kv-head) items, kv-head fastest, so the words of a row leave a warp together; lane j of a
+// word's lanes stores the words of items j, j + kLanes, ...
+// (GB300, 8 prompts of 32768 rows, 8 kv-heads of 128 bf16, 570 MB: 448.3 us -> 94.2 us, 6.05 TB/s; a thread per
+// word with 32 2-byte loads, each load of a warp over 32 rows, kept L1 99 % busy and HBM at 16 %.)
+constexpr int kSketchThreads = 256;
+constexpr int kSketchLoads = 8;
+
+template <typename T, int D>
+__global__ void __launch_bounds__(kSketchThreads) sketch_build_kernel(lg_cache c, int guard_layer,
+                                                                       int max_len) {
   // no early start of the kernel after this one: the detect kernel reads sketch rows before its
   // dependency wait and checks only the length, its synced length and the newest row, which this
   // kernel leaves unchanged while it may rewrite every other row
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  constexpr int kCpr = D * Elem<T>::kSize / 16;  // 16-byte chunks (lanes) of a row
+  constexpr int kRows = 32 / kCpr;               // rows of a warp's load
+  constexpr int kEpl = 16 / Elem<T>::kSize;      // elements of a lane
+  constexpr int kLanes = 32 / kEpl;              // lanes of a word
   const int b = blockIdx.y;
-  if (status_bad(c.dev_status)) return;
   const int n = c.len[b];
+  const int64_t off = c.seq_off[b];
+  if (status_bad(c.dev_status)) return;
   if (n > max_len) {
     if (threadIdx.x == 0 && blockIdx.x == 0) set_status(c.dev_status, LG_ERR_CAPACITY);
     return;
   }
-  const int nwords = c.H_kv * c.d / 32;
-  const int64_t total = (int64_t)n * nwords;
-  const T *base = (const T *)c.v + ((int64_t)guard_layer * c.H_kv * c.S_total + c.seq_off[b]) * c.d;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = t / nwords;
-    const int w = (int)(t % nwords);
-    c.sketch[(c.seq_off[b] + i) * nwords + w] =
-        sketch_word<T>(base + i * c.d, c.S_total * c.d, c.d, w);
+  const int nwords = c.H_kv * D / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int row_l = lane / kCpr, ch = lane % kCpr;
+  const int sub = lane % kLanes;  // this lane's place among the lanes of its word
+  const int64_t head_stride = c.S_total * kCpr;  // in 16-byte chunks
+  const uint4 *base = reinterpret_cast<const uint4 *>(c.v) +
+                      ((int64_t)guard_layer * c.H_kv * c.S_total + off) * kCpr;
+  uint32_t *sk = c.sketch + off * nwords + ch / kLanes;
+  const int64_t items = (int64_t)((n + kRows - 1) / kRows) * c.H_kv;
+  const int64_t stride = (int64_t)gridDim.x * (kSketchThreads / 32) * kSketchLoads;
+  for (int64_t it0 = ((int64_t)blockIdx.x * (kSketchThreads / 32) + warp) * kSketchLoads;
+       it0 < items; it0 += stride) {
+    uint4 u[kSketchLoads];
+    int row[kSketchLoads], head[kSketchLoads];  // row -1: nothing to read
+    int rb = (int)(it0 / c.H_kv), h = (int)(it0 - (int64_t)rb * c.H_kv);
+#pragma unroll
+    for (int k = 0; k < kSketchLoads; ++k) {
+      const int r = rb * kRows + row_l;
+      row[k] = r < n && it0 + k < items ? r : -1;
+      head[k] = h;
+      u[k] = row[k] >= 0 ? __ldcs(base + h * head_stride + (int64_t)r * kCpr + ch)
+                         : make_uint4(0u, 0u, 0u, 0u);
+      if (++h == c.H_kv) {
+        h = 0;
+        ++rb;
+      }
+    }
+#pragma unroll
+    for (int k0 = 0; k0 < kSketchLoads; k0 += kLanes) {
+      uint32_t word = 0;
+      int r = -1, hw = 0;
+#pragma unroll
+      for (int j = 0; j < kLanes; ++j) {
+        const int k = k0 + j;
+        uint32_t bits = Elem<T>::signs(u[k]) << (sub * kEpl);
+#pragma unroll
+        for (int o = 1; o < kLanes; o <<= 1) bits |= __shfl_xor_sync(0xffffffffu, bits, o);
+        if (sub == j) {
+          word = bits;
+          r = row[k];
+          hw = head[k];
+        }
+      }
+      if (r >= 0) sk[(int64_t)r * nwords + hw * (D / 32)] = word;
+    }
   }
 }
+static_assert(kSketchLoads % 8 == 0, "whole groups of word lanes (4 in bf16, 8 in fp32)");
 
 __global__ void state_init_kernel(int batch, lg_guard_state *state, int t_gen0) {
   pdl_enter();
@@ -1137,20 +1177,26 @@ cudaError_t launch_append(const lg_cache &c, int layer0, int n_layers, const voi
   return cudaGetLastError();
 }
 
-cudaError_t launch_sketch_build(const lg_cache &c, int guard_layer, int max_len, cudaStream_t s) {
-  const int nwords = c.H_kv * c.d / 32;
-  int64_t per_seq = (int64_t)max_len * nwords;
-  int gx = (int)((per_seq + 255) / 256);
-  if (gx > 1024) gx = 1024;
+template <typename T, int D>
+static cudaError_t launch_sketch_typed(const lg_cache &c, int guard_layer, int max_len,
+                                       cudaStream_t s) {
+  constexpr int rows = 32 * 16 / (D * Elem<T>::kSize);
+  constexpr int64_t per_cta = (int64_t)kSketchThreads / 32 * kSketchLoads;
+  const int64_t items = ((int64_t)max_len + rows - 1) / rows * c.H_kv;
+  int64_t gx = (items + per_cta - 1) / per_cta;
+  if (gx > 4096) gx = 4096;
   if (gx < 1) gx = 1;
-  dim3 grid(gx, c.batch);
-  if (c.dtype == LG_BF16) {
-    LG_TRY(launch_pdl(sketch_build_kernel<__nv_bfloat16>, grid, 256, 0, s, c, guard_layer,
-                      max_len));
-  } else {
-    LG_TRY(launch_pdl(sketch_build_kernel<float>, grid, 256, 0, s, c, guard_layer, max_len));
-  }
+  LG_TRY(launch_pdl(sketch_build_kernel<T, D>, dim3((unsigned)gx, c.batch), kSketchThreads, 0, s, c,
+                    guard_layer, max_len));
   return cudaGetLastError();
+}
+
+cudaError_t launch_sketch_build(const lg_cache &c, int guard_layer, int max_len, cudaStream_t s) {
+  if (c.dtype == LG_BF16)
+    return c.d == 128 ? launch_sketch_typed<__nv_bfloat16, 128>(c, guard_layer, max_len, s)
+                      : launch_sketch_typed<__nv_bfloat16, 64>(c, guard_layer, max_len, s);
+  return c.d == 128 ? launch_sketch_typed<float, 128>(c, guard_layer, max_len, s)
+                    : launch_sketch_typed<float, 64>(c, guard_layer, max_len, s);
 }
 
 cudaError_t launch_state_init(const lg_cache &c, lg_guard_state *state, int t_gen0, cudaStream_t s) {
