@@ -141,6 +141,13 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
                : "memory");
 }
 
+// 4-byte asynchronous copy global -> shared, in the same commit groups
+__device__ __forceinline__ void cp_async4(void *smem_dst, const void *gmem_src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(smem_dst)),
+               "l"(gmem_src)
+               : "memory");
+}
+
 __device__ __forceinline__ void cp_async_commit() {
   asm volatile("cp.async.commit_group;" ::: "memory");
 }

@@ -106,8 +106,9 @@ __global__ void append_kernel(lg_cache c, int layer0, int n_layers, const uint4 
 // 32-element word join theirs by shuffles.  The loads of a warp are consecutive (row block,
 // kv-head) items, kv-head fastest, so the words of a row leave a warp together; lane j of a
 // word's lanes stores the words of items j, j + kLanes, ...
-// (GB300, 8 prompts of 32768 rows, 8 kv-heads of 128 bf16, 570 MB: 448.3 us -> 94.2 us, 6.05 TB/s; a thread per
-// word with 32 2-byte loads, each load of a warp over 32 rows, kept L1 99 % busy and HBM at 16 %.)
+// (GB300, 8 prompts of 32768 rows, 8 kv-heads of 128 bf16, 570 MB: 448.3 -> 94.2 us, 6.05 TB/s;
+// a thread per word with 32 2-byte loads, each load of a warp over 32 rows, kept L1 99 % busy
+// and HBM at 16 %.)
 constexpr int kSketchThreads = 256;
 constexpr int kSketchLoads = 8;
 
@@ -928,25 +929,253 @@ __device__ __forceinline__ uint64_t h2o_key(float score, int32_t pos) {
 }
 
 constexpr int kH2OThreads = 256;
-constexpr int kH2OTile = 32;
-constexpr int kH2OMaxQ = 2 * kH2OTile * 32 / kH2OThreads;  // 16-byte chunks per thread, 512 B rows
+constexpr int kH2OWarps = kH2OThreads / 32;
+constexpr int kH2OScan = 8;         // rows a thread has in flight in a scan of a stream
+constexpr int kCutWindow = 2048;    // source rows whose kept ones are listed at once
+constexpr int kCutHalf = 8192;      // bytes of K (and of V) of one tile of destination rows
+constexpr int kCutMaxRows = kCutHalf / 128;                          // rows of a tile, d = 64 bf16
+constexpr int kCutStage = 2 * kCutHalf + 2 * kCutMaxRows * 4;        // K, V, scores, positions
+constexpr int kCutStages = 3;       // ring of tiles: two gathers in flight, one store
+constexpr int kCutChunks = kCutHalf / 16 / kH2OThreads;              // 16-byte chunks, per tensor
+constexpr int kCutBins = 2048;      // bins of an 11-bit digit, in the ring's memory
+constexpr size_t kCutSmem = (size_t)kCutStages * kCutStage + kCutWindow * sizeof(uint16_t);
+static_assert(kCutWindow == kH2OThreads * kH2OScan, "a window is one scan round of the CTA");
+static_assert(kCutBins * 4 <= kCutStages * kCutStage && kCutBins == kH2OThreads * 8, "digit bins");
 
-// One CTA per (sequence, layer, kv-head) stream of a sequence over budget.
 // kMode kEvictH2O: keep the recent half of the budget and the highest (score, pos) rows.
 // kMode kEvictStreaming: keep positions < n_sink and the budget - n_sink most recent ones.
 enum { kEvictH2O = 0, kEvictStreaming = 1 };
 
+struct EvictStream {
+  float *sc;             // scores of the stream's slots
+  int32_t *ps;           // their positions
+  unsigned char *K, *V;  // their rows
+  int n, B;              // rows in use, budget
+  int32_t thrp;          // recent: position above this one
+  int n_sink;
+  template <int kMode>
+  __device__ __forceinline__ bool kept_always(int32_t pos) const {
+    return pos > thrp || (kMode == kEvictStreaming && pos < n_sink);
+  }
+};
+
+// One digit of a descending radix select over the CTA: the bins (kCutBins counts in shared
+// memory) are searched from the highest for the one that holds the rem-th value; *digit is that
+// bin, *left how many are still wanted in it and *in its count.  Every thread calls it.
+__device__ __forceinline__ void select_bin(const unsigned *hist, int rem, int *wtot, int *digit,
+                                           int *left, int *in, int tid) {
+  const int lane = tid & 31, warp = tid >> 5;
+  const int hi = kCutBins - 1 - 8 * tid;  // thread 0 takes the highest eight bins
+  int own = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) own += hist[hi - j];
+  int upto = own;  // this thread's bins and all above, within the warp
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xffffffffu, upto, o);
+    if (lane >= o) upto += x;
+  }
+  if (lane == 31) wtot[warp] = upto;
+  __syncthreads();
+  for (int w = 0; w < warp; ++w) upto += wtot[w];
+  int above = upto - own;
+  if (above < rem && rem <= upto) {
+    for (int j = 0; j < 8; ++j) {
+      const int c = hist[hi - j];
+      if (above + c >= rem) {
+        *digit = hi - j;
+        *left = rem - above;
+        *in = c;
+        break;
+      }
+      above += c;
+    }
+  }
+  __syncthreads();
+}
+
+// The key of the k-th highest (score, position) among the stream's rows outside the recent ones
+// (k >= 1, at least k of them): a radix select of 11, 11 and 10 bits over the score's
+// order-preserving bits, then over the positions of the rows that share the k-th score if not
+// all of them are wanted.  Each digit is one scan of the stream (from L2) into bins in shared
+// memory and a parallel search of the bins.
+__device__ __forceinline__ unsigned long long kth_key(const EvictStream &e, int k, unsigned *hist,
+                                                      int tid) {
+  __shared__ int s_wtot[kH2OWarps];
+  __shared__ int s_digit, s_left, s_in;
+  uint32_t score = 0, pos = 0;  // the bits fixed so far
+  int rem = k;
+  for (int pass = 0; pass < 6; ++pass) {
+    const int part = pass % 3;
+    const int shift = part == 0 ? 21 : (part == 1 ? 10 : 0);
+    const uint32_t bins = part == 2 ? 1024u : 2048u;
+    const uint32_t mask = part == 0 ? 0u : (part == 1 ? 0xffe00000u : 0xfffffc00u);
+    for (int i = tid; i < kCutBins; i += kH2OThreads) hist[i] = 0;
+    __syncthreads();
+    for (int i0 = tid; i0 < e.n; i0 += kH2OThreads * kH2OScan) {
+      uint32_t sk[kH2OScan];
+      int32_t pk[kH2OScan];
+#pragma unroll
+      for (int u = 0; u < kH2OScan; ++u) {
+        const int i = i0 + u * kH2OThreads;
+        pk[u] = i < e.n ? e.ps[i] : 0x7fffffff;
+        sk[u] = i < e.n ? (uint32_t)(h2o_key(e.sc[i], 0) >> 32) : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < kH2OScan; ++u) {
+        if (i0 + u * kH2OThreads >= e.n || pk[u] > e.thrp) continue;
+        const uint32_t v = pass < 3 ? sk[u] : (uint32_t)pk[u];
+        const uint32_t fixed = pass < 3 ? score : pos;
+        if ((pass < 3 || sk[u] == score) && (v & mask) == fixed)
+          atomicAdd(&hist[(v >> shift) & (bins - 1u)], 1u);
+      }
+    }
+    __syncthreads();
+    select_bin(hist, rem, s_wtot, &s_digit, &s_left, &s_in, tid);
+    rem = s_left;
+    (pass < 3 ? score : pos) |= (uint32_t)s_digit << shift;
+    const bool all = pass >= 2 && rem == s_in;  // every row with these bits is wanted
+    __syncthreads();
+    if (pass >= 2 && all) break;
+  }
+  return (unsigned long long)score << 32 | pos;
+}
+
+// Ordered in-place cut of one stream by one CTA.  Windows of kCutWindow source rows: the CTA
+// lists the window's kept rows (ballots and a prefix over the warps), then moves them to the
+// slots after those kept before, in tiles of kCutHalf bytes of K and of V: 16-byte asynchronous
+// copies into a ring of stages two tiles ahead, scores and positions with 4-byte ones, then a
+// bulk store of each tensor's contiguous slots.  In place without further ordering as in
+// compact_kernel: destination slots ascend and never pass their sources, so a store (issued
+// once its tile's copies have landed) only overwrites rows that are already in shared memory or
+// not kept, and a later window's rows, scores and positions lie above every slot written.
 template <int kMode>
-__global__ void __launch_bounds__(kH2OThreads) evict_kernel(lg_cache c, const int32_t *budget,
-                                                            const int32_t *pos_now, int max_len,
-                                                            int n_sink) {
+__device__ __forceinline__ void evict_cut(const EvictStream &e, unsigned long long kth, bool by_key,
+                                          int rb, unsigned char *smem, int tid) {
+  __shared__ int s_wtot[kH2OWarps];
+  __shared__ int s_first;  // first listed row that changes its slot
+  uint16_t *list = reinterpret_cast<uint16_t *>(smem + kCutStages * kCutStage);
+  const int lane = tid & 31, warp = tid >> 5;
+  const int cpr = rb >> 4, T = kCutHalf / rb;
+  int c_row[kCutChunks], c_off[kCutChunks];
+#pragma unroll
+  for (int k = 0; k < kCutChunks; ++k) {
+    const int ci = k * kH2OThreads + tid;
+    c_row[k] = ci / cpr;
+    c_off[k] = (ci - c_row[k] * cpr) * 16;
+  }
+  int out = 0;  // rows kept so far
+  for (int w0 = 0; w0 < e.n; w0 += kCutWindow) {
+    // the window's kept rows: warp w looks at 256 consecutive rows, 32 at a time
+    unsigned bal[kH2OScan];
+    int mine = 0;
+    {
+      int32_t pk[kH2OScan];
+      float sk[kH2OScan];
+#pragma unroll
+      for (int u = 0; u < kH2OScan; ++u) {
+        const int i = w0 + warp * 32 * kH2OScan + u * 32 + lane;
+        pk[u] = i < e.n ? e.ps[i] : 0;
+        sk[u] = kMode == kEvictH2O && i < e.n ? e.sc[i] : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < kH2OScan; ++u) {
+        const int i = w0 + warp * 32 * kH2OScan + u * 32 + lane;
+        const bool keep = i < e.n && (e.kept_always<kMode>(pk[u]) ||
+                                      (by_key && h2o_key(sk[u], pk[u]) >= kth));
+        bal[u] = __ballot_sync(0xffffffffu, keep);
+        mine += __popc(bal[u]);
+      }
+    }
+    if (lane == 0) s_wtot[warp] = mine;
+    if (tid == 0) s_first = kCutWindow;
+    __syncthreads();
+    int at = 0, cnt = 0;
+    for (int w = 0; w < kH2OWarps; ++w) {
+      at += w < warp ? s_wtot[w] : 0;
+      cnt += s_wtot[w];
+    }
+    int first = kCutWindow;
+#pragma unroll
+    for (int u = 0; u < kH2OScan; ++u) {
+      const int r = warp * 32 * kH2OScan + u * 32 + lane;  // row within the window
+      if ((bal[u] >> lane) & 1u) {
+        const int j = at + __popc(bal[u] & ((1u << lane) - 1u));
+        list[j] = (uint16_t)r;
+        if (w0 + r != out + j) first = min(first, j);
+      }
+      at += __popc(bal[u]);
+    }
+    first = (int)__reduce_min_sync(0xffffffffu, (unsigned)first);
+    if (lane == 0 && first < kCutWindow) atomicMin(&s_first, first);
+    __syncthreads();
+    const int j0 = min(s_first, cnt);
+    const int n_tiles = (cnt - j0 + T - 1) / T;
+    auto gather = [&](int p) {
+      const int t0 = j0 + p * T, rows = min(T, cnt - t0);
+      unsigned char *st = smem + (p % kCutStages) * kCutStage;
+#pragma unroll
+      for (int k = 0; k < kCutChunks; ++k)
+        if (c_row[k] < rows) {
+          const int64_t src = (int64_t)(w0 + list[t0 + c_row[k]]) * rb + c_off[k];
+          unsigned char *d = st + (k * kH2OThreads + tid) * 16;
+          cp_async16(d, e.K + src);
+          cp_async16(d + kCutHalf, e.V + src);
+        }
+      if (tid < rows) {
+        const int src = w0 + list[t0 + tid];
+        cp_async4(st + 2 * kCutHalf + tid * 4, e.sc + src);
+        cp_async4(st + 2 * kCutHalf + (kCutMaxRows + tid) * 4, e.ps + src);
+      }
+    };
+    for (int p = 0; p < kCutStages - 1; ++p) {
+      if (p < n_tiles) gather(p);
+      cp_async_commit();  // one group per tile, empty past the end (uniform group counting)
+    }
+    for (int i = 0; i < n_tiles; ++i) {
+      cp_async_wait<kCutStages - 2>();  // this thread's copies of tile i have landed
+      fence_proxy_async_smem();
+      if (tid == 0) bulk_wait_read_all();  // tile i-1's stores have read their stage
+      __syncthreads();
+      const int t0 = j0 + i * T, rows = min(T, cnt - t0);
+      const unsigned char *st = smem + (i % kCutStages) * kCutStage;
+      if (tid == 0) {
+        bulk_store(e.K + (int64_t)(out + t0) * rb, st, (uint32_t)(rows * rb));
+        bulk_store(e.V + (int64_t)(out + t0) * rb, st + kCutHalf, (uint32_t)(rows * rb));
+        bulk_commit();
+      }
+      if (tid < rows) {
+        const float *s4 = reinterpret_cast<const float *>(st + 2 * kCutHalf);
+        e.sc[out + t0 + tid] = s4[tid];
+        e.ps[out + t0 + tid] = reinterpret_cast<const int32_t *>(s4)[kCutMaxRows + tid];
+      }
+      const int p = i + kCutStages - 1;  // into the stage tile i-1 used
+      if (p < n_tiles) gather(p);
+      cp_async_commit();
+    }
+    out += cnt;
+    // the next window's list and first copies reuse the list and the stages
+    if (tid == 0) bulk_wait_read_all();
+    __syncthreads();
+  }
+  if (tid == 0) bulk_wait_all();
+}
+
+// One CTA per (sequence, layer, kv-head) stream of a sequence over budget.  A cut of several rows
+// is bound by HBM (every kept row read and written once); one row over budget, the steady state,
+// by one scan of the stream's scores and positions.
+// (GB300, H2O cut of 512 streams from 8193 to 4096 rows of 128 bf16, 2.2 GB: 1370 -> 360 us,
+// 6.0 TB/s.  Before: eight 8-bit digits with a serial search of the bins, then 32-row tiles through
+// registers with four barriers each; DRAM 20 % busy.)
+template <int kMode>
+__global__ void __launch_bounds__(kH2OThreads, 4) evict_kernel(lg_cache c, const int32_t *budget,
+                                                               const int32_t *pos_now, int max_len,
+                                                               int n_sink) {
   pdl_enter();
-  __shared__ unsigned long long s_wbest[kH2OThreads / 32];
-  __shared__ int s_wslot[kH2OThreads / 32];
-  __shared__ int s_slot, s_count, s_out;
-  __shared__ unsigned int hist[256];
-  __shared__ unsigned long long s_prefix;
-  __shared__ int s_remaining;
+  extern __shared__ __align__(128) unsigned char s_cut[];
+  __shared__ unsigned long long s_wbest[kH2OWarps];
+  __shared__ int s_wslot[kH2OWarps];
+  __shared__ int s_slot, s_count;
   const int lh = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
   if (cta_status_bad(c.dev_status)) return;
   const int n = c.len[b], B = budget[b];
@@ -955,32 +1184,29 @@ __global__ void __launch_bounds__(kH2OThreads) evict_kernel(lg_cache c, const in
     if (tid == 0) set_status(c.dev_status, LG_ERR_CAPACITY);
     return;
   }
-  // recent: pos > thrp (H2O: the newest B/2 positions; streaming: the newest B - n_sink)
-  const int32_t thrp = pos_now[b] - (kMode == kEvictH2O ? B / 2 : B - n_sink);
   const int64_t o = (int64_t)lh * c.S_total + c.seq_off[b];
-  float *sc = c.h2o + o;
-  int32_t *ps = c.pos + o;
   const int rb = c.d * (c.dtype == LG_BF16 ? 2 : 4);
-  const int cpr = rb / 16;
-  uint4 *K4 = reinterpret_cast<uint4 *>((unsigned char *)c.k + o * rb);
-  uint4 *V4 = reinterpret_cast<uint4 *>((unsigned char *)c.v + o * rb);
+  EvictStream e;
+  e.sc = c.h2o + o;
+  e.ps = c.pos + o;
+  e.K = (unsigned char *)c.k + o * rb;
+  e.V = (unsigned char *)c.v + o * rb;
+  e.n = n;
+  e.B = B;
+  // recent: pos > thrp (H2O: the newest B/2 positions; streaming: the newest B - n_sink)
+  e.thrp = pos_now[b] - (kMode == kEvictH2O ? B / 2 : B - n_sink);
+  e.n_sink = n_sink;
 
-  // eviction order among the rows outside the protected set: lowest key first
-  auto evict_key = [&](int i) -> unsigned long long {
-    return kMode == kEvictH2O ? (unsigned long long)h2o_key(sc[i], ps[i])
-                              : (unsigned long long)(uint32_t)ps[i];
-  };
-  auto protected_row = [&](int i) -> bool {
-    return ps[i] > thrp || (kMode == kEvictStreaming && ps[i] < n_sink);
-  };
   auto refill = [&](int x) {  // slot x takes the last slot's row, score and position
+    const int cpr = rb >> 4;
+    uint4 *K4 = reinterpret_cast<uint4 *>(e.K), *V4 = reinterpret_cast<uint4 *>(e.V);
     for (int ch = tid; ch < cpr; ch += kH2OThreads) {
       K4[(int64_t)x * cpr + ch] = K4[(int64_t)(n - 1) * cpr + ch];
       V4[(int64_t)x * cpr + ch] = V4[(int64_t)(n - 1) * cpr + ch];
     }
     if (tid == 0) {
-      sc[x] = sc[n - 1];
-      ps[x] = ps[n - 1];
+      e.sc[x] = e.sc[n - 1];
+      e.ps[x] = e.ps[n - 1];
     }
   };
   if (kMode == kEvictStreaming && n == B + 1 && B > n_sink) {
@@ -990,9 +1216,9 @@ __global__ void __launch_bounds__(kH2OThreads) evict_kernel(lg_cache c, const in
     // mod (B - n_sink).  One check of that slot's position replaces the scan below, which
     // runs whenever the check fails (the same slot in every case the ring holds).
     const int w = B - n_sink;
-    const int64_t r = ((int64_t)thrp - ps[n_sink]) % w;
+    const int64_t r = ((int64_t)e.thrp - e.ps[n_sink]) % w;
     const int x = n_sink + (int)(r < 0 ? r + w : r);
-    if (ps[x] == thrp) {
+    if (e.ps[x] == e.thrp) {
       refill(x);
       return;
     }
@@ -1003,14 +1229,29 @@ __global__ void __launch_bounds__(kH2OThreads) evict_kernel(lg_cache c, const in
     // keeps each thread's lowest key with its slot, and a reduction picks the CTA's.
     unsigned long long best = ~0ull;
     int slot = -1;
-    for (int i = tid; i < n; i += kH2OThreads)
-      if (!protected_row(i)) {
-        const unsigned long long key = evict_key(i);
-        if (key < best) {
-          best = key;
-          slot = i;
+    for (int i0 = tid; i0 < n; i0 += kH2OThreads * kH2OScan) {
+      int32_t pk[kH2OScan];
+      float sk[kH2OScan];
+#pragma unroll
+      for (int u = 0; u < kH2OScan; ++u) {
+        const int i = i0 + u * kH2OThreads;
+        pk[u] = i < n ? e.ps[i] : 0x7fffffff;
+        sk[u] = kMode == kEvictH2O && i < n ? e.sc[i] : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < kH2OScan; ++u) {
+        const int i = i0 + u * kH2OThreads;
+        if (i < n && !e.kept_always<kMode>(pk[u])) {
+          const unsigned long long key = kMode == kEvictH2O
+                                             ? (unsigned long long)h2o_key(sk[u], pk[u])
+                                             : (unsigned long long)(uint32_t)pk[u];
+          if (key < best) {
+            best = key;
+            slot = i;
+          }
         }
       }
+    }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) {
       const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
@@ -1028,7 +1269,7 @@ __global__ void __launch_bounds__(kH2OThreads) evict_kernel(lg_cache c, const in
     if (tid == 0) {
       unsigned long long m = ~0ull;
       int x = -1;
-      for (int w = 0; w < kH2OThreads / 32; ++w)
+      for (int w = 0; w < kH2OWarps; ++w)
         if (s_wbest[w] < m) {
           m = s_wbest[w];
           x = s_wslot[w];
@@ -1041,106 +1282,29 @@ __global__ void __launch_bounds__(kH2OThreads) evict_kernel(lg_cache c, const in
     refill(x);
     return;
   }
-  if (kMode == kEvictStreaming) {
-    // closed form: sinks and the newest B - n_sink positions
-    if (tid == 0) s_out = 0;
-    __syncthreads();
-  }
-
-  // cut to B rows: recent rows plus the k = B - n_recent highest keys among the others
+  // cut to B rows: the protected rows (streaming: sinks and the newest B - n_sink positions),
+  // and for H2O the k = B - n_recent highest keys among the others
   int k = 0;
   unsigned long long kth = 0;
   if (kMode == kEvictH2O) {
-  if (tid == 0) s_count = 0;
-  __syncthreads();
-  int cnt_local = 0;
-  for (int i = tid; i < n; i += kH2OThreads) cnt_local += ps[i] > thrp;
-  atomicAdd(&s_count, cnt_local);
-  if (tid == 0) {
-    s_prefix = 0;
-    s_out = 0;
-  }
-  __syncthreads();
-  k = B - s_count;
-  unsigned long long mask = 0;
-  if (tid == 0) s_remaining = k;
-  for (int digit = 7; digit >= 0; --digit) {
-    hist[tid] = 0;
+    if (tid == 0) s_count = 0;
     __syncthreads();
-    const unsigned long long prefix = s_prefix;
-    for (int i = tid; i < n; i += kH2OThreads) {
-      if (ps[i] > thrp) continue;
-      const unsigned long long key = h2o_key(sc[i], ps[i]);
-      if ((key & mask) == prefix) atomicAdd(&hist[(key >> (8 * digit)) & 255u], 1u);
-    }
-    __syncthreads();
-    if (tid == 0) {
-      int rem = s_remaining, cum = 0, v = 255;
-      for (; v > 0; --v) {
-        if (cum + (int)hist[v] >= rem) break;
-        cum += hist[v];
-      }
-      s_remaining = rem - cum;
-      s_prefix = prefix | ((unsigned long long)v << (8 * digit));
-    }
-    mask |= 255ull << (8 * digit);
-    __syncthreads();
-  }
-  kth = s_prefix;  // key of the k-th highest non-recent row
-  }
-
-  // ordered compaction of K, V, score and pos over source tiles of kH2OTile rows
-  const int lane = tid & 31, warp = tid >> 5;
-  for (int t0 = 0; t0 < n; t0 += kH2OTile) {
-    __shared__ int s_dest[kH2OTile];
-    __shared__ int s_tile_kept;
-    if (warp == 0) {
-      const int i = t0 + lane;
-      bool keep = false;
-      if (i < n)
-        keep = protected_row(i) || (kMode == kEvictH2O && k > 0 && h2o_key(sc[i], ps[i]) >= kth);
-      const unsigned bal = __ballot_sync(0xffffffffu, keep);
-      s_dest[lane] = keep ? s_out + __popc(bal & ((1u << lane) - 1u)) : -1;
-      if (lane == 0) s_tile_kept = __popc(bal);
-    }
-    __syncthreads();
-    // each thread moves chunks of the kept rows of this tile
-    uint4 kv[kH2OMaxQ];
-    float scv = 0.f;
-    int32_t psv = 0;
-    const int nchunks = kH2OTile * cpr;  // per tensor
+    int recent = 0;
+    for (int i0 = tid; i0 < n; i0 += kH2OThreads * kH2OScan) {
 #pragma unroll
-    for (int q = 0; q < kH2OMaxQ; ++q) {
-      const int ci = q * kH2OThreads + tid;
-      const int tensor = ci / nchunks, rc = ci % nchunks;
-      const int r = rc / cpr, ch = rc % cpr;
-      if (tensor < 2 && s_dest[r] >= 0 && t0 + r != s_dest[r]) {
-        const uint4 *src = tensor ? V4 : K4;
-        kv[q] = src[(int64_t)(t0 + r) * cpr + ch];
+      for (int u = 0; u < kH2OScan; ++u) {
+        const int i = i0 + u * kH2OThreads;
+        recent += i < n && e.ps[i] > e.thrp;
       }
     }
-    if (tid < kH2OTile && s_dest[tid] >= 0) {
-      scv = sc[t0 + tid];
-      psv = ps[t0 + tid];
-    }
+    recent = __reduce_add_sync(0xffffffffu, recent);
+    if ((tid & 31) == 0) atomicAdd(&s_count, recent);
     __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kH2OMaxQ; ++q) {
-      const int ci = q * kH2OThreads + tid;
-      const int tensor = ci / nchunks, rc = ci % nchunks;
-      const int r = rc / cpr, ch = rc % cpr;
-      if (tensor < 2 && s_dest[r] >= 0 && t0 + r != s_dest[r]) {
-        uint4 *dst = tensor ? V4 : K4;
-        dst[(int64_t)s_dest[r] * cpr + ch] = kv[q];
-      }
-    }
-    if (tid < kH2OTile && s_dest[tid] >= 0) {
-      sc[s_dest[tid]] = scv;
-      ps[s_dest[tid]] = psv;
-    }
-    if (tid == 0) s_out += s_tile_kept;
-    __syncthreads();
+    k = B - s_count;
+    if (k > 0) kth = kth_key(e, k, reinterpret_cast<unsigned *>(s_cut), tid);
+    __syncthreads();  // the bins become stages
   }
+  evict_cut<kMode>(e, kth, k > 0, rb, s_cut, tid);
 }
 
 __global__ void h2o_len_kernel(lg_cache c, const int32_t *budget) {
@@ -1290,29 +1454,27 @@ cudaError_t launch_h2o_reset(const lg_cache &c, int max_len, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_h2o_evict(const lg_cache &c, const int32_t *budget, const int32_t *pos_now,
-                             int max_len, cudaStream_t s) {
-  LG_TRY(launch_pdl(evict_kernel<kEvictH2O>, dim3(c.L * c.H_kv, c.batch), kH2OThreads, 0, s, c,
-                    budget, pos_now, max_len, 0));
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+template <int kMode>
+static cudaError_t launch_evict(const lg_cache &c, const int32_t *budget, const int32_t *pos_now,
+                                int max_len, int n_sink, cudaStream_t s) {
+  LG_TRY(cudaFuncSetAttribute(evict_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)kCutSmem));
+  LG_TRY(launch_pdl(evict_kernel<kMode>, dim3(c.L * c.H_kv, c.batch), kH2OThreads, kCutSmem, s, c,
+                    budget, pos_now, max_len, n_sink));
+  LG_TRY(cudaGetLastError());
   LG_TRY(launch_pdl(h2o_len_kernel, (c.batch + 127) / 128, 128, 0, s, c, budget));
   return cudaGetLastError();
 }
 
-}  // namespace lg
-
-namespace lg {
+cudaError_t launch_h2o_evict(const lg_cache &c, const int32_t *budget, const int32_t *pos_now,
+                             int max_len, cudaStream_t s) {
+  return launch_evict<kEvictH2O>(c, budget, pos_now, max_len, 0, s);
+}
 
 cudaError_t launch_streaming_evict(const lg_cache &c, const int32_t *budget,
                                    const int32_t *pos_now, int n_sink, int max_len,
                                    cudaStream_t s) {
-  LG_TRY(launch_pdl(evict_kernel<kEvictStreaming>, dim3(c.L * c.H_kv, c.batch), kH2OThreads, 0, s,
-                    c, budget, pos_now, max_len, n_sink));
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  LG_TRY(launch_pdl(h2o_len_kernel, (c.batch + 127) / 128, 128, 0, s, c, budget));
-  return cudaGetLastError();
+  return launch_evict<kEvictStreaming>(c, budget, pos_now, max_len, n_sink, s);
 }
 
 }  // namespace lg
