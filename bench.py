@@ -560,7 +560,7 @@ def source_hash():
     DRAM-traffic summary holds the value for the code it was captured on"""
     import hashlib
     h = hashlib.sha256()
-    for f in ("lg_attend_mma.cu", "lg_common.cuh"):
+    for f in ("lg_attend_mma.cu", "lg_mma_tile.cuh", "lg_common.cuh"):
         with open(os.path.join(ROOT, "paper_2604_10044_gb300", "csrc", f)) as fh:
             h.update(code_only(fh.read()).encode())
     return h.hexdigest()

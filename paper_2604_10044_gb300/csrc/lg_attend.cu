@@ -411,7 +411,8 @@ static cudaError_t launch_typed(const AttendArgs &a, int64_t rows_total, void *o
   cudaError_t e;
   if (Elem<T>::kDtype == LG_BF16) {
     // tensor-core partial pass (lg_attend_mma.cu)
-    e = launch_attend_mma_partial(a, D, G, rows_total, s);
+    e = attend_cluster_takes(a) ? launch_attend_cluster(a, D, G, rows_total, s)
+                                   : launch_attend_mma_partial(a, D, G, rows_total, s);
     if (e != cudaSuccess) return e;
   } else {
     auto kp = attend_partial_kernel<T, D, G>;

@@ -1,5 +1,6 @@
 // Decode attention over a bf16 KV cache fused with the guard's per-head statistics (LoopGuard
-// Sec. 3.1, Eq. 1; statistics read by Sec. 5.2), on tensor cores.
+// Sec. 3.1, Eq. 1; statistics read by Sec. 5.2), on tensor cores: the pass for batches of more than
+// 64 sequences and the longest calls (lg_attend_cluster.cu takes the others).
 //
 // Persistent CTAs (one per SM) start on chunks blockIdx.x and blockIdx.x + gridDim.x and take
 // further chunks from a shared counter, each a run of consecutive rows of one (layer,
@@ -29,14 +30,14 @@
 
 #include "lg_common.cuh"
 #include "lg_internal.h"
+#include "lg_mma_tile.cuh"
 
 namespace lg {
 
 namespace {
 
-constexpr int kTile = 128;          // rows per tile (TMA box height)
-constexpr int kBoxBytes = kTile * 128;  // one box: 128 rows x 64 bf16
-constexpr int kConsumerWarps = 4;
+constexpr int kTile = 128;          // rows per tile
+static_assert(kTile == kTileRows, "a chunk is whole tiles");
 constexpr int kProducerWarp = kConsumerWarps;
 constexpr int kMergerWarp0 = kConsumerWarps + 1;
 constexpr int kMergers = 4;   // merger warps; ticket k goes to merger k % kMergers
@@ -44,21 +45,6 @@ constexpr int kThreads = (kConsumerWarps + 1 + kMergers) * 32;
 constexpr int kTickets = 2 * kMergers;  // finished chunks queued from the consumers to the mergers
                                         // (ticket k in slot k % kTickets, owned by merger k % 4)
 constexpr int kMaxChunkRows = 4096;  // chunk rows at most (the tail of a call is about one chunk)
-constexpr int kStagedSeqs = 256;     // lengths and offsets kept in shared memory up to this batch
-constexpr int kL2KeepBytes = 32 << 20;  // K/V a short pass leaves in L2 at normal priority
-
-template <int D>
-struct MmaCfg {
-  static constexpr int kHalves = D / 64;                      // boxes per row
-  static constexpr int kStageBytes = 2 * kHalves * kBoxBytes;  // K and V
-  static constexpr int kStages = D == 128 ? 3 : 6;
-  static constexpr int kRingBytes = kStages * kStageBytes;
-  // ticket buffers: room for one buffer of 8 heads; fewer heads fit more buffers
-  static constexpr int kMergeBytes = kConsumerWarps * 8 * (D + 8) * 4;
-  static constexpr int kQBytes = 8 * D * 2;  // a stage's query rows (up to 8 heads), bf16
-  static constexpr int kSmem = kRingBytes + kMergeBytes + kStages * kQBytes + 1024;  // + slack
-  static constexpr int kKSteps = D / 16;
-};
 
 // One ticket buffer: every consumer warp's chunk partial of the G real heads,
 // o as [warp][head][D + 4] (the padding spreads the fragment stores over all banks), then
@@ -78,56 +64,6 @@ __device__ __forceinline__ int arrive_acq_rel(int *p) {
   int old;
   asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(p) : "memory");
   return old;
-}
-
-// 2-D tensor copy of one box into shared memory, completing on `bar`, with an L2 eviction
-// policy (createpolicy) for the lines it brings in.
-__device__ __forceinline__ void tma_load_2d(void *smem_dst, const CUtensorMap *map, int x,
-                                                 int y, uint64_t *bar, uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      ".L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_addr(smem_dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar)), "l"(policy)
-      : "memory");
-}
-
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2,
-                                        uint32_t &r3) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-               : "r"(addr));
-}
-
-__device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t &r0, uint32_t &r1,
-                                              uint32_t &r2, uint32_t &r3) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-               : "r"(addr));
-}
-
-__device__ __forceinline__ void mma_bf16(float *d, uint32_t a0, uint32_t a1, uint32_t a2,
-                                         uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, "
-      "{%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
-  uint32_t d;
-  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
-  return d;
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t *>(&v);
-}
-
-// byte offset of 16-byte chunk c8 (0..7) of row r in a 128-byte-swizzled box
-__device__ __forceinline__ uint32_t swz(int r, int c8) {
-  return (uint32_t)(r * 128 + ((c8 ^ (r & 7)) << 4));
 }
 
 struct ChunkId {
@@ -582,15 +518,11 @@ attend_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
   }
 
   // -------------------------------------------------------------- consumers
-  const int g = lane >> 2, t4 = lane & 3;
-  const int mrow = lane & 7, msel = lane >> 3;  // ldmatrix: row within 8x8, matrix index
   ChunkId id;
   int n = 0, row0 = 0, rows = 0, ntiles = 0, suffix_lo = 0;
   int64_t lrow0 = 0;
   uint32_t qf[C::kKSteps][2];
-  float o[C::kKSteps][4];
-  float m2[2], l2[2], u2[2], sg2[2];
-  float *logits = a.logits;
+  WarpSums<D> acc;
   uint32_t tk = 0;        // tickets issued (the same count in every consumer warp)
   bool handoff = true;    // false once a buffer or ticket slot was not released in time
   for (uint32_t it = 0;; ++it) {
@@ -611,162 +543,19 @@ attend_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
       ntiles = (rows + kTile - 1) / kTile;
       suffix_lo = n - min(a.suffix_w, n);
       lrow0 = stage_lrow0[st];
-      // B fragments of q^T: head g (zero for padded heads), d = 16 ks + 2 t4 (+1, +8, +9)
-      const uint32_t *qp = reinterpret_cast<const uint32_t *>(qbuf + st * C::kQBytes) + g * (D / 2);
-#pragma unroll
-      for (int ks = 0; ks < C::kKSteps; ++ks) {
-        qf[ks][0] = g < G ? qp[ks * 8 + t4] : 0u;
-        qf[ks][1] = g < G ? qp[ks * 8 + 4 + t4] : 0u;
-      }
-#pragma unroll
-      for (int eb = 0; eb < C::kKSteps; ++eb) o[eb][0] = o[eb][1] = o[eb][2] = o[eb][3] = 0.f;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        m2[h] = -INFINITY;
-        l2[h] = u2[h] = sg2[h] = 0.f;
-      }
+      load_q<D, G>(qf, qbuf + st * C::kQBytes, lane);
+      acc.reset();
     }
-    unsigned char *stage = smem + (size_t)st * C::kStageBytes;
-    const uint32_t kbase = smem_addr(stage);
-    const uint32_t vbase = kbase + C::kHalves * kBoxBytes;
-    const int tile_rows = min(kTile, rows - t * kTile);
-    const int r_w = warp * 32;  // this warp's first row in the tile
-    if (tile_rows < r_w + 32) {
-      // ragged tail: zero the V rows past the end so that 0 * stale stays 0
-      for (int idx = lane; idx < 32 * C::kHalves * 8; idx += 32) {
-        const int rr = r_w + idx / (C::kHalves * 8);
-        const int hc = idx % (C::kHalves * 8);
-        if (rr >= tile_rows)
-          *reinterpret_cast<uint4 *>(stage + (C::kHalves + hc / 8) * kBoxBytes + rr * 128 +
-                                     (hc % 8) * 16) = make_uint4(0u, 0u, 0u, 0u);
-      }
-      __syncwarp();
-    }
-
-    // S^T for the warp's two 16-row blocks
-    float s[2][4];
-#pragma unroll
-    for (int mb = 0; mb < 2; ++mb) {
-      s[mb][0] = s[mb][1] = s[mb][2] = s[mb][3] = 0.f;
-      const int r = r_w + mb * 16 + (msel & 1) * 8 + mrow;
-#pragma unroll
-      for (int ks = 0; ks < C::kKSteps; ++ks) {
-        const int c8 = (ks & 3) * 2 + (msel >> 1);
-        uint32_t a0, a1, a2, a3;
-        ldsm_x4(kbase + (ks >> 2) * kBoxBytes + swz(r, c8), a0, a1, a2, a3);
-        mma_bf16(s[mb], a0, a1, a2, a3, qf[ks][0], qf[ks][1]);
-      }
-    }
-    // scale to log2 units, mask rows past the end; tile max per head (heads 2 t4, 2 t4 + 1)
-    float mx[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-    for (int mb = 0; mb < 2; ++mb)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int rl = r_w + mb * 16 + g + (j >> 1) * 8;  // row within the tile
-        const bool valid = rl < tile_rows;
-        s[mb][j] = valid ? s[mb][j] * a.qscale : -INFINITY;
-        mx[j & 1] = fmaxf(mx[j & 1], s[mb][j]);
-      }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 4));
-      mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 8));
-      mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 16));
-    }
-    const bool raise = mx[0] > m2[0] || mx[1] > m2[1];
-    if (__any_sync(0xffffffffu, raise)) {
-      float corr[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float mn = fmaxf(m2[h], mx[h]);
-        corr[h] = mn == m2[h] ? 1.f : exp2f(m2[h] - mn);
-        u2[h] = l2[h] > 0.f ? corr[h] * (u2[h] + (m2[h] - mn) * l2[h]) : 0.f;
-        l2[h] *= corr[h];
-        sg2[h] *= corr[h];
-        m2[h] = mn;
-      }
-#pragma unroll
-      for (int eb = 0; eb < C::kKSteps; ++eb) {
-        o[eb][0] *= corr[0];
-        o[eb][1] *= corr[1];
-        o[eb][2] *= corr[0];
-        o[eb][3] *= corr[1];
-      }
-    }
-    // probabilities, sums, and P^T fragments
-    uint32_t pb[2][2], pl[2][2];
-#pragma unroll
-    for (int mb = 0; mb < 2; ++mb) {
-      float p[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int h = j & 1;
-        const int rl = r_w + mb * 16 + g + (j >> 1) * 8;
-        const bool valid = rl < tile_rows;
-        p[j] = valid ? exp2f(s[mb][j] - m2[h]) : 0.f;
-        if (valid) {
-          l2[h] += p[j];
-          u2[h] += p[j] * (s[mb][j] - m2[h]);
-          if (row0 + t * kTile + rl >= suffix_lo) sg2[h] += p[j];
-        }
-      }
-      if (logits) {
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          const int rl = r_w + mb * 16 + g + half * 8;
-          if (rl < tile_rows) {
-            float *dst = logits + (lrow0 + t * kTile + rl) * G;
-            if (G % 2 == 0) {
-              // heads 2 t4 and 2 t4 + 1 side by side: one 8-byte store (rows of an even G
-              // start 8-byte aligned)
-              if (2 * t4 < G)
-                *reinterpret_cast<float2 *>(dst + 2 * t4) =
-                    make_float2(s[mb][half * 2], s[mb][half * 2 + 1]);
-            } else {
-              if (2 * t4 < G) dst[2 * t4] = s[mb][half * 2];
-              if (2 * t4 + 1 < G) dst[2 * t4 + 1] = s[mb][half * 2 + 1];
-            }
-          }
-        }
-      }
-      // P = hi + lo, both bf16: the P.V product keeps ~16 mantissa bits of P
-      const uint32_t h01 = pack_bf16(p[0], p[1]), h23 = pack_bf16(p[2], p[3]);
-      const float2 f01 = bf16x2_to_float2(h01), f23 = bf16x2_to_float2(h23);
-      pb[mb][0] = movmatrix_trans(h01);  // rows 0-7 of the block
-      pb[mb][1] = movmatrix_trans(h23);  // rows 8-15
-      pl[mb][0] = movmatrix_trans(pack_bf16(p[0] - f01.x, p[1] - f01.y));
-      pl[mb][1] = movmatrix_trans(pack_bf16(p[2] - f23.x, p[3] - f23.y));
-    }
-    // o^T += V^T P^T
-#pragma unroll
-    for (int mb = 0; mb < 2; ++mb) {
-      const int r = r_w + mb * 16 + (msel >> 1) * 8 + mrow;
-#pragma unroll
-      for (int eb = 0; eb < C::kKSteps; ++eb) {
-        const int c8 = (eb & 3) * 2 + (msel & 1);
-        uint32_t a0, a1, a2, a3;
-        ldsm_x4_trans(vbase + (eb >> 2) * kBoxBytes + swz(r, c8), a0, a1, a2, a3);
-        mma_bf16(o[eb], a0, a1, a2, a3, pb[mb][0], pb[mb][1]);
-        mma_bf16(o[eb], a0, a1, a2, a3, pl[mb][0], pl[mb][1]);
-      }
-    }
-    __syncwarp();
-    if (tile_rows < r_w + 32) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tile_update<D, G, 2>(acc, qf, smem + (size_t)st * C::kStageBytes,
+                         min(kTile, rows - t * kTile), suffix_lo - row0 - t * kTile,
+                         a.logits ? a.logits + (lrow0 + t * kTile) * G : nullptr, a.qscale, warp,
+                         lane);
     if (lane == 0) mbar_arrive(&empty_bar[st]);
     if (t != ntiles - 1) continue;
 
     // ---------------------------------------------------------- chunk done: hand it off
     // This warp's sums over its rows (lanes of one t4 hold the rows g, g + 8 of a head pair).
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-#pragma unroll
-      for (int off = 4; off <= 16; off <<= 1) {
-        l2[h] += __shfl_xor_sync(0xffffffffu, l2[h], off);
-        u2[h] += __shfl_xor_sync(0xffffffffu, u2[h], off);
-        sg2[h] += __shfl_xor_sync(0xffffffffu, sg2[h], off);
-      }
-    }
+    acc.join_lanes();
     if (!handoff) continue;
     const int buf = tk % TB::kBufs, slot = tk % kTickets;
     int ok = 1;
@@ -792,25 +581,9 @@ attend_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
       continue;
     }
     __syncwarp();  // the lanes' stores below follow lane 0's wait
-    {
-      // o^T fragments: this thread holds o[e][2 t4 + h2] for e = 16 eb + g (+8)
-      float *ob = tbuf + (size_t)buf * TB::kFloats + warp * G * TB::kOStride;
-      float *sb =
-          tbuf + (size_t)buf * TB::kFloats + kConsumerWarps * G * TB::kOStride + warp * G * 4;
-#pragma unroll
-      for (int h2 = 0; h2 < 2; ++h2) {
-        const int h = 2 * t4 + h2;
-        if (h < G) {
-#pragma unroll
-          for (int eb = 0; eb < C::kKSteps; ++eb) {
-            ob[h * TB::kOStride + eb * 16 + g] = o[eb][h2];
-            ob[h * TB::kOStride + eb * 16 + g + 8] = o[eb][h2 + 2];
-          }
-          if (g == 0)
-            *reinterpret_cast<float4 *>(sb + h * 4) = make_float4(m2[h2], l2[h2], u2[h2], sg2[h2]);
-        }
-      }
-    }
+    float *ob = tbuf + (size_t)buf * TB::kFloats;
+    acc.template store<G, 4>(ob + warp * G * TB::kOStride,
+                             ob + kConsumerWarps * G * TB::kOStride + warp * G * 4, lane);
     __syncwarp();
     if (lane == 0) mbar_arrive(&tfull[slot]);
     ++tk;
@@ -861,19 +634,6 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// 2-D view [L * H_kv * S_total rows][d] of one cache tensor, boxes of 128 rows x 64 columns
-bool make_map(CUtensorMap *m, const void *base, int d, int64_t rows) {
-  auto fn = encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)d * 2};
-  cuuint32_t box[2] = {64, (cuuint32_t)kTile};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <int D, int G>
 cudaError_t launch_mma_typed(const CUtensorMap &mk, const CUtensorMap &mv, const AttendArgs &a,
                              int grid, int *counter, cudaStream_t s) {
@@ -903,12 +663,25 @@ cudaError_t launch_mma_d(const CUtensorMap &mk, const CUtensorMap &mv, const Att
 
 }  // namespace
 
+// 2-D view [L * H_kv * S_total rows][d] of one cache tensor, boxes of 128 rows x 64 columns
+bool make_kv_map(CUtensorMap *m, const void *base, int d, int64_t rows) {
+  auto fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)d * 2};
+  cuuint32_t box[2] = {64, (cuuint32_t)kTileRows};
+  cuuint32_t estr[2] = {1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box,
+            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 int mma_tile_rows() { return kTile; }
 
 cudaError_t launch_attend_mma_partial(const AttendArgs &a, int d, int g, int64_t rows_total,
                                       cudaStream_t s) {
   CUtensorMap mk, mv;
-  if (!make_map(&mk, a.K, d, rows_total) || !make_map(&mv, a.V, d, rows_total))
+  if (!make_kv_map(&mk, a.K, d, rows_total) || !make_kv_map(&mv, a.V, d, rows_total))
     return cudaErrorInvalidValue;
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);

@@ -37,6 +37,11 @@ int mma_tile_rows();
 cudaError_t launch_attend_mma_partial(const AttendArgs &a, int d, int g, int64_t rows_total,
                                       cudaStream_t s);
 
+// short bf16 calls (lg_attend_cluster.cu): whether a call takes that pass, and the pass
+bool attend_cluster_takes(const AttendArgs &a);
+cudaError_t launch_attend_cluster(const AttendArgs &a, int d, int g, int64_t rows_total,
+                                  cudaStream_t s);
+
 // guard kernels (lg_guard.cu)
 cudaError_t launch_begin_step(const lg_cache &c, cudaStream_t s);
 cudaError_t launch_append(const lg_cache &c, int layer0, int n_layers, const void *k_new,

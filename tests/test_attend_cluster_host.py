@@ -1,0 +1,112 @@
+"""The cluster pass's bookkeeping (quick_div, TileSpace, run_bound in csrc/lg_attend_cluster.cu),
+compiled for the host from the kernel's own source text, over random batches with empty and
+uneven sequences: quotients exact over their range with the float division off by two units in
+the last place either way; tiles found in their groups; clusters' runs and their CTAs' ranges that cover
+every tile once, runs of whole groups."""
+import os
+import re
+import shutil
+import subprocess
+import tempfile
+
+import pytest
+
+from test_attend_geometry_host import _block
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SRC = os.path.join(ROOT, "paper_2604_10044_gb300", "csrc", "lg_attend_cluster.cu")
+
+HARNESS = r'''
+#include <cmath>
+#include <cstdint>
+#include <cstdio>
+#include <cstdlib>
+#include <algorithm>
+#include <random>
+#include <vector>
+#define __device__
+#define __forceinline__ inline
+using std::max; using std::min;
+constexpr int kTileRows = 128, kClusterSeqs = 64, kMaxCluster = 8;
+static int g_ulp = 0;  // error of the float division, units in the last place
+static inline float __fdividef(float a, float b) {
+  float q = a / b;
+  for (int i = 0; i < std::abs(g_ulp); ++i) q = std::nextafter(q, g_ulp > 0 ? INFINITY : -INFINITY);
+  return q < 0 ? 0 : q;
+}
+%(code)s
+static int fails = 0;
+#define CHECK(c, ...) do { if (!(c) && fails++ < 10) { std::printf(__VA_ARGS__); std::printf("\n"); } } while (0)
+int main() {
+  std::mt19937_64 rng(1);
+  auto pick = [&](long long lo, long long hi) { return lo + (long long)(rng() %% (unsigned long long)(hi - lo + 1)); };
+  for (g_ulp = -2; g_ulp <= 2; ++g_ulp)
+    for (int it = 0; it < 400000; ++it) {
+      const int d = (int)pick(1, it %% 2 ? 200 : 1 << 20);
+      const long long x = pick(0, std::min((1LL << 24) - 1, ((long long)d << 20) - 1));
+      CHECK(quick_div((int)x, d) == x / d, "quick_div %%lld / %%d", x, d);
+    }
+  for (int it = 0; it < 4000; ++it) {
+    g_ulp = (int)pick(-2, 2);
+    const int batch = (int)pick(1, 64), H_kv = (int)pick(1, 8), L = (int)pick(1, 6);
+    std::vector<int> len(batch), pre(batch);
+    int total = 0;
+    const int top = (int)pick(1, it %% 3 ? 3000 : 60000);
+    for (int b = 0; b < batch; ++b) {
+      len[b] = pick(0, 3) ? (int)pick(0, top) : 0;
+      pre[b] = total;
+      total += (len[b] + kTileRows - 1) / kTileRows;
+    }
+    TileSpace ts{len.data(), pre.data(), batch, H_kv, L, total};
+    const int T = total * H_kv * L;
+    if (T == 0 || T >= 1 << 20) continue;
+    TileGroup g = ts.find(0);
+    std::vector<int> starts;  // group starts, walked
+    for (int t = 0; t < T;) {
+      CHECK(g.start == t && g.tiles > 0 && g.tiles == ts.tiles(g.b), "walk at %%d", t);
+      for (int x : {t, t + g.tiles / 2, t + g.tiles - 1}) {
+        const TileGroup f = ts.find(x);
+        CHECK(f.start == g.start && f.lloc == g.lloc && f.b == g.b && f.kvh == g.kvh, "find %%d", x);
+      }
+      starts.push_back(t);
+      t += g.tiles;
+      if (t < T) ts.next(g);
+    }
+    const int n_cl = (int)pick(1, std::min(152, L * batch * H_kv)), ctas = (int)pick(1, 8);
+    int at = 0;
+    for (int k = 0; k < n_cl; ++k) {
+      const int c0 = run_bound(ts, T, k, n_cl), c1 = run_bound(ts, T, k + 1, n_cl);
+      CHECK(c0 == at && c1 >= c0, "runs %%d: %%d %%d", k, c0, c1);
+      CHECK(c1 == T || std::binary_search(starts.begin(), starts.end(), c1), "run end %%d", c1);
+      at = c1;
+      int u = c0;
+      for (int r = 0; r < ctas; ++r) {
+        const int u0 = c0 + quick_div((c1 - c0) * r, ctas), u1 = c0 + quick_div((c1 - c0) * (r + 1), ctas);
+        CHECK(u0 == u && u1 >= u0, "cta ranges");
+        u = u1;
+      }
+      CHECK(u == c1, "cta cover");
+    }
+    CHECK(at == T, "cluster cover %%d of %%d", at, T);
+  }
+  std::printf("mismatches %%d\n", fails);
+  return fails != 0;
+}
+'''
+
+
+def test_cluster_bookkeeping():
+    if shutil.which("g++") is None:
+        pytest.skip("needs g++")
+    text = open(SRC).read()
+    assert re.search(r"kClusterSeqs = 64;", text) and re.search(r"kMaxCluster = 8;", text)
+    assert "groups <= 1 << 16 && tiles < 1 << 20" in text  # the ranges checked here
+    code = "\n".join([_block(text, r"^__device__ __forceinline__ int quick_div\("),
+                      _block(text, r"^struct TileGroup \{"), _block(text, r"^struct TileSpace \{"),
+                      _block(text, r"^__device__ __forceinline__ int run_bound\(")])
+    with tempfile.TemporaryDirectory() as d:
+        cpp, exe = os.path.join(d, "c.cpp"), os.path.join(d, "c")
+        open(cpp, "w").write(HARNESS % dict(code=code))
+        subprocess.run(["g++", "-O2", "-std=c++17", cpp, "-o", exe], check=True)
+        r = subprocess.run([exe], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout

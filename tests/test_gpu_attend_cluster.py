@@ -1,0 +1,110 @@
+"""The cluster pass of lg_decode_attend (bf16, batch up to 64) against a plain fp64 attention and
+against the persistent pass on the same cache: empty sequences appended until the batch passes
+the cluster pass's limit send the same call there.
+
+Lengths around its 128-row tiles, empty and one-row sequences, equal lengths (the clusters' runs
+known before the lengths) and uneven ones, groups within one CTA, shared by two, by a whole
+cluster, and several groups a CTA, every GQA group, both head sizes, several layers a call, and
+the H2O logits it leaves for the score update."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2604_10044_gb300 import lg
+
+pytestmark = pytest.mark.gpu
+
+LIMIT = 64  # kClusterSeqs in csrc/lg_attend_cluster.cu
+
+
+def _run(k, v, q, lens, layer0, n_layers, suffix_w, h2o, pad):
+    """out, stats (and scores) of layers [layer0, layer0 + n_layers) over cache rows k, v
+    [L][H_kv][S][d]; pad: empty sequences after the real ones"""
+    L, H_kv, S, d = k.shape
+    b, H_q = len(lens), q.shape[2]
+    cap = np.concatenate([np.asarray(lens) + 1, np.ones(pad, np.int64)]).astype(np.int32)
+    off = np.concatenate([[0], np.cumsum(cap)[:-1]]).astype(np.int64)
+    extra = int(cap.sum()) - S
+    kk, vv = (torch.cat([x, torch.full((L, H_kv, extra, d), 3.0, dtype=x.dtype, device=x.device)],
+                        2) for x in (k, v))
+    n = np.concatenate([lens, np.zeros(pad, np.int64)]).astype(np.int32)
+    c = lg.Cache(L, H_kv, d, "bf16", off, cap, n, k.device, "h2o" if h2o else "loopguard", kk, vv)
+    g = lg.Guard(c, H_q, policy="h2o" if h2o else "loopguard", n_layers_per_call=n_layers)
+    qq = torch.cat([q, torch.ones((n_layers, pad, H_q, d), dtype=q.dtype, device=q.device)], 1)
+    out = torch.full((n_layers, b + pad, H_q, d), 7.0, dtype=torch.bfloat16, device=k.device)
+    st = torch.full((n_layers, b + pad, H_q, 4), 7.0, dtype=torch.float32, device=k.device)
+    lg.lg_decode_attend(c, layer0, n_layers, qq.contiguous(), H_q, g.scale, out, st, suffix_w,
+                        1 if h2o else 0, int(cap.max()), g.ws)
+    assert lg.lg_read_device_status(c) == 0
+    sc = c.h2o[layer0:layer0 + n_layers, :, :S].clone() if h2o else None
+    return out[:, :b], st[:, :b], sc, off
+
+
+def _exact(k, v, q, lens, off, layer0, n_layers, suffix_w):
+    H_kv, d = k.shape[1], k.shape[3]
+    H_q = q.shape[2]
+    out = torch.zeros((n_layers, len(lens), H_q, d), dtype=torch.float64, device=k.device)
+    st = torch.zeros((n_layers, len(lens), H_q, 4), dtype=torch.float64, device=k.device)
+    st[..., 0] = -float("inf")
+    for l in range(n_layers):
+        for b, n in enumerate(lens):
+            if n == 0:
+                continue
+            rows = slice(int(off[b]), int(off[b]) + int(n))
+            K, V = k[layer0 + l, :, rows].double(), v[layer0 + l, :, rows].double()
+            z = q[l, b].double().view(H_kv, -1, d) @ K.transpose(1, 2) / np.sqrt(d)
+            m = z.amax(-1, keepdim=True)
+            e = torch.exp(z - m)
+            t = e.sum(-1, keepdim=True)
+            a = e / t
+            out[l, b] = (a @ V).reshape(H_q, d)
+            H = torch.log(t[..., 0]) - (a * (z - m)).sum(-1)
+            st[l, b] = torch.stack([m[..., 0], t[..., 0], H, a[..., -min(suffix_w, int(n)):].sum(-1)],
+                                   -1).reshape(H_q, 4)
+    return out, st
+
+
+def _close(got, want, rtol, atol, what):
+    got, want = got.double(), want.double()
+    fine = torch.isfinite(want)
+    assert torch.equal(fine, torch.isfinite(got)), what
+    off = (got - want).abs()[fine] - (atol + rtol * want.abs()[fine])
+    assert off.numel() == 0 or off.max().item() <= 0, (what, off.max().item())
+
+
+CASES = [  # lengths, H_kv, G, d, layers of the call
+    ([1], 1, 1, 128, 1), ([127], 2, 2, 128, 1), ([128], 8, 2, 128, 1), ([129], 8, 3, 128, 1),
+    ([1024], 8, 2, 128, 1), ([1025], 8, 4, 128, 2), ([5000], 1, 8, 128, 1), ([4096], 2, 5, 128, 3),
+    ([9000], 8, 8, 128, 1), ([300] * 5, 8, 4, 128, 1), ([640] * 16, 8, 6, 128, 2),
+    ([130] * 64, 2, 7, 128, 1), ([0], 8, 2, 128, 1), ([0, 0, 0], 2, 4, 128, 2),
+    ([0, 1, 2, 127, 128, 129, 0, 4000, 3], 4, 4, 128, 2), ([4000] + [1] * 63, 8, 4, 128, 1),
+    (list(range(0, 1280, 20)), 2, 6, 128, 1), ([2047, 60, 0, 513], 8, 8, 128, 2),
+    ([1024], 8, 2, 64, 1), ([777] * 3, 2, 4, 64, 3), ([0, 1500, 64, 63], 4, 8, 64, 2),
+    ([3000, 10], 2, 1, 64, 1),
+]
+
+
+@pytest.mark.parametrize("h2o", [False, True])
+@pytest.mark.parametrize("lens,H_kv,G,d,nl", CASES)
+def test_cluster_pass(cuda, lens, H_kv, G, d, nl, h2o):
+    assert len(lens) <= LIMIT
+    g = torch.Generator(device=cuda)
+    g.manual_seed(len(lens) * 1000 + G * 10 + d)
+    L, S = nl + 1, int(sum(lens)) + len(lens)
+    k, v = (torch.randn((L, H_kv, S, d), generator=g, device=cuda).to(torch.bfloat16)
+            for _ in range(2))
+    k *= 1.5
+    q = torch.randn((nl, len(lens), H_kv * G, d), generator=g, device=cuda).to(torch.bfloat16)
+    got, st, sc, off = _run(k, v, q, lens, 1, nl, 50, h2o, 0)
+    want, ws = _exact(k, v, q, lens, off, 1, nl, 50)
+    # the parity tests' bounds: bf16 output rounding, fp32 sums
+    _close(got, want, 2e-2, 1e-3, "out")
+    _close(st, ws, 1e-4, 1e-6, "stats")
+    gen, gst, gsc, _ = _run(k, v, q, lens, 1, nl, 50, h2o, LIMIT + 1 - len(lens))
+    # both within 2^-8 of the same value: they differ by one bf16 step at most
+    _close(got, gen, 2.0 ** -7, 1e-5, "out against the persistent pass")
+    _close(st, gst, 2e-5, 1e-6, "stats against the persistent pass")
+    if h2o:
+        _close(sc, gsc, 2e-5, 1e-9, "scores against the persistent pass")
+        total = sc.double().sum(-1)  # every non-empty sequence adds G to its kv-head's scores
+        assert torch.allclose(total, torch.full_like(total, G * sum(n > 0 for n in lens)), rtol=1e-5)
