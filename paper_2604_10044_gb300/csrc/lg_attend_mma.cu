@@ -612,7 +612,7 @@ attend_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
 // after it keeps its programmatic launch edge), and the word after them flipped: its low bit
 // is the direction of this call's pass (any start value will do; it only alternates).
 __global__ void zero_counters_kernel(int *p, int n) {
-  pdl_enter();
+  pdl_enter_early();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) p[n] ^= 1;
 }

@@ -21,7 +21,7 @@ namespace lg {
 // (Here and in append_kernel the inputs are read before the status word, so that every load
 // of a thread is in flight at once; neither kernel has a barrier after its status check.)
 __global__ void begin_step_kernel(lg_cache c) {
-  pdl_enter();
+  pdl_enter_early();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= c.batch) return;
   const int n = c.len[b], cap = c.cap[b];
@@ -40,7 +40,7 @@ template <typename T>
 __global__ void append_kernel(lg_cache c, int layer0, int n_layers, const uint4 *k_new,
                               const uint4 *v_new, const int32_t *pos_new, int row_blocks,
                               int lguard) {
-  pdl_enter();
+  pdl_enter_early();
   if ((int)blockIdx.x >= row_blocks) {
     const int b = blockIdx.x - row_blocks;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
