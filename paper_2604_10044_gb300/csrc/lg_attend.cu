@@ -1,11 +1,12 @@
 // Split-K decode attention over the KV cache fused with the guard's per-head statistics
 // (LoopGuard Sec. 3.1, Eq. 1; statistics read by Sec. 5.2), plus the H2O score accumulation
-// of the comparator policy (Sec. 2.2, Sec. 6.1).
+// of the comparator policy (Sec. 2.2, Sec. 6.1), and the choice of a call's pass.
 //
-// One CTA streams CH consecutive rows of one (layer, sequence, kv-head) and serves all g query
-// heads of that kv-head, so every K/V byte is read from HBM once per step.  A producer warp
-// moves 8 KB K and V tiles into a 4-stage shared-memory ring with 1-D bulk copies (TMA)
-// completing on mbarriers; four consumer warps compute.  A row is split over LPR lanes
+// The chunk kernel here serves fp32 caches past the cluster pass's limits (lg_attend_cluster.cuh:
+// more than 64 sequences, the longest calls).  One CTA streams CH consecutive rows of one (layer,
+// sequence, kv-head) and serves all g query heads of that kv-head, so every K/V byte is read from
+// HBM once per step.  A producer warp moves 8 KB K and V tiles into a 4-stage shared-memory ring
+// with 1-D bulk copies (TMA) completing on mbarriers; four consumer warps compute.  A row is split over LPR lanes
 // (16 B each): the lanes form partial dot products for all heads with packed fp32 FMAs, a
 // transposed butterfly leaves each lane with the full logit of one head, that lane runs the
 // online softmax for its head (in log2 units) and the probabilities are broadcast back for
@@ -40,29 +41,6 @@ struct AttendCfg {
   static_assert(kGP <= kLPR, "GQA group wider than the lanes of a row");
   static_assert(kSteps >= 1, "tile too small");
   static_assert(kGroups * G * D * 4 + kGroups * kGP * 16 <= kSmem, "combine scratch");
-};
-
-// Leaves in v[0] the sum over the LPR lanes of a row of the partials of head
-// lane_in_row / (LPR / GP): halving levels first (each lane keeps half of its heads and sends
-// the other half to its partner), plain butterfly levels after.
-template <int CNT, int OFF>
-struct HeadReduce {
-  __device__ __forceinline__ static void run(float *v, int lane) {
-    if constexpr (CNT > 1) {
-      constexpr int H = CNT / 2;
-      const bool upper = (lane & OFF) != 0;
-#pragma unroll
-      for (int i = 0; i < H; ++i) {
-        const float send = upper ? v[i] : v[i + H];
-        const float keep = upper ? v[i + H] : v[i];
-        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, OFF);
-      }
-      HeadReduce<H, OFF / 2>::run(v, lane);
-    } else if constexpr (OFF >= 1) {
-      v[0] += __shfl_xor_sync(0xffffffffu, v[0], OFF);
-      HeadReduce<1, OFF / 2>::run(v, lane);
-    }
-  }
 };
 
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -410,20 +388,19 @@ static cudaError_t launch_typed(const AttendArgs &a, int64_t rows_total, void *o
   using C = AttendCfg<T, D, G>;
   cudaError_t e;
   if (Elem<T>::kDtype == LG_BF16) {
-    // tensor-core partial pass (lg_attend_mma.cu)
-    e = attend_cluster_takes(a) ? launch_attend_cluster(a, D, G, rows_total, s)
-                                   : launch_attend_mma_partial(a, D, G, rows_total, s);
+    // tensor-core passes (lg_attend_cluster.cu, lg_attend_mma.cu), which merge their partials
+    e = attend_cluster_takes(a, mma_tile_rows(), rows_total)
+            ? launch_attend_cluster(a, D, G, rows_total, s)
+            : launch_attend_mma_partial(a, D, G, rows_total, s);
     if (e != cudaSuccess) return e;
+  } else if (attend_cluster_takes(a, cluster_f32_tile_rows(), rows_total)) {
+    LG_TRY(launch_attend_cluster_f32(a, D, G, rows_total, s));
   } else {
     auto kp = attend_partial_kernel<T, D, G>;
     e = cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
     if (e != cudaSuccess) return e;
     dim3 grid(a.max_chunks, a.H_kv, a.n_layers * a.batch);
     LG_TRY(launch_pdl(kp, grid, C::kThreads, C::kSmem, s, a));
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  if (Elem<T>::kDtype != LG_BF16) {
-    // the tensor-core pass merges its chunk partials itself
     const int64_t heads = (int64_t)a.n_layers * a.batch * a.H_q;
     LG_TRY(launch_pdl(attend_combine_kernel<T, D>, (unsigned)((heads + 7) / 8), 256, 0, s, a, out,
                       stats, final_ml));

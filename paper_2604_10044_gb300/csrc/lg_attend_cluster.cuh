@@ -1,0 +1,681 @@
+// Decode attention by thread-block clusters that merge their split-K partials through distributed
+// shared memory, for bf16 caches (lg_attend_cluster.cu, tensor cores) and fp32 ones
+// (lg_attend_cluster_f32.cu).  lg_attend_mma.cu and lg_attend.cu hold the passes for batches and
+// calls past its limits.
+//
+// What bounds a call: a long one the memory, a short one (a layer at one sequence: 64 KB a CTA)
+// latency.  The persistent pass pays for its work sharing there: a kernel before it that resets
+// its counters, a claim per chunk, and a merge through L2 (partials, an arrival count, partials
+// again, one warp for all heads of a group).  Here each cluster owns a run of whole (layer,
+// sequence, kv-head) groups, about the same number of tiles each, and splits the run's tiles
+// evenly over its CTAs, so every CTA streams one contiguous range of tiles through a ring of
+// tensor copies.  A group that lies within one CTA is finished there.  The (at most two) groups
+// a CTA shares with its neighbours are folded over its warps, and the folded pieces {M, l, u, sigma, o[32]} go straight into the
+// shared memory of the CTAs that own them (the sharing CTAs own a group's pieces in turn); after
+// one cluster barrier each owner merges what it received.  No counters, no workspace, no other
+// launch.  Uneven lengths cost little: a CTA with less to read leaves its bandwidth to the others
+// (one CTA streams up to 80 GB/s, 1.6 times its even share).
+//
+// GB300, one layer of 28 (append and attention, called one by one in a graph), one sequence of
+// 1024 rows, 16/8 heads of 128: 12.0 -> 7.3 us.  Of a CTA's 5.0 us after its wait, 0.5 go to the
+// lengths, 0.4 to its range and first copy, 1.1 to that copy, 0.8 to the tile, 1.0 to the fold,
+// 0.5 to the barrier and 0.5 to the merge (clock64 at each phase).
+#pragma once
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <math.h>
+#include <stdint.h>
+
+#include <atomic>
+
+#include "lg_common.cuh"
+#include "lg_internal.h"
+#include "lg_mma_tile.cuh"
+
+namespace lg {
+
+namespace {
+
+constexpr int kClusterSeqs = 64;  // batch at most (two sequences a lane in the prologue's scan)
+constexpr int kMaxCluster = 8;    // CTAs of a cluster at most (portable)
+
+// What differs between the element types: the tile and the ring, and a consumer warp's work.
+//   kTile rows a tile, kBoxes boxes of kBoxCols columns per tensor, kStages stages in the ring
+//   kWarps consumer warps, which share every tile; kTileUs one CTA's time for a tile
+//   begin(the segment's query rows), update(a tile), join() (the lanes' sums) and store(a row of
+//   D + 4 floats per head: o, then {M, l, u, sigma})
+template <typename T, int D, int G>
+struct Pass;
+
+template <typename T, int D, int G>
+struct ClusterCfg {
+  using P = Pass<T, D, G>;
+  static constexpr int kSize = Elem<T>::kSize;
+  static constexpr int kWarps = P::kWarps, kStages = P::kStages;
+  static constexpr int kThreads = (kWarps + 1) * 32;
+  static constexpr int kBoxBytes = P::kTile * P::kBoxCols * kSize;
+  static constexpr int kStageBytes = 2 * P::kBoxes * kBoxBytes;
+  static constexpr int kTileBytes = 2 * P::kTile * D * kSize;
+  static_assert(kStageBytes == kTileBytes && P::kBoxCols * kSize == 128, "whole rows");
+  static constexpr int kQBytes = G * D * kSize;         // a group's query rows
+  static constexpr int kRow = D + 4;                    // one head's o, then {M, l, u, sigma}
+  static constexpr int kWarpFloats = kWarps * G * kRow;  // one segment's warp partials
+  static constexpr int kUnits = G * (D / 32);           // (head, 32 output elements) of a group
+  static constexpr int kUnit = 36;                      // floats of a unit's partial: o, then stats
+  // a CTA owns every np-th unit of a group shared by np CTAs and receives np partials of each
+  static constexpr int recv_max() {
+    int m = 0;
+    for (int np = 2; np <= kMaxCluster; ++np) {
+      const int r = (kUnits + np - 1) / np * np;
+      if (r > m) m = r;
+    }
+    return m;
+  }
+  static constexpr int kRecvFloats = recv_max() * kUnit;
+  static constexpr int kSmem = kStages * kStageBytes + 2 * kQBytes +
+                               (kWarpFloats + 2 * kRecvFloats) * (int)sizeof(float) + 1024;
+  static_assert(kSmem + 1024 <= 227 * 1024, "shared memory of a CTA, with its static arrays");
+};
+
+__device__ __forceinline__ int cluster_rank() {
+  int r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// the cluster's barrier (every thread; whole warps, converged): release at the arrival, acquire
+// at the wait, cluster scope
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// shared-memory address of the same variable in another CTA of the cluster, and stores to it
+__device__ __forceinline__ uint32_t peer_addr(const void *p, int rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void peer_st(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void peer_st4(uint32_t addr, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y),
+               "f"(v.z), "f"(v.w)
+               : "memory");
+}
+
+template <int kThreads>
+__device__ __forceinline__ void named_sync(int id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kThreads) : "memory");
+}
+template <int kThreads>
+__device__ __forceinline__ void named_arrive(int id) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kThreads) : "memory");
+}
+
+// floor(x / d) for 0 <= x < 2^24, d >= 1 and a quotient below 2^20: in floats it is off by at most
+// one (the integer division's longer chain sat on the way to the first copy)
+__device__ __forceinline__ int quick_div(int x, int d) {
+  int q = (int)__fdividef((float)x, (float)d);
+  q -= q * d > x;
+  q += (q + 1) * d <= x;
+  return q;
+}
+
+// One (layer, sequence, kv-head) group among the call's tiles, numbered layer by layer, sequence
+// by sequence, kv-head by kv-head.
+struct TileGroup {
+  int lloc, b, kvh;
+  int start, tiles;  // its first tile and their number
+};
+
+// The call's tiles: pre[b] tiles in the sequences before b (of one kv-head of one layer), total
+// over the batch, rows to a tile.
+struct TileSpace {
+  const int *len, *pre;  // [batch]
+  int batch, H_kv, n_layers, total, rows;
+  __device__ __forceinline__ int tiles(int b) const { return (len[b] + rows - 1) / rows; }
+  __device__ __forceinline__ TileGroup find(int t) const {
+    TileGroup g;
+    const int per_layer = total * H_kv;
+    g.lloc = n_layers > 1 ? quick_div(t, per_layer) : 0;
+    const int r = t - g.lloc * per_layer;
+    int b = 0;
+    if (batch > 1) {
+#pragma unroll
+      for (int st = kClusterSeqs / 2; st >= 1; st >>= 1)
+        if (b + st < batch && pre[b + st] * H_kv <= r) b += st;
+    }
+    g.b = b;
+    g.tiles = tiles(b);
+    const int r0 = pre[b] * H_kv;
+    g.kvh = quick_div(r - r0, g.tiles);
+    g.start = g.lloc * per_layer + r0 + g.kvh * g.tiles;
+    return g;
+  }
+  __device__ __forceinline__ void next(TileGroup &g) const {
+    g.start += g.tiles;
+    if (++g.kvh < H_kv) return;
+    g.kvh = 0;
+    do {
+      if (++g.b == batch) {
+        g.b = 0;
+        ++g.lloc;
+      }
+      g.tiles = tiles(g.b);
+    } while (g.tiles == 0);
+  }
+};
+
+// The first tile of cluster k's run among n_cl (of T tiles): an even share of the tiles, rounded
+// to the nearest group boundary.
+__device__ __forceinline__ int run_bound(const TileSpace &ts, int T, int k, int n_cl) {
+  const int x = (int)((unsigned)T * (unsigned)k / (unsigned)n_cl);
+  if (x <= 0 || x >= T) return x;
+  const TileGroup g = ts.find(x);
+  return 2 * (x - g.start) < g.tiles ? g.start : g.start + g.tiles;
+}
+
+// out and statistics of one head from its merged sums (a warp's 32 elements of the output)
+template <typename T, int D>
+__device__ __forceinline__ void finish(const AttendArgs &a, int64_t head, int e, bool first,
+                                       float M, float l, float u, float sg, float o) {
+  const float inv_l = 1.f / l;
+  Elem<T>::store(a.out, head * D + e, o * inv_l);
+  if (first) {
+    constexpr float kLn2 = 0.69314718055994530942f;
+    *reinterpret_cast<float4 *>(a.stats + head * 4) =
+        make_float4(M * kLn2, l, logf(l) - u * kLn2 * inv_l, sg * inv_l);
+    if (a.final_ml) {
+      a.final_ml[head * 2] = M;
+      a.final_ml[head * 2 + 1] = l;
+    }
+  }
+}
+
+}  // namespace
+
+template <typename T, int D, int G>
+__global__ void __launch_bounds__(ClusterCfg<T, D, G>::kThreads, 1)
+attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
+                      const __grid_constant__ CUtensorMap tmV, AttendArgs a, int ctas, int n_cl) {
+  using P = Pass<T, D, G>;
+  using Cl = ClusterCfg<T, D, G>;
+  constexpr int kWarps = Cl::kWarps, kRow = Cl::kRow, kTile = P::kTile;
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t full_bar[Cl::kStages];
+  __shared__ __align__(8) uint64_t empty_bar[Cl::kStages];
+  __shared__ __align__(8) uint64_t q_full[2], q_empty[2];  // query rows of segment i in buffer i & 1
+  __shared__ int s_len[kClusterSeqs], s_pre[kClusterSeqs], s_off[kClusterSeqs];
+  __shared__ int s_total, s_c0, s_c1, s_empty;
+  unsigned char *smem = reinterpret_cast<unsigned char *>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  unsigned char *qbuf = smem + Cl::kStages * Cl::kStageBytes;  // [2][G][D]
+  float *part = reinterpret_cast<float *>(qbuf + 2 * Cl::kQBytes);  // [warp][G][kRow]
+  float *recv = part + Cl::kWarpFloats;  // [2][recv_max][kUnit]
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = cluster_rank(), cluster = quick_div(blockIdx.x, ctas);
+  cluster_arrive();  // waited for before the first store to a peer: every CTA has started then
+  if (threadIdx.x == kWarps * 32) {
+    for (int s = 0; s < Cl::kStages; ++s) {
+      mbar_init(&full_bar[s], 1);
+      mbar_init(&empty_bar[s], kWarps);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&q_full[s], 1);
+      mbar_init(&q_empty[s], kWarps);
+    }
+    mbar_fence_init();
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmK)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
+  }
+  TileSpace ts;
+  ts.len = s_len;
+  ts.pre = s_pre;
+  ts.batch = a.batch;
+  ts.H_kv = a.H_kv;
+  ts.n_layers = a.n_layers;
+  ts.rows = kTile;
+
+  if (warp == kWarps) {
+    // ------------------------------------------------------------ producer
+    // (this warp alone reads the lengths and forms the ranges: the others pick them up from
+    // shared memory while its first copies are in flight)
+    uint64_t evict_first, evict_normal;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(evict_first));
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(evict_normal));
+    // The groups of this cluster if all have as many tiles: [gi0, gi1), and the first one's place
+    // (known before the lengths are: a group's share of the tiles is then its share of the groups)
+    const int groups = a.n_layers * a.batch * a.H_kv;
+    const int gi0 = quick_div(groups * cluster, n_cl), gi1 = quick_div(groups * (cluster + 1), n_cl);
+    TileGroup g;
+    {
+      const int lb = quick_div(gi0, a.H_kv);
+      g.kvh = gi0 - lb * a.H_kv;
+      g.lloc = quick_div(lb, a.batch);
+      g.b = lb - g.lloc * a.batch;
+    }
+    pdl_enter();
+    // lengths and the tiles before each sequence, two sequences a lane
+    int n[2], t[2], any_empty = 0;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int b = 2 * lane + k;
+      n[k] = b < a.batch ? a.len[b] : -1;
+      if (b < a.batch) s_off[b] = (int)a.seq_off[b];
+    }
+    const int bad = __shfl_sync(0xffffffffu, lane == 0 ? (int)status_bad(a.status) : 0, 0);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      if (n[k] > a.max_len) {
+        set_status(a.status, LG_ERR_CAPACITY);
+        n[k] = -1;
+      }
+      any_empty |= n[k] == 0;
+      n[k] = max(n[k], 0);
+      t[k] = (n[k] + kTile - 1) / kTile;
+    }
+    const int t_first = __shfl_sync(0xffffffffu, t[0], 0);
+    const bool same = (2 * lane >= a.batch || t[0] == t_first) &&
+                      (2 * lane + 1 >= a.batch || t[1] == t_first);
+    int c0 = 0, c1 = 0, u0 = 0, u1 = 0;
+    if (__all_sync(0xffffffffu, same)) {
+      ts.total = t_first * a.batch;
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        if (2 * lane + k < a.batch) {
+          s_len[2 * lane + k] = n[k];
+          s_pre[2 * lane + k] = (2 * lane + k) * t_first;
+        }
+      if (!bad) {
+        c0 = gi0 * t_first;
+        c1 = gi1 * t_first;
+      }
+      u0 = c0 + quick_div((c1 - c0) * rank, ctas);
+      u1 = c0 + quick_div((c1 - c0) * (rank + 1), ctas);
+      g.tiles = t_first;
+      g.start = c0;
+      __syncwarp();
+      while (g.start + t_first <= u0 && u0 < u1) ts.next(g);
+    } else {
+      int upto = t[0] + t[1];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= o) upto += x;
+      }
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        if (2 * lane + k < a.batch) {
+          s_len[2 * lane + k] = n[k];
+          s_pre[2 * lane + k] = upto - t[0] - t[1] + (k ? t[0] : 0);
+        }
+      ts.total = __shfl_sync(0xffffffffu, upto, 31);
+      __syncwarp();
+      const int all = ts.total * a.H_kv * a.n_layers;
+      if (!bad) {
+        // this cluster's run of groups [c0, c1) (even lanes form its start, odd lanes its end)
+        const int x = run_bound(ts, all, cluster + (lane & 1), n_cl);
+        c0 = __shfl_sync(0xffffffffu, x, 0);
+        c1 = __shfl_sync(0xffffffffu, x, 1);
+      }
+      u0 = c0 + quick_div((c1 - c0) * rank, ctas);
+      u1 = c0 + quick_div((c1 - c0) * (rank + 1), ctas);
+      if (u0 < u1) g = ts.find(u0);
+    }
+    any_empty = __any_sync(0xffffffffu, any_empty);
+    if (lane == 0) {
+      s_total = ts.total;
+      s_c0 = c0;
+      s_c1 = c1;
+      s_empty = any_empty && !bad;
+    }
+    __syncwarp();
+    named_arrive<Cl::kThreads>(1);
+    if (lane == 0 && u0 < u1) {
+      // K/V are streamed once; a call that fits beside the rest of the step stays in L2
+      const uint64_t policy = ts.total * a.H_kv * a.n_layers <= kL2KeepBytes / Cl::kTileBytes
+                                  ? evict_normal
+                                  : evict_first;
+      uint32_t it = 0, seg = 0;
+      auto timed_out = [&](uint64_t *bar, uint32_t parity) {
+        if (mbar_wait(bar, parity)) return false;
+        set_status(a.status, LG_ERR_TIMEOUT);
+        return true;
+      };
+      bool ok = true;
+      for (int t = u0; t < u1 && ok; ++seg) {
+        const int end = min(g.start + g.tiles, u1);
+        const int row = (int)(((int64_t)(a.layer0 + g.lloc) * a.H_kv + g.kvh) * a.S_total) +
+                        s_off[g.b] - g.start * kTile;
+        const int64_t head0 = ((int64_t)g.lloc * a.batch + g.b) * a.H_q + (int64_t)g.kvh * G;
+        const int qb = seg & 1;
+        if (seg >= 2 && timed_out(&q_empty[qb], ((seg >> 1) - 1) & 1)) break;
+        mbar_arrive_expect_tx(&q_full[qb], Cl::kQBytes);
+        bulk_load(qbuf + qb * Cl::kQBytes, (const unsigned char *)a.q + head0 * D * Cl::kSize,
+                  Cl::kQBytes, &q_full[qb]);
+        for (; t < end; ++t, ++it) {
+          const int st = it % Cl::kStages;
+          if (it >= (uint32_t)Cl::kStages &&
+              timed_out(&empty_bar[st], ((it / Cl::kStages) - 1) & 1)) {
+            ok = false;
+            break;
+          }
+          unsigned char *stage = smem + (size_t)st * Cl::kStageBytes;
+          mbar_arrive_expect_tx(&full_bar[st], Cl::kStageBytes);
+#pragma unroll
+          for (int h = 0; h < P::kBoxes; ++h) {
+            tma_load_2d(stage + h * Cl::kBoxBytes, &tmK, h * P::kBoxCols, row + t * kTile,
+                        &full_bar[st], policy);
+            tma_load_2d(stage + (P::kBoxes + h) * Cl::kBoxBytes, &tmV, h * P::kBoxCols,
+                        row + t * kTile, &full_bar[st], policy);
+          }
+        }
+        if (ok && t < u1) ts.next(g);
+      }
+    }
+    __syncwarp();
+    cluster_wait();
+    cluster_arrive();
+    cluster_wait();
+    return;
+  }
+
+  // -------------------------------------------------------------- consumers
+  pdl_enter();
+  named_sync<Cl::kThreads>(1);
+  cluster_wait();
+  ts.total = s_total;
+  const int c0 = s_c0, c1 = s_c1;
+  // this CTA's tiles [u0, u1): an even share of the cluster's
+  auto first_tile = [&](int r) { return c0 + quick_div((c1 - c0) * r, ctas); };
+  // The CTAs of the cluster that share a group: lane r stands for CTA r (np of them, mine before
+  // this one).  CTA number i of them owns units i, i + np, ... of the group.
+  struct Sharers {
+    int lo, nth;   // lane r: CTA r's first tile, its number among the sharers (-1: none)
+    int mine, np;
+  };
+  auto sharers = [&](const TileGroup &g) {
+    Sharers s;
+    s.lo = first_tile(min(lane, ctas));
+    const int hi = first_tile(min(lane + 1, ctas));
+    const bool in = lane < ctas && s.lo < hi && s.lo < g.start + g.tiles && hi > g.start;
+    const unsigned mask = __ballot_sync(0xffffffffu, in);
+    s.nth = in ? __popc(mask & ((1u << lane) - 1u)) : -1;
+    s.mine = __popc(mask & ((1u << rank) - 1u));
+    s.np = __popc(mask);
+    return s;
+  };
+  const int u0 = first_tile(rank), u1 = first_tile(rank + 1);
+  TileGroup g = {};
+  if (u0 < u1) g = ts.find(u0);
+  if (s_empty) {
+    // empty sequences: zero output, m = -inf, l = H = S = 0
+    for (int i = blockIdx.x; i < a.n_layers * a.batch * a.H_kv; i += gridDim.x) {
+      const int lb = i / a.H_kv;
+      if (a.len[lb % a.batch] != 0) continue;
+      const int64_t head0 = (int64_t)lb * a.H_q + (int64_t)(i % a.H_kv) * G;
+      for (int x = threadIdx.x; x < G * D; x += kWarps * 32)
+        Elem<T>::store(a.out, head0 * D + x, 0.f);
+      if (threadIdx.x < G * 4)
+        a.stats[head0 * 4 + threadIdx.x] = threadIdx.x % 4 == 0 ? -INFINITY : 0.f;
+    }
+  }
+  // groups in the slots: 0 for a segment that starts at u0, 1 for another that ends at u1
+  bool shared0 = false, shared1 = false;
+  TileGroup grp0 = {}, grp1 = {};
+  P pass;
+  uint32_t it = 0, seg = 0;
+  bool ok = true;  // false once a copy did not land in time (the barriers below stay matched)
+  auto landed = [&](uint64_t *bar, uint32_t parity) {
+    if (ok && !mbar_wait(bar, parity)) {
+      set_status(a.status, LG_ERR_TIMEOUT);
+      ok = false;
+    }
+    return ok;
+  };
+  for (int t = u0; t < u1; ++seg) {
+    const int start = t, end = min(g.start + g.tiles, u1);
+    const int n = s_len[g.b];
+    const int suffix_lo = n - min(a.suffix_w, n);
+    const int64_t lrow = ((int64_t)g.lloc * a.H_kv + g.kvh) * a.S_total + s_off[g.b];
+    const int qb = seg & 1;
+    if (landed(&q_full[qb], (seg >> 1) & 1)) pass.begin(qbuf + qb * Cl::kQBytes, a.qscale, lane);
+    for (; t < end; ++t, ++it) {
+      const int st = it % Cl::kStages;
+      if (landed(&full_bar[st], (it / Cl::kStages) & 1)) {
+        const int r0 = (t - g.start) * kTile;
+        pass.update(smem + (size_t)st * Cl::kStageBytes, min(kTile, n - r0), suffix_lo - r0,
+                    a.logits ? a.logits + (lrow + r0) * G : nullptr, a.qscale, warp, lane);
+      }
+      if (lane == 0) mbar_arrive(&empty_bar[st]);
+    }
+    if (lane == 0) mbar_arrive(&q_empty[qb]);
+    // the segment's warp partials folded: a whole group is finished here, a part of a group goes
+    // to the owners of its units
+    pass.join();
+    const bool whole = start == g.start && end == g.start + g.tiles;
+    const int64_t head0 = ((int64_t)g.lloc * a.batch + g.b) * a.H_q + (int64_t)g.kvh * G;
+    Sharers sh = {};
+    if (!whole) sh = sharers(g);
+    if (start != u0) named_sync<kWarps * 32>(2);  // the segment before has been folded
+    pass.store(part + warp * G * kRow, lane);
+    named_sync<kWarps * 32>(2);
+#pragma unroll 1
+    for (int un = warp; un < Cl::kUnits; un += kWarps) {
+      const int h = un / (D / 32), e = un % (D / 32) * 32 + lane;
+      uint32_t dst = 0;
+      if (!whole) {
+        // the owner, sharer number un % np, and its slot of this group
+        const int j = quick_div(un, sh.np);
+        const int owner = __ffs(__ballot_sync(0xffffffffu, sh.nth == un - j * sh.np)) - 1;
+        const int slot = __shfl_sync(0xffffffffu, sh.lo, owner) >= g.start ? 0 : 1;
+        dst = peer_addr(recv + slot * Cl::kRecvFloats + (j * sh.np + sh.mine) * Cl::kUnit, owner);
+      }
+      float4 w4[kWarps];
+      float wo[kWarps];
+      float M = -INFINITY;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) {
+        w4[w] = *reinterpret_cast<const float4 *>(part + (w * G + h) * kRow + D);
+        wo[w] = part[(w * G + h) * kRow + e];
+        M = fmaxf(M, w4[w].x);
+      }
+      float l = 0.f, u = 0.f, sg = 0.f, o = 0.f;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) {
+        // a warp that saw no row of this segment has l = u = 0 and M = -inf: no weight
+        const float dm = fmaxf(w4[w].x - M, -1e30f);
+        const float f = exp2f(dm);
+        l += f * w4[w].y;
+        u += f * (w4[w].z + dm * w4[w].y);
+        sg += f * w4[w].w;
+        o += f * wo[w];
+      }
+      if (whole) {
+        finish<T, D>(a, head0 + h, e, un % (D / 32) == 0 && lane == 0, M, l, u, sg, o);
+      } else {
+        peer_st(dst + lane * 4, o);
+        if (lane == 0) peer_st4(dst + 32 * 4, make_float4(M, l, u, sg));
+      }
+    }
+    if (!whole && start == u0) {
+      shared0 = true;
+      grp0 = g;
+    } else if (!whole) {
+      shared1 = true;
+      grp1 = g;
+    }
+    if (t < u1) ts.next(g);
+  }
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();  // every partial has arrived
+#pragma unroll 1
+  for (int slot = 0; slot < 2; ++slot) {
+    if (!(slot ? shared1 : shared0)) continue;
+    const TileGroup gs = slot ? grp1 : grp0;
+    const Sharers sh = sharers(gs);
+    const int mine = sh.mine, np = sh.np;
+    const int64_t head0 = ((int64_t)gs.lloc * a.batch + gs.b) * a.H_q + (int64_t)gs.kvh * G;
+#pragma unroll 1
+    for (int j = warp; j * np + mine < Cl::kUnits; j += kWarps) {
+      const int un = j * np + mine;
+      const float *src = recv + slot * Cl::kRecvFloats + j * np * Cl::kUnit;
+      float4 s4[kMaxCluster];
+      float so[kMaxCluster];
+      float M = -INFINITY;
+#pragma unroll
+      for (int r = 0; r < kMaxCluster; ++r) {
+        s4[r] = r < np ? *reinterpret_cast<const float4 *>(src + r * Cl::kUnit + 32)
+                       : make_float4(-INFINITY, 0.f, 0.f, 0.f);
+        so[r] = r < np ? src[r * Cl::kUnit + lane] : 0.f;
+        M = fmaxf(M, s4[r].x);
+      }
+      float l = 0.f, u = 0.f, sg = 0.f, o = 0.f;
+#pragma unroll
+      for (int r = 0; r < kMaxCluster; ++r) {
+        const float dm = fmaxf(s4[r].x - M, -1e30f);
+        const float f = exp2f(dm);
+        l += f * s4[r].y;
+        u += f * (s4[r].z + dm * s4[r].y);
+        sg += f * s4[r].w;
+        o += f * so[r];
+      }
+      finish<T, D>(a, head0 + un / (D / 32), un % (D / 32) * 32 + lane,
+                un % (D / 32) == 0 && lane == 0, M, l, u, sg, o);
+    }
+  }
+}
+
+namespace {
+
+constexpr int kMaxDev = 64;
+constexpr int kSizes[] = {8, 6, 4, 2, 1};  // cluster sizes used (5 and 7 fit no better than 4 and 6
+                                           // beside the GPU's clusters of SMs)
+constexpr int kNumSizes = sizeof(kSizes) / sizeof(kSizes[0]);
+
+template <typename T, int D, int G>
+struct ClusterLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  ClusterLaunch(int clusters, int ctas, cudaStream_t s) {
+    cfg.gridDim = clusters * ctas;
+    cfg.blockDim = ClusterCfg<T, D, G>::kThreads;
+    cfg.dynamicSmemBytes = ClusterCfg<T, D, G>::kSmem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+  }
+};
+
+// How many clusters of each size the current device holds at once, looked up once per device and
+// kernel (a function of the kernel's shared memory alone).
+template <typename T, int D, int G>
+cudaError_t resident_clusters(int (&n)[kNumSizes]) {
+  static std::atomic<int> known[kMaxDev][kNumSizes];  // 0: not looked up yet
+  int dev = 0;
+  LG_TRY(cudaGetDevice(&dev));
+  for (int i = 0; i < kNumSizes; ++i) {
+    n[i] = dev < kMaxDev ? known[dev][i].load(std::memory_order_relaxed) : 0;
+    if (n[i] > 0) continue;
+    auto kern = attend_cluster_kernel<T, D, G>;
+    LG_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                ClusterCfg<T, D, G>::kSmem));
+    ClusterLaunch<T, D, G> l(1, kSizes[i], nullptr);
+    l.cfg.numAttrs = 1;
+    LG_TRY(cudaOccupancyMaxActiveClusters(&n[i], kern, &l.cfg));
+    if (n[i] < 1) n[i] = 1;
+    if (dev < kMaxDev) known[dev][i].store(n[i], std::memory_order_relaxed);
+  }
+  return cudaSuccess;
+}
+
+// Cluster size and count for `groups` groups of at most `tiles` tiles: the size whose estimated
+// time is least.  With K clusters, each takes groups / K groups and then groups mod K of them one
+// more; either phase is bound by the memory (kTilesPerUs tiles a microsecond over all CTAs) or by
+// the CTAs (kTileUs a tile, kSegmentUs a segment end).  Smaller clusters fill the GPU better
+// (152 SMs hold 15, 23, 36, 76, 152 clusters of 8, 6, 4, 2, 1), larger ones split a group further
+// and stream a little better (about a percent per halving on passes of half a millisecond).
+// Measured per call (append and attention, layers called one by one in a graph, us, sizes 8 / 6 /
+// 4 / 2 / 1; 8 kv-heads of 128): 1 sequence of 1024 rows 7.3 / 7.9 / 7.9 / 9.1 / 10.9; 8 of 4096
+// 30.2 / 26.6 / 26.8 / 26.6 / 29.4; 2 of 131071, 8 heads a group, 238 / 157 / 207 / 397 / 780; 16
+// of 32768, 8 heads a group, 309 / 302 / 303 / 302 / 296.
+struct ClusterShape {
+  int ctas, clusters;
+};
+inline ClusterShape cluster_shape(int groups, int tiles, int tile_bytes, float kTileUs,
+                                  const int (&resident)[kNumSizes]) {
+  const float kTilesPerUs = 7.3e6f / (float)tile_bytes;
+  constexpr float kSegmentUs = 1.f;
+  ClusterShape best = {1, 1};
+  float best_us = 0.f;
+  for (int i = 0; i < kNumSizes; ++i) {
+    const int c = kSizes[i], k = resident[i] < groups ? resident[i] : groups;
+    const int q = groups / k, r = groups % k;
+    const float cta = (float)tiles / (float)c * kTileUs;  // a group's tiles on one of its CTAs
+    float us = fmaxf((float)k * (float)q * (float)tiles / kTilesPerUs,
+                     (float)q * cta + kSegmentUs * (1.f + (float)(q - 1) / (float)c));
+    if (r) us += fmaxf((float)r * (float)tiles / kTilesPerUs, cta + kSegmentUs / (float)c);
+    us *= 1.f + 0.0125f * log2f((float)kMaxCluster / (float)c);
+    if (best_us == 0.f || us < best_us) {
+      best_us = us;
+      best = {c, k};
+    }
+  }
+  return best;
+}
+
+template <typename T, int D, int G>
+cudaError_t launch_cluster_typed(const AttendArgs &a, int64_t rows_total, cudaStream_t s) {
+  int resident[kNumSizes];
+  LG_TRY((resident_clusters<T, D, G>(resident)));
+  constexpr int rows = Pass<T, D, G>::kTile;
+  CUtensorMap mk, mv;
+  if (!make_kv_map(&mk, a.K, Elem<T>::kDtype, D, rows_total, rows) ||
+      !make_kv_map(&mv, a.V, Elem<T>::kDtype, D, rows_total, rows))
+    return cudaErrorInvalidValue;
+  const ClusterShape sh =
+      cluster_shape(a.n_layers * a.batch * a.H_kv, (a.max_len + rows - 1) / rows,
+                    ClusterCfg<T, D, G>::kTileBytes, Pass<T, D, G>::kTileUs, resident);
+  auto kern = attend_cluster_kernel<T, D, G>;
+  LG_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              ClusterCfg<T, D, G>::kSmem));
+  ClusterLaunch<T, D, G> l(sh.clusters, sh.ctas, s);
+  return cudaLaunchKernelEx(&l.cfg, kern, mk, mv, a, sh.ctas, sh.clusters);
+}
+
+template <typename T, int D>
+cudaError_t launch_cluster_d(const AttendArgs &a, int g, int64_t rows_total, cudaStream_t s) {
+  switch (g) {
+    case 1: return launch_cluster_typed<T, D, 1>(a, rows_total, s);
+    case 2: return launch_cluster_typed<T, D, 2>(a, rows_total, s);
+    case 3: return launch_cluster_typed<T, D, 3>(a, rows_total, s);
+    case 4: return launch_cluster_typed<T, D, 4>(a, rows_total, s);
+    case 5: return launch_cluster_typed<T, D, 5>(a, rows_total, s);
+    case 6: return launch_cluster_typed<T, D, 6>(a, rows_total, s);
+    case 7: return launch_cluster_typed<T, D, 7>(a, rows_total, s);
+    case 8: return launch_cluster_typed<T, D, 8>(a, rows_total, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
+// the pass over a cache of rows_total rows of T
+template <typename T>
+cudaError_t launch_cluster(const AttendArgs &a, int d, int g, int64_t rows_total, cudaStream_t s) {
+  if (d == 128) return launch_cluster_d<T, 128>(a, g, rows_total, s);
+  if (d == 64) return launch_cluster_d<T, 64>(a, g, rows_total, s);
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+}  // namespace lg

@@ -663,17 +663,19 @@ cudaError_t launch_mma_d(const CUtensorMap &mk, const CUtensorMap &mv, const Att
 
 }  // namespace
 
-// 2-D view [L * H_kv * S_total rows][d] of one cache tensor, boxes of 128 rows x 64 columns
-bool make_kv_map(CUtensorMap *m, const void *base, int d, int64_t rows) {
+// 2-D view [L * H_kv * S_total rows][d] of one cache tensor, in boxes of 128-byte rows
+bool make_kv_map(CUtensorMap *m, const void *base, int dtype, int d, int64_t rows, int box_rows) {
   auto fn = encode_fn();
   if (!fn) return false;
+  const int size = dtype == LG_BF16 ? 2 : 4;
   cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)d * 2};
-  cuuint32_t box[2] = {64, (cuuint32_t)kTileRows};
+  cuuint64_t strides[1] = {(cuuint64_t)d * size};
+  cuuint32_t box[2] = {(cuuint32_t)(128 / size), (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return fn(m, dtype == LG_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+            2, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 int mma_tile_rows() { return kTile; }
@@ -681,7 +683,7 @@ int mma_tile_rows() { return kTile; }
 cudaError_t launch_attend_mma_partial(const AttendArgs &a, int d, int g, int64_t rows_total,
                                       cudaStream_t s) {
   CUtensorMap mk, mv;
-  if (!make_kv_map(&mk, a.K, d, rows_total) || !make_kv_map(&mv, a.V, d, rows_total))
+  if (!make_kv_map(&mk, a.K, LG_BF16, d, rows_total, kTile) || !make_kv_map(&mv, a.V, LG_BF16, d, rows_total, kTile))
     return cudaErrorInvalidValue;
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);

@@ -262,4 +262,48 @@ struct Elem<float> {
 __host__ __device__ constexpr int ilog2(int x) { return x <= 1 ? 0 : 1 + ilog2(x / 2); }
 __host__ __device__ constexpr int pow2_ceil(int x) { return x <= 1 ? 1 : 2 * pow2_ceil((x + 1) / 2); }
 
+// Leaves in v[0] the sum over the LPR lanes of a row of the partials of head
+// lane_in_row / (LPR / GP): halving levels first (each lane keeps half of its heads and sends
+// the other half to its partner), plain butterfly levels after.
+template <int CNT, int OFF>
+struct HeadReduce {
+  __device__ __forceinline__ static void run(float *v, int lane) {
+    if constexpr (CNT > 1) {
+      constexpr int H = CNT / 2;
+      const bool upper = (lane & OFF) != 0;
+#pragma unroll
+      for (int i = 0; i < H; ++i) {
+        const float send = upper ? v[i] : v[i + H];
+        const float keep = upper ? v[i + H] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, OFF);
+      }
+      HeadReduce<H, OFF / 2>::run(v, lane);
+    } else if constexpr (OFF >= 1) {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], OFF);
+      HeadReduce<1, OFF / 2>::run(v, lane);
+    }
+  }
+  // the same for N rows at once, level by level (their shuffles do not wait for one another)
+  template <int N, int M>
+  __device__ __forceinline__ static void run_all(float (&v)[N][M], int lane) {
+    if constexpr (CNT > 1) {
+      constexpr int H = CNT / 2;
+      const bool upper = (lane & OFF) != 0;
+#pragma unroll
+      for (int i = 0; i < H; ++i)
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+          const float send = upper ? v[n][i] : v[n][i + H];
+          const float keep = upper ? v[n][i + H] : v[n][i];
+          v[n][i] = keep + __shfl_xor_sync(0xffffffffu, send, OFF);
+        }
+      HeadReduce<H, OFF / 2>::run_all(v, lane);
+    } else if constexpr (OFF >= 1) {
+#pragma unroll
+      for (int n = 0; n < N; ++n) v[n][0] += __shfl_xor_sync(0xffffffffu, v[n][0], OFF);
+      HeadReduce<1, OFF / 2>::run_all(v, lane);
+    }
+  }
+};
+
 }  // namespace lg

@@ -302,7 +302,7 @@ __device__ __forceinline__ void tile_update(WarpSums<D> &acc, const uint32_t (&q
   if (tile_rows < r_w + kRows) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// tensor map of one cache tensor: [rows][d] bf16, boxes of 128 rows x 64 columns
-bool make_kv_map(CUtensorMap *m, const void *base, int d, int64_t rows);
+// tensor map of one cache tensor [rows][d] of a dtype: boxes of box_rows rows x 128 bytes
+bool make_kv_map(CUtensorMap *m, const void *base, int dtype, int d, int64_t rows, int box_rows);
 
 }  // namespace lg

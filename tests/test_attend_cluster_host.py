@@ -1,4 +1,4 @@
-"""The cluster pass's bookkeeping (quick_div, TileSpace, run_bound in csrc/lg_attend_cluster.cu),
+"""The cluster pass's bookkeeping (quick_div, TileSpace, run_bound in csrc/lg_attend_cluster.cuh),
 compiled for the host from the kernel's own source text, over random batches with empty and
 uneven sequences: quotients exact over their range with the float division off by two units in
 the last place either way; tiles found in their groups; clusters' runs and their CTAs' ranges that cover
@@ -14,7 +14,7 @@ import pytest
 from test_attend_geometry_host import _block
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-SRC = os.path.join(ROOT, "paper_2604_10044_gb300", "csrc", "lg_attend_cluster.cu")
+SRC = os.path.join(ROOT, "paper_2604_10044_gb300", "csrc", "lg_attend_cluster.cuh")
 
 HARNESS = r'''
 #include <cmath>
@@ -27,7 +27,7 @@ HARNESS = r'''
 #define __device__
 #define __forceinline__ inline
 using std::max; using std::min;
-constexpr int kTileRows = 128, kClusterSeqs = 64, kMaxCluster = 8;
+constexpr int kClusterSeqs = 64, kMaxCluster = 8;
 static int g_ulp = 0;  // error of the float division, units in the last place
 static inline float __fdividef(float a, float b) {
   float q = a / b;
@@ -51,13 +51,14 @@ int main() {
     const int batch = (int)pick(1, 64), H_kv = (int)pick(1, 8), L = (int)pick(1, 6);
     std::vector<int> len(batch), pre(batch);
     int total = 0;
+    const int rows = it %% 2 ? 128 : 32;
     const int top = (int)pick(1, it %% 3 ? 3000 : 60000);
     for (int b = 0; b < batch; ++b) {
       len[b] = pick(0, 3) ? (int)pick(0, top) : 0;
       pre[b] = total;
-      total += (len[b] + kTileRows - 1) / kTileRows;
+      total += (len[b] + rows - 1) / rows;
     }
-    TileSpace ts{len.data(), pre.data(), batch, H_kv, L, total};
+    TileSpace ts{len.data(), pre.data(), batch, H_kv, L, total, rows};
     const int T = total * H_kv * L;
     if (T == 0 || T >= 1 << 20) continue;
     TileGroup g = ts.find(0);
@@ -100,7 +101,7 @@ def test_cluster_bookkeeping():
         pytest.skip("needs g++")
     text = open(SRC).read()
     assert re.search(r"kClusterSeqs = 64;", text) and re.search(r"kMaxCluster = 8;", text)
-    assert "groups <= 1 << 16 && tiles < 1 << 20" in text  # the ranges checked here
+    assert "groups <= 1 << 16 && tiles < 1 << 20" in open(SRC[:-1]).read()  # the ranges checked here
     code = "\n".join([_block(text, r"^__device__ __forceinline__ int quick_div\("),
                       _block(text, r"^struct TileGroup \{"), _block(text, r"^struct TileSpace \{"),
                       _block(text, r"^__device__ __forceinline__ int run_bound\(")])

@@ -1,6 +1,6 @@
-"""The cluster pass of lg_decode_attend (bf16, batch up to 64) against a plain fp64 attention and
-against the persistent pass on the same cache: empty sequences appended until the batch passes
-the cluster pass's limit send the same call there.
+"""The cluster pass of lg_decode_attend (batch up to 64) against a plain fp64 attention and against
+the general pass on the same cache: empty sequences appended until the batch passes the cluster
+pass's limit send the same call there.
 
 Lengths around its 128-row tiles, empty and one-row sequences, equal lengths (the clusters' runs
 known before the lengths) and uneven ones, groups within one CTA, shared by two, by a whole
@@ -14,7 +14,7 @@ from paper_2604_10044_gb300 import lg
 
 pytestmark = pytest.mark.gpu
 
-LIMIT = 64  # kClusterSeqs in csrc/lg_attend_cluster.cu
+LIMIT = 64  # kClusterSeqs in csrc/lg_attend_cluster.cuh
 
 
 def _run(k, v, q, lens, layer0, n_layers, suffix_w, h2o, pad):
@@ -28,10 +28,11 @@ def _run(k, v, q, lens, layer0, n_layers, suffix_w, h2o, pad):
     kk, vv = (torch.cat([x, torch.full((L, H_kv, extra, d), 3.0, dtype=x.dtype, device=x.device)],
                         2) for x in (k, v))
     n = np.concatenate([lens, np.zeros(pad, np.int64)]).astype(np.int32)
-    c = lg.Cache(L, H_kv, d, "bf16", off, cap, n, k.device, "h2o" if h2o else "loopguard", kk, vv)
+    c = lg.Cache(L, H_kv, d, "bf16" if k.dtype == torch.bfloat16 else "f32", off, cap, n, k.device,
+                 "h2o" if h2o else "loopguard", kk, vv)
     g = lg.Guard(c, H_q, policy="h2o" if h2o else "loopguard", n_layers_per_call=n_layers)
     qq = torch.cat([q, torch.ones((n_layers, pad, H_q, d), dtype=q.dtype, device=q.device)], 1)
-    out = torch.full((n_layers, b + pad, H_q, d), 7.0, dtype=torch.bfloat16, device=k.device)
+    out = torch.full((n_layers, b + pad, H_q, d), 7.0, dtype=k.dtype, device=k.device)
     st = torch.full((n_layers, b + pad, H_q, 4), 7.0, dtype=torch.float32, device=k.device)
     lg.lg_decode_attend(c, layer0, n_layers, qq.contiguous(), H_q, g.scale, out, st, suffix_w,
                         1 if h2o else 0, int(cap.max()), g.ws)
@@ -59,8 +60,8 @@ def _exact(k, v, q, lens, off, layer0, n_layers, suffix_w):
             a = e / t
             out[l, b] = (a @ V).reshape(H_q, d)
             H = torch.log(t[..., 0]) - (a * (z - m)).sum(-1)
-            st[l, b] = torch.stack([m[..., 0], t[..., 0], H, a[..., -min(suffix_w, int(n)):].sum(-1)],
-                                   -1).reshape(H_q, 4)
+            S = a[..., -min(suffix_w, int(n)):].sum(-1)
+            st[l, b] = torch.stack([m[..., 0], t[..., 0], H, S], -1).reshape(H_q, 4)
     return out, st
 
 
@@ -84,27 +85,29 @@ CASES = [  # lengths, H_kv, G, d, layers of the call
 ]
 
 
-@pytest.mark.parametrize("h2o", [False, True])
+@pytest.mark.parametrize("dtype,h2o", [("bf16", False), ("bf16", True), ("f32", False),
+                                       ("f32", True)])
 @pytest.mark.parametrize("lens,H_kv,G,d,nl", CASES)
-def test_cluster_pass(cuda, lens, H_kv, G, d, nl, h2o):
+def test_cluster_pass(cuda, lens, H_kv, G, d, nl, dtype, h2o):
     assert len(lens) <= LIMIT
     g = torch.Generator(device=cuda)
     g.manual_seed(len(lens) * 1000 + G * 10 + d)
     L, S = nl + 1, int(sum(lens)) + len(lens)
-    k, v = (torch.randn((L, H_kv, S, d), generator=g, device=cuda).to(torch.bfloat16)
-            for _ in range(2))
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    k, v = (torch.randn((L, H_kv, S, d), generator=g, device=cuda).to(tdt) for _ in range(2))
     k *= 1.5
-    q = torch.randn((nl, len(lens), H_kv * G, d), generator=g, device=cuda).to(torch.bfloat16)
+    q = torch.randn((nl, len(lens), H_kv * G, d), generator=g, device=cuda).to(tdt)
     got, st, sc, off = _run(k, v, q, lens, 1, nl, 50, h2o, 0)
     want, ws = _exact(k, v, q, lens, off, 1, nl, 50)
     # the parity tests' bounds: bf16 output rounding, fp32 sums
-    _close(got, want, 2e-2, 1e-3, "out")
+    _close(got, want, *((2e-2, 1e-3) if dtype == "bf16" else (1e-4, 1e-5)), "out")
     _close(st, ws, 1e-4, 1e-6, "stats")
     gen, gst, gsc, _ = _run(k, v, q, lens, 1, nl, 50, h2o, LIMIT + 1 - len(lens))
-    # both within 2^-8 of the same value: they differ by one bf16 step at most
-    _close(got, gen, 2.0 ** -7, 1e-5, "out against the persistent pass")
-    _close(st, gst, 2e-5, 1e-6, "stats against the persistent pass")
+    # bf16: both within 2^-8 of the same value, so they differ by one step at most
+    _close(got, gen, 2.0 ** -7 if dtype == "bf16" else 2e-5, 1e-5, "out against the general pass")
+    _close(st, gst, 2e-5, 1e-6, "stats against the general pass")
     if h2o:
-        _close(sc, gsc, 2e-5, 1e-9, "scores against the persistent pass")
-        total = sc.double().sum(-1)  # every non-empty sequence adds G to its kv-head's scores
-        assert torch.allclose(total, torch.full_like(total, G * sum(n > 0 for n in lens)), rtol=1e-5)
+        _close(sc, gsc, 2e-5, 1e-9, "scores against the general pass")
+        # every non-empty sequence adds G to its kv-head's scores
+        total, all_ = sc.double().sum(-1), float(G * sum(n > 0 for n in lens))
+        assert torch.allclose(total, torch.full_like(total, all_), rtol=1e-5)
