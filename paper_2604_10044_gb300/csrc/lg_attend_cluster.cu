@@ -16,6 +16,7 @@ struct Pass<__nv_bfloat16, D, G> {
   static constexpr int kWarps = G <= 4 ? 8 : 4;
   static constexpr int kBlocks = kTile / 16 / kWarps;  // 16-row blocks of a warp
   static constexpr float kTileUs = 0.72f * D / 128.f;  // one CTA's time for a tile
+  static constexpr int kFoldUnits = 1;
 
   WarpSums<D> acc;
   uint32_t qf[D / 16][2];

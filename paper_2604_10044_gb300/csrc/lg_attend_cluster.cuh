@@ -17,9 +17,9 @@
 // (one CTA streams up to 80 GB/s, 1.6 times its even share).
 //
 // GB300, one layer of 28 (append and attention, called one by one in a graph), one sequence of
-// 1024 rows, 16/8 heads of 128: 12.0 -> 7.3 us.  Of a CTA's 5.0 us after its wait, 0.5 go to the
-// lengths, 0.4 to its range and first copy, 1.1 to that copy, 0.8 to the tile, 1.0 to the fold,
-// 0.5 to the barrier and 0.5 to the merge (clock64 at each phase).
+// 1024 rows, 16/8 heads of 128: 12.0 -> 6.4 us.  Of a CTA's 4.4 us after its wait, 0.3 go to the
+// lengths, 0.5 to its range and first copy, 1.3 to that copy, 0.7 to the tile, 0.8 to the fold,
+// 0.4 to the barrier and 0.4 to the merge (clock64 at each phase).
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -61,7 +61,19 @@ struct ClusterCfg {
   static constexpr int kQBytes = G * D * kSize;         // a group's query rows
   static constexpr int kRow = D + 4;                    // one head's o, then {M, l, u, sigma}
   static constexpr int kWarpFloats = kWarps * G * kRow;  // one segment's warp partials
-  static constexpr int kUnits = G * (D / 32);           // (head, 32 output elements) of a group
+  // a group's output in units of 32 elements of a head: unit u is elements 32 (u / G) ... of
+  // head u mod G
+  static constexpr int kUnits = G * (D / 32);
+  // the fold of a segment: kTasks warps, each kTaskUnits units of one head, for which the weights
+  // of the warps' partials are formed once (Pass::kFoldUnits units at most: same-box A/B of 1
+  // against 4, the fp32 layer of 4 sequences of 8191 rows 47.5 -> 45.6 us, the bf16 one of 16384
+  // rows 17.2 -> 17.7, its tile loop short of registers)
+  static constexpr int split() {
+    int s = 1;
+    while (2 * s <= D / 32 && (G * 2 * s <= kWarps || D / 32 / s > P::kFoldUnits)) s *= 2;
+    return s;
+  }
+  static constexpr int kTasks = G * split(), kTaskUnits = D / 32 / split();
   static constexpr int kUnit = 36;                      // floats of a unit's partial: o, then stats
   // a CTA owns every np-th unit of a group shared by np CTAs and receives np partials of each
   static constexpr int recv_max() {
@@ -258,6 +270,12 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
       g.lloc = quick_div(lb, a.batch);
       g.b = lb - g.lloc * a.batch;
     }
+    // cache row of slot 0 of a group's layer and kv-head (the first group's before the wait)
+    auto stream_row = [&](const TileGroup &g) {
+      return (int)(((int64_t)(a.layer0 + g.lloc) * a.H_kv + g.kvh) * a.S_total);
+    };
+    int row0 = stream_row(g);
+    const int first_kvh = g.kvh, first_lloc = g.lloc;
     pdl_enter();
     // lengths and the tiles before each sequence, two sequences a lane
     int n[2], t[2], any_empty = 0;
@@ -349,15 +367,9 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
       bool ok = true;
       for (int t = u0; t < u1 && ok; ++seg) {
         const int end = min(g.start + g.tiles, u1);
-        const int row = (int)(((int64_t)(a.layer0 + g.lloc) * a.H_kv + g.kvh) * a.S_total) +
-                        s_off[g.b] - g.start * kTile;
-        const int64_t head0 = ((int64_t)g.lloc * a.batch + g.b) * a.H_q + (int64_t)g.kvh * G;
-        const int qb = seg & 1;
-        if (seg >= 2 && timed_out(&q_empty[qb], ((seg >> 1) - 1) & 1)) break;
-        mbar_arrive_expect_tx(&q_full[qb], Cl::kQBytes);
-        bulk_load(qbuf + qb * Cl::kQBytes, (const unsigned char *)a.q + head0 * D * Cl::kSize,
-                  Cl::kQBytes, &q_full[qb]);
-        for (; t < end; ++t, ++it) {
+        if (seg > 0 || g.kvh != first_kvh || g.lloc != first_lloc) row0 = stream_row(g);
+        const int row = row0 + s_off[g.b] - g.start * kTile;
+        for (bool first = true; t < end; ++t, ++it, first = false) {
           const int st = it % Cl::kStages;
           if (it >= (uint32_t)Cl::kStages &&
               timed_out(&empty_bar[st], ((it / Cl::kStages) - 1) & 1)) {
@@ -372,6 +384,17 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
                         &full_bar[st], policy);
             tma_load_2d(stage + (P::kBoxes + h) * Cl::kBoxBytes, &tmV, h * P::kBoxCols,
                         row + t * kTile, &full_bar[st], policy);
+          }
+          if (first) {
+            const int64_t head0 = ((int64_t)g.lloc * a.batch + g.b) * a.H_q + (int64_t)g.kvh * G;
+            const int qb = seg & 1;
+            if (seg >= 2 && timed_out(&q_empty[qb], ((seg >> 1) - 1) & 1)) {
+              ok = false;
+              break;
+            }
+            mbar_arrive_expect_tx(&q_full[qb], Cl::kQBytes);
+            bulk_load(qbuf + qb * Cl::kQBytes, (const unsigned char *)a.q + head0 * D * Cl::kSize,
+                      Cl::kQBytes, &q_full[qb]);
           }
         }
         if (ok && t < u1) ts.next(g);
@@ -409,6 +432,14 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     s.np = __popc(mask);
     return s;
   };
+  // where this CTA's partial of a group's unit goes: the owner, sharer number un % np, and its
+  // slot of this group
+  auto unit_addr = [&](const Sharers &sh, const TileGroup &g, int un) {
+    const int j = quick_div(un, sh.np);
+    const int owner = __ffs(__ballot_sync(0xffffffffu, sh.nth == un - j * sh.np)) - 1;
+    const int slot = __shfl_sync(0xffffffffu, sh.lo, owner) >= g.start ? 0 : 1;
+    return peer_addr(recv + slot * Cl::kRecvFloats + (j * sh.np + sh.mine) * Cl::kUnit, owner);
+  };
   const int u0 = first_tile(rank), u1 = first_tile(rank + 1);
   TileGroup g = {};
   if (u0 < u1) g = ts.find(u0);
@@ -425,8 +456,12 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     }
   }
   // groups in the slots: 0 for a segment that starts at u0, 1 for another that ends at u1
-  bool shared0 = false, shared1 = false;
-  TileGroup grp0 = {}, grp1 = {};
+  // (np 0: not in use; mine and np as above, the group's first head)
+  struct Slot {
+    int mine, np;
+    int64_t head0;
+  };
+  Slot slot0 = {}, slot1 = {};
   P pass;
   uint32_t it = 0, seg = 0;
   bool ok = true;  // false once a copy did not land in time (the barriers below stay matched)
@@ -443,6 +478,16 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     const int suffix_lo = n - min(a.suffix_w, n);
     const int64_t lrow = ((int64_t)g.lloc * a.H_kv + g.kvh) * a.S_total + s_off[g.b];
     const int qb = seg & 1;
+    // who shares the group and where this warp's first unit goes, formed while the first copies
+    // are in flight (after the tiles they would sit on the way to the merge)
+    const bool whole = start == g.start && end == g.start + g.tiles;
+    const int64_t head0 = ((int64_t)g.lloc * a.batch + g.b) * a.H_q + (int64_t)g.kvh * G;
+    Sharers sh = {};
+    uint32_t dst0 = 0;
+    if (!whole) {
+      sh = sharers(g);
+      dst0 = unit_addr(sh, g, warp / G * Cl::kTaskUnits * G + warp % G);
+    }
     if (landed(&q_full[qb], (seg >> 1) & 1)) pass.begin(qbuf + qb * Cl::kQBytes, a.qscale, lane);
     for (; t < end; ++t, ++it) {
       const int st = it % Cl::kStages;
@@ -457,58 +502,46 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     // the segment's warp partials folded: a whole group is finished here, a part of a group goes
     // to the owners of its units
     pass.join();
-    const bool whole = start == g.start && end == g.start + g.tiles;
-    const int64_t head0 = ((int64_t)g.lloc * a.batch + g.b) * a.H_q + (int64_t)g.kvh * G;
-    Sharers sh = {};
-    if (!whole) sh = sharers(g);
     if (start != u0) named_sync<kWarps * 32>(2);  // the segment before has been folded
     pass.store(part + warp * G * kRow, lane);
     named_sync<kWarps * 32>(2);
 #pragma unroll 1
-    for (int un = warp; un < Cl::kUnits; un += kWarps) {
-      const int h = un / (D / 32), e = un % (D / 32) * 32 + lane;
-      uint32_t dst = 0;
-      if (!whole) {
-        // the owner, sharer number un % np, and its slot of this group
-        const int j = quick_div(un, sh.np);
-        const int owner = __ffs(__ballot_sync(0xffffffffu, sh.nth == un - j * sh.np)) - 1;
-        const int slot = __shfl_sync(0xffffffffu, sh.lo, owner) >= g.start ? 0 : 1;
-        dst = peer_addr(recv + slot * Cl::kRecvFloats + (j * sh.np + sh.mine) * Cl::kUnit, owner);
-      }
-      float4 w4[kWarps];
-      float wo[kWarps];
-      float M = -INFINITY;
+    for (int task = warp; task < Cl::kTasks; task += kWarps) {
+      const int h = task % G, first_slice = task / G * Cl::kTaskUnits;
+      float f[kWarps], M = -INFINITY, l = 0.f, u = 0.f, sg = 0.f;
+      {
+        float4 w4[kWarps];
 #pragma unroll
-      for (int w = 0; w < kWarps; ++w) {
-        w4[w] = *reinterpret_cast<const float4 *>(part + (w * G + h) * kRow + D);
-        wo[w] = part[(w * G + h) * kRow + e];
-        M = fmaxf(M, w4[w].x);
-      }
-      float l = 0.f, u = 0.f, sg = 0.f, o = 0.f;
+        for (int w = 0; w < kWarps; ++w) {
+          w4[w] = *reinterpret_cast<const float4 *>(part + (w * G + h) * kRow + D);
+          M = fmaxf(M, w4[w].x);
+        }
 #pragma unroll
-      for (int w = 0; w < kWarps; ++w) {
-        // a warp that saw no row of this segment has l = u = 0 and M = -inf: no weight
-        const float dm = fmaxf(w4[w].x - M, -1e30f);
-        const float f = exp2f(dm);
-        l += f * w4[w].y;
-        u += f * (w4[w].z + dm * w4[w].y);
-        sg += f * w4[w].w;
-        o += f * wo[w];
+        for (int w = 0; w < kWarps; ++w) {
+          // a warp that saw no row of this segment has l = u = 0 and M = -inf: no weight
+          const float dm = fmaxf(w4[w].x - M, -1e30f);
+          f[w] = exp2f(dm);
+          l += f[w] * w4[w].y;
+          u += f[w] * (w4[w].z + dm * w4[w].y);
+          sg += f[w] * w4[w].w;
+        }
       }
-      if (whole) {
-        finish<T, D>(a, head0 + h, e, un % (D / 32) == 0 && lane == 0, M, l, u, sg, o);
-      } else {
-        peer_st(dst + lane * 4, o);
-        if (lane == 0) peer_st4(dst + 32 * 4, make_float4(M, l, u, sg));
+#pragma unroll
+      for (int k = 0; k < Cl::kTaskUnits; ++k) {
+        const int slice = first_slice + k, un = slice * G + h, e = slice * 32 + lane;
+        float o = 0.f;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) o += f[w] * part[(w * G + h) * kRow + e];
+        if (whole) {
+          finish<T, D>(a, head0 + h, e, slice == 0 && lane == 0, M, l, u, sg, o);
+        } else {
+          const uint32_t dst = k == 0 && task == warp ? dst0 : unit_addr(sh, g, un);
+          peer_st(dst + lane * 4, o);
+          if (lane == 0) peer_st4(dst + 32 * 4, make_float4(M, l, u, sg));
+        }
       }
     }
-    if (!whole && start == u0) {
-      shared0 = true;
-      grp0 = g;
-    } else if (!whole) {
-      shared1 = true;
-      grp1 = g;
-    }
+    if (!whole) (start == u0 ? slot0 : slot1) = Slot{sh.mine, sh.np, head0};
     if (t < u1) ts.next(g);
   }
   __syncwarp();
@@ -516,11 +549,9 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
   cluster_wait();  // every partial has arrived
 #pragma unroll 1
   for (int slot = 0; slot < 2; ++slot) {
-    if (!(slot ? shared1 : shared0)) continue;
-    const TileGroup gs = slot ? grp1 : grp0;
-    const Sharers sh = sharers(gs);
-    const int mine = sh.mine, np = sh.np;
-    const int64_t head0 = ((int64_t)gs.lloc * a.batch + gs.b) * a.H_q + (int64_t)gs.kvh * G;
+    const int mine = slot ? slot1.mine : slot0.mine, np = slot ? slot1.np : slot0.np;
+    const int64_t head0 = slot ? slot1.head0 : slot0.head0;
+    if (np == 0) continue;
 #pragma unroll 1
     for (int j = warp; j * np + mine < Cl::kUnits; j += kWarps) {
       const int un = j * np + mine;
@@ -545,8 +576,7 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
         sg += f * s4[r].w;
         o += f * so[r];
       }
-      finish<T, D>(a, head0 + un / (D / 32), un % (D / 32) * 32 + lane,
-                un % (D / 32) == 0 && lane == 0, M, l, u, sg, o);
+      finish<T, D>(a, head0 + un % G, un / G * 32 + lane, un < G && lane == 0, M, l, u, sg, o);
     }
   }
 }
@@ -602,7 +632,10 @@ cudaError_t resident_clusters(int (&n)[kNumSizes]) {
 // Cluster size and count for `groups` groups of at most `tiles` tiles: the size whose estimated
 // time is least.  With K clusters, each takes groups / K groups and then groups mod K of them one
 // more; either phase is bound by the memory (kTilesPerUs tiles a microsecond over all CTAs) or by
-// the CTAs (kTileUs a tile, kSegmentUs a segment end).  Smaller clusters fill the GPU better
+// the CTAs (kTileUs a tile, kSegmentUs a segment end).  Of a batch the host knows the longest
+// length it may have, not the others, so a ragged one (lengths kRagged of the longest on average,
+// as log-uniform ones are) counts as much: its clusters' runs are even but for half of a longest
+// group on one cluster.  Smaller clusters fill the GPU better
 // (152 SMs hold 15, 23, 36, 76, 152 clusters of 8, 6, 4, 2, 1), larger ones split a group further
 // and stream a little better (about a percent per halving on passes of half a millisecond).
 // Measured per call (append and attention, layers called one by one in a graph, us, sizes 8 / 6 /
@@ -612,10 +645,10 @@ cudaError_t resident_clusters(int (&n)[kNumSizes]) {
 struct ClusterShape {
   int ctas, clusters;
 };
-inline ClusterShape cluster_shape(int groups, int tiles, int tile_bytes, float kTileUs,
+inline ClusterShape cluster_shape(int groups, int batch, int tiles, int tile_bytes, float kTileUs,
                                   const int (&resident)[kNumSizes]) {
   const float kTilesPerUs = 7.3e6f / (float)tile_bytes;
-  constexpr float kSegmentUs = 1.f;
+  constexpr float kSegmentUs = 1.f, kRagged = 0.35f;
   ClusterShape best = {1, 1};
   float best_us = 0.f;
   for (int i = 0; i < kNumSizes; ++i) {
@@ -626,6 +659,9 @@ inline ClusterShape cluster_shape(int groups, int tiles, int tile_bytes, float k
                      (float)q * cta + kSegmentUs * (1.f + (float)(q - 1) / (float)c));
     if (r) us += fmaxf((float)r * (float)tiles / kTilesPerUs, cta + kSegmentUs / (float)c);
     us *= 1.f + 0.0125f * log2f((float)kMaxCluster / (float)c);
+    if (batch > 1)
+      us += fmaxf(kRagged * (float)groups * (float)tiles / kTilesPerUs,
+                  kRagged * (float)groups * (float)tiles / (float)(k * c) * kTileUs) + 0.5f * cta;
     if (best_us == 0.f || us < best_us) {
       best_us = us;
       best = {c, k};
@@ -644,7 +680,7 @@ cudaError_t launch_cluster_typed(const AttendArgs &a, int64_t rows_total, cudaSt
       !make_kv_map(&mv, a.V, Elem<T>::kDtype, D, rows_total, rows))
     return cudaErrorInvalidValue;
   const ClusterShape sh =
-      cluster_shape(a.n_layers * a.batch * a.H_kv, (a.max_len + rows - 1) / rows,
+      cluster_shape(a.n_layers * a.batch * a.H_kv, a.batch, (a.max_len + rows - 1) / rows,
                     ClusterCfg<T, D, G>::kTileBytes, Pass<T, D, G>::kTileUs, resident);
   auto kern = attend_cluster_kernel<T, D, G>;
   LG_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,

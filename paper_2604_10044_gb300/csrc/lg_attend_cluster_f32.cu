@@ -24,6 +24,7 @@ struct Pass<float, D, G> {
   static constexpr int kTile = G <= 4 ? 64 : kF32TileMin, kBoxCols = 32, kBoxes = D / 32;
   static constexpr int kStages = (G <= 4 ? 3 : 5) * 128 / D;
   static constexpr int kWarps = 8;
+  static constexpr int kFoldUnits = 4;
   static constexpr float kTileUs = (G <= 4 ? 1.f : 1.2f) * D / 128.f;
   static constexpr int kBox = kTile * 128;       // bytes of a box
   static constexpr int kEpl = G <= 2 ? 16 : (G <= 4 ? 8 : 4);  // elements of a lane

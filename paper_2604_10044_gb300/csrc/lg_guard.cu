@@ -32,20 +32,25 @@ __global__ void begin_step_kernel(lg_cache c) {
     c.len[b] = n + 1;
 }
 
-// Blocks [0, row_blocks): one thread per 16-byte chunk of a new row, written to slot
-// len[b] - 1.  Blocks [row_blocks, row_blocks + batch) when the guard layer is in the call:
-// the sketch of that layer's new V row (read from v_new [n_layers][b][H_kv][d]), a warp per
-// word: lane j reads element 32w + j and the ballot of the sign bits is word w.
-template <typename T>
-__global__ void append_kernel(lg_cache c, int layer0, int n_layers, const uint4 *k_new,
-                              const uint4 *v_new, const int32_t *pos_new, int row_blocks,
-                              int lguard) {
-  pdl_enter_early();
+// Blocks (x < row_blocks, layer y): one thread per 16-byte chunk of a new row, written to slot
+// len[b] - 1.  Blocks x in [row_blocks, row_blocks + batch) of the guard layer when it is in the
+// call: the sketch of that layer's new V row (read from v_new [n_layers][b][H_kv][d]), a warp per
+// word: lane j reads element 32w + j and the ballot of the sign bits is word w.  The indices come
+// before the dependency wait: in a step of one sequence the kernel is one link of a chain of short
+// kernels, bound by what follows the wait (one round trip for all its loads, then the stores).
+// (GB300, layers called one by one in a graph, one sequence of 1024 rows: with the cluster pass's
+// own savings before its first copy and in its fold, 7.25 -> 6.42 us a layer.)
+template <typename T, int D>
+__global__ void append_kernel(lg_cache c, int layer0, const uint4 *k_new, const uint4 *v_new,
+                              const int32_t *pos_new, int row_blocks, int lguard) {
+  constexpr int kCpr = D * (int)sizeof(T) / 16;
   if ((int)blockIdx.x >= row_blocks) {
+    if ((int)blockIdx.y != lguard) return;
     const int b = blockIdx.x - row_blocks;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nwords = c.H_kv * c.d / 32;
-    const T *row = (const T *)v_new + ((int64_t)lguard * c.batch + b) * c.H_kv * c.d;
+    const int nwords = c.H_kv * D / 32;
+    const T *row = (const T *)v_new + ((int64_t)lguard * c.batch + b) * c.H_kv * D;
+    pdl_enter_early();
     // the sign bits this warp packs are requested with the length and the status (one round
     // trip for all), up to 8 words a warp at once
     constexpr int kWordsPerWarp = 8;
@@ -73,16 +78,14 @@ __global__ void append_kernel(lg_cache c, int layer0, int n_layers, const uint4 
     }
     return;
   }
-  const int cpr = c.d * (int)sizeof(T) / 16;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t rows = (int64_t)n_layers * c.batch * c.H_kv;
-  if (t >= rows * cpr) return;
-  const int64_t row = t / cpr;
-  const int ch = (int)(t % cpr);
-  const int kvh = (int)(row % c.H_kv);
-  const int b = (int)((row / c.H_kv) % c.batch);
-  const int layer = layer0 + (int)(row / ((int64_t)c.H_kv * c.batch));
-  const uint4 kr = k_new[row * cpr + ch], vr = v_new[row * cpr + ch];
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;  // chunk of the layer's new rows
+  const unsigned row_l = t / kCpr, ch = t % kCpr;
+  const int b = (int)(row_l / (unsigned)c.H_kv), kvh = (int)(row_l - (unsigned)b * c.H_kv);
+  const int64_t src = (int64_t)blockIdx.y * c.batch * c.H_kv * kCpr + t;
+  const int64_t row0 = ((int64_t)(layer0 + (int)blockIdx.y) * c.H_kv + kvh) * c.S_total;
+  pdl_enter_early();
+  if (b >= c.batch) return;
+  const uint4 kr = k_new[src], vr = v_new[src];
   const int slot = c.len[b] - 1;
   const int64_t off = c.seq_off[b];
   if (status_bad(c.dev_status)) return;
@@ -90,9 +93,9 @@ __global__ void append_kernel(lg_cache c, int layer0, int n_layers, const uint4 
     set_status(c.dev_status, LG_ERR_CAPACITY);
     return;
   }
-  const int64_t s = ((int64_t)layer * c.H_kv + kvh) * c.S_total + off + slot;
-  reinterpret_cast<uint4 *>(c.k)[s * cpr + ch] = kr;
-  reinterpret_cast<uint4 *>(c.v)[s * cpr + ch] = vr;
+  const int64_t s = row0 + off + slot;
+  reinterpret_cast<uint4 *>(c.k)[s * kCpr + ch] = kr;
+  reinterpret_cast<uint4 *>(c.v)[s * kCpr + ch] = vr;
   if (ch == 0 && c.pos) {
     c.pos[s] = pos_new[b];
     c.h2o[s] = 0.f;
@@ -1321,24 +1324,34 @@ cudaError_t launch_begin_step(const lg_cache &c, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+template <typename T, int D>
+static cudaError_t launch_append_typed(const lg_cache &c, int layer0, int n_layers,
+                                       const void *k_new, const void *v_new,
+                                       const int32_t *pos_new, int guard_layer, cudaStream_t s) {
+  constexpr int cpr = D * (int)sizeof(T) / 16;
+  const int64_t chunks = (int64_t)c.batch * c.H_kv * cpr;  // of one layer's new rows
+  // few chunks in blocks of 128 threads: a layer of one sequence then spreads over more SMs
+  const int threads = chunks <= 4096 ? 128 : 256;
+  const int row_blocks = (int)((chunks + threads - 1) / threads);
+  const bool sk = c.sketch && guard_layer >= layer0 && guard_layer < layer0 + n_layers;
+  const dim3 grid(row_blocks + (sk ? c.batch : 0), n_layers);
+  LG_TRY(launch_pdl(append_kernel<T, D>, grid, threads, 0, s, c, layer0, (const uint4 *)k_new,
+                    (const uint4 *)v_new, pos_new, row_blocks, guard_layer - layer0));
+  return cudaGetLastError();
+}
+
 cudaError_t launch_append(const lg_cache &c, int layer0, int n_layers, const void *k_new,
                           const void *v_new, const int32_t *pos_new, int guard_layer,
                           cudaStream_t s) {
-  const int cpr = c.d * (c.dtype == LG_BF16 ? 2 : 4) / 16;
-  const int64_t total = (int64_t)n_layers * c.batch * c.H_kv * cpr;
-  const int row_blocks = (int)((total + 255) / 256);
-  const bool sk = c.sketch && guard_layer >= layer0 && guard_layer < layer0 + n_layers;
-  const int grid = row_blocks + (sk ? c.batch : 0);
-  if (c.dtype == LG_BF16) {
-    LG_TRY(launch_pdl(append_kernel<__nv_bfloat16>, grid, 256, 0, s, c, layer0, n_layers,
-                      (const uint4 *)k_new, (const uint4 *)v_new, pos_new, row_blocks,
-                      guard_layer - layer0));
-  } else {
-    LG_TRY(launch_pdl(append_kernel<float>, grid, 256, 0, s, c, layer0, n_layers,
-                      (const uint4 *)k_new, (const uint4 *)v_new, pos_new, row_blocks,
-                      guard_layer - layer0));
-  }
-  return cudaGetLastError();
+  if (c.dtype == LG_BF16)
+    return c.d == 128 ? launch_append_typed<__nv_bfloat16, 128>(c, layer0, n_layers, k_new, v_new,
+                                                                pos_new, guard_layer, s)
+                      : launch_append_typed<__nv_bfloat16, 64>(c, layer0, n_layers, k_new, v_new,
+                                                               pos_new, guard_layer, s);
+  return c.d == 128 ? launch_append_typed<float, 128>(c, layer0, n_layers, k_new, v_new, pos_new,
+                                                      guard_layer, s)
+                    : launch_append_typed<float, 64>(c, layer0, n_layers, k_new, v_new, pos_new,
+                                                     guard_layer, s);
 }
 
 template <typename T, int D>
