@@ -119,15 +119,21 @@ NOALLOC_SCRATCH_BYTES = 32 << 20  # LG_NOALLOC_SCRATCH_BYTES in include/lg.h
 
 
 def _ptr(t):
-    if t is None:
-        return None
-    if isinstance(t, int):
+    if t is None or isinstance(t, int):
         return t
     return t.data_ptr()
 
 
+# The current stream's handle without building a torch.cuda.Stream around it: 2.8 us of the
+# 8.9 us a lg_decode_attend call took its caller (Grace), more than the launch itself.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_get_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream):
     if stream is None:
+        if _raw_stream is not None and _get_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_get_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -135,7 +141,7 @@ def _stream(stream):
 
 
 def _call(name, *args):
-    rc = getattr(lib(), name)(*args)
+    rc = getattr(_lib or lib(), name)(*args)
     if rc != LG_OK:
         raise LgError(name, rc)
 
