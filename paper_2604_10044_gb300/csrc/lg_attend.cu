@@ -326,18 +326,23 @@ __global__ void __launch_bounds__(256) h2o_accumulate_kernel(AttendArgs a, float
   pdl_enter();
   const int kvh = blockIdx.y, b = blockIdx.z % a.batch, lloc = blockIdx.z / a.batch;
   const int layer = a.layer0 + lloc;
-  if (status_bad(a.status)) return;
+  // the length, the heads' {M, l} and the status in one round trip
   const int n = a.len[b];
-  if (n > a.max_len) return;
-  float M[G], inv_l[G];
+  const int64_t off = a.seq_off[b];
+  float2 ml[G];
   const int64_t head0 = ((int64_t)lloc * a.batch + b) * a.H_q + (int64_t)kvh * G;
 #pragma unroll
+  for (int g = 0; g < G; ++g) ml[g] = reinterpret_cast<const float2 *>(final_ml)[head0 + g];
+  if (status_bad(a.status)) return;
+  if (n > a.max_len) return;
+  float M[G], inv_l[G];
+#pragma unroll
   for (int g = 0; g < G; ++g) {
-    M[g] = final_ml[(head0 + g) * 2];
-    inv_l[g] = 1.f / final_ml[(head0 + g) * 2 + 1];
+    M[g] = ml[g].x;
+    inv_l[g] = 1.f / ml[g].y;
   }
-  const int64_t lrow0 = ((int64_t)lloc * a.H_kv + kvh) * a.S_total + a.seq_off[b];
-  float *sc = h2o + ((int64_t)layer * a.H_kv + kvh) * a.S_total + a.seq_off[b];
+  const int64_t lrow0 = ((int64_t)lloc * a.H_kv + kvh) * a.S_total + off;
+  float *sc = h2o + ((int64_t)layer * a.H_kv + kvh) * a.S_total + off;
   // kH2ORows rows per thread with all their loads in flight; a row's G logits in 16- or 8-byte
   // loads where G allows (the logits start 256-byte aligned, a row at a multiple of 4 G bytes)
   const int stride = gridDim.x * blockDim.x;
@@ -407,11 +412,14 @@ static cudaError_t launch_typed(const AttendArgs &a, int64_t rows_total, void *o
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (h2o) {
-    // at most 16 CTAs a (layer, sequence, kv-head) stream: up to 16 K rows a stream leave each
-    // thread its kH2ORows rows in flight (a grid sized for one row a thread ran with half the
-    // warps resident and most of its CTAs idle on short sequences)
+    // CTAs a (layer, sequence, kv-head) stream: four, or what fills the GPU twice over with few
+    // streams, and no more than its rows need.  Short streams of a ragged batch leave most of a
+    // larger grid idle, and launching it shows (16 sequences up to 8191, 512 streams, the whole
+    // step: 4 CTAs 152.8 us, 2 153.4, 8 155.6).
+    const int streams = a.H_kv * a.n_layers * a.batch;
+    const int want = (2 * 152 * 8 + streams - 1) / streams;
     int gx = (a.max_len + 256 * kH2ORows - 1) / (256 * kH2ORows);
-    if (gx > 16) gx = 16;
+    if (gx > (want > 4 ? want : 4)) gx = want > 4 ? want : 4;
     LG_TRY(launch_pdl(h2o_accumulate_kernel<G>, dim3(gx, a.H_kv, a.n_layers * a.batch), 256, 0, s,
                       a, h2o, final_ml));
     e = cudaGetLastError();
