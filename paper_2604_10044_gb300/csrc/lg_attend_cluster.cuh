@@ -212,7 +212,8 @@ __device__ __forceinline__ void finish(const AttendArgs &a, int64_t head, int e,
 template <typename T, int D, int G>
 __global__ void __launch_bounds__(ClusterCfg<T, D, G>::kThreads, 1)
 attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
-                      const __grid_constant__ CUtensorMap tmV, AttendArgs a, int ctas, int n_cl) {
+                      const __grid_constant__ CUtensorMap tmV, AttendArgs a, int ctas, int n_cl,
+                      int rows_total) {
   using P = Pass<T, D, G>;
   using Cl = ClusterCfg<T, D, G>;
   constexpr int kWarps = Cl::kWarps, kRow = Cl::kRow, kTile = P::kTile;
@@ -276,6 +277,44 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     };
     int row0 = stream_row(g);
     const int first_kvh = g.kvh, first_lloc = g.lloc;
+    // Before the wait, this CTA's first tiles are requested into L2 (all lengths alike: the range
+    // is a few instructions then).  Only hints come of what is read here, past L1: a kernel still
+    // in flight may be writing the lengths and rows, L2 holds what it writes, and everything is
+    // read again after the wait.  In a step the kernel before is a short one (the append), and
+    // without this the memory idles beside it.  (GB300, layers one by one in a graph, 1 sequence
+    // of 1024 rows: 6.39 -> 6.06 us, 8 of 4096 25.7 -> 23.5 us)
+    {
+      int t[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int b = 2 * lane + k;
+        const int n = b < a.batch ? min(__ldcg(a.len + b), a.max_len) : 0;
+        t[k] = (max(n, 0) + kTile - 1) / kTile;
+      }
+      const int tiles = __shfl_sync(0xffffffffu, t[0], 0);
+      const bool same = (2 * lane >= a.batch || t[0] == tiles) &&
+                        (2 * lane + 1 >= a.batch || t[1] == tiles);
+      const int x = lane % (2 * P::kBoxes), i = lane / (2 * P::kBoxes);  // box, tile of this lane
+      if (__all_sync(0xffffffffu, same) && i < Cl::kStages) {
+        const int len = (gi1 - gi0) * tiles;
+        const int u = quick_div(len * rank, ctas) + i;
+        if (u < quick_div(len * (rank + 1), ctas)) {
+          const int skip = quick_div(u, tiles), gi = gi0 + skip;
+          TileGroup gp = g;
+          if (skip > 0) {
+            const int lb = quick_div(gi, a.H_kv);
+            gp.kvh = gi - lb * a.H_kv;
+            gp.lloc = quick_div(lb, a.batch);
+            gp.b = lb - gp.lloc * a.batch;
+          }
+          const int64_t row = stream_row(gp) + __ldcg(a.seq_off + gp.b) +
+                              (int64_t)(u - skip * tiles) * kTile;
+          if (row >= 0 && row < rows_total)
+            tma_prefetch_2d(x < P::kBoxes ? &tmK : &tmV, x % P::kBoxes * P::kBoxCols, (int)row);
+        }
+      }
+      __syncwarp();
+    }
     pdl_enter();
     // lengths and the tiles before each sequence, two sequences a lane
     int n[2], t[2], any_empty = 0;
@@ -686,7 +725,7 @@ cudaError_t launch_cluster_typed(const AttendArgs &a, int64_t rows_total, cudaSt
   LG_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               ClusterCfg<T, D, G>::kSmem));
   ClusterLaunch<T, D, G> l(sh.clusters, sh.ctas, s);
-  return cudaLaunchKernelEx(&l.cfg, kern, mk, mv, a, sh.ctas, sh.clusters);
+  return cudaLaunchKernelEx(&l.cfg, kern, mk, mv, a, sh.ctas, sh.clusters, (int)rows_total);
 }
 
 template <typename T, int D>
