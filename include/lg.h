@@ -20,18 +20,21 @@
  *  - Every pointer inside lg_cache and every array argument marked "device" is device memory
  *    owned by the caller; the library allocates nothing and keeps no global state, except
  *    the static scratch array that lg_decode_attend_noalloc uses in place of a workspace and
- *    two lookups cached for the process (the driver's tensor-map encoder, and per GPU the
- *    compaction kernel's resident CTAs), which no result depends on.
+ *    lookups cached for the process (the driver's tensor-map encoder, and per GPU the compaction
+ *    kernel's resident CTAs and the attention pass's resident clusters), on which at most the
+ *    order of a sum depends.
  *  - Every call is asynchronous on the caller's stream; nothing synchronises except
  *    lg_read_device_status.
  *  - Kernels are launched with programmatic stream serialization (programmatic dependent
  *    launch): each may be scheduled while the kernel before it in the stream is still running,
  *    and waits (griddepcontrol.wait) for that kernel to complete before it touches memory, so
- *    stream order holds as usual.  One exception, invisible to the caller: lg_detect's kernel
+ *    stream order holds as usual.  Two exceptions, invisible to the caller: lg_detect's kernel
  *    reads the lengths, the monitor state and the sketches before its wait, then reads the
  *    length, the synced length and the new row again after it and drops everything read early
- *    unless all three are unchanged.  Only a library kernel can be running at that point: a
- *    kernel of the caller's (launched without the attribute) completes before the next
+ *    unless all three are unchanged; and lg_decode_attend's kernel reads the lengths and the
+ *    sequence offsets before its wait to ask for its first rows sooner, reads them again after
+ *    it and drops what was fetched for others.  Only a library kernel can be running at that
+ *    point: a kernel of the caller's (launched without the attribute) completes before the next
  *    kernel starts.  A kernel of the caller's that follows one of the library's on the same
  *    stream keeps full stream order unless the caller launches it with the same attribute, in
  *    which case it must wait the same way.
@@ -181,10 +184,11 @@ LG_API lg_status lg_sketch_build(const lg_cache *c, const lg_guard_params *p, in
    stats: device [n_layers][batch][H_q][4] fp32.  Query head h reads kv-head h / (H_q/H_kv).
    accumulate_h2o: also add sum over the GQA group of a_i to h2o[l][kvh][slot] (c->h2o).
    max_len: host bound on every len[b] (sizes the grid; a longer sequence is an error).
-   ws: device workspace of at least lg_workspace_size(...) bytes, 256-byte aligned.  On the bf16
-   path successive calls with one workspace walk the cache in alternating directions (one word
-   of ws keeps the direction), so that a call starts on the rows the previous call read last,
-   which may still be in L2; no result depends on the direction. */
+   ws: device workspace of at least lg_workspace_size(...) bytes, 256-byte aligned.  Batches of up
+   to 64 sequences use only its logits and {M, l} part (accumulate_h2o); bf16 calls with more
+   walk the cache in alternating directions from call to call (one word of ws keeps the
+   direction), so that a call starts on the rows the previous call read last, which may still be
+   in L2; no result depends on the direction. */
 LG_API lg_status lg_decode_attend(const lg_cache *c, int layer0, int n_layers, const void *q, int H_q,
                            float scale, void *out, float *stats, int suffix_w,
                            int accumulate_h2o, int max_len, void *ws, size_t ws_bytes,

@@ -222,7 +222,7 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
   __shared__ __align__(8) uint64_t empty_bar[Cl::kStages];
   __shared__ __align__(8) uint64_t q_full[2], q_empty[2];  // query rows of segment i in buffer i & 1
   __shared__ int s_len[kClusterSeqs], s_pre[kClusterSeqs], s_off[kClusterSeqs];
-  __shared__ int s_total, s_c0, s_c1, s_empty;
+  __shared__ int s_total, s_c0, s_c1, s_empty, s_skip;
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   unsigned char *qbuf = smem + Cl::kStages * Cl::kStageBytes;  // [2][G][D]
@@ -231,6 +231,16 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = cluster_rank(), cluster = quick_div(blockIdx.x, ctas);
+  // the producer's early look at the lengths and offsets (see there), two sequences a lane
+  int early_n[2] = {0, 0}, early_off[2] = {0, 0};
+  if (warp == kWarps) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+      if (2 * lane + k < a.batch) {
+        early_n[k] = __ldcg(a.len + 2 * lane + k);
+        early_off[k] = (int)__ldcg(a.seq_off + 2 * lane + k);
+      }
+  }
   cluster_arrive();  // waited for before the first store to a peer: every CTA has started then
   if (threadIdx.x == kWarps * 32) {
     for (int s = 0; s < Cl::kStages; ++s) {
@@ -277,64 +287,112 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     };
     int row0 = stream_row(g);
     const int first_kvh = g.kvh, first_lloc = g.lloc;
-    // Before the wait, this CTA's first tiles are requested into L2 (all lengths alike: the range
-    // is a few instructions then).  Only hints come of what is read here, past L1: a kernel still
-    // in flight may be writing the lengths and rows, L2 holds what it writes, and everything is
-    // read again after the wait.  In a step the kernel before is a short one (the append), and
-    // without this the memory idles beside it.  (GB300, layers one by one in a graph, 1 sequence
-    // of 1024 rows: 6.39 -> 6.06 us, 8 of 4096 25.7 -> 23.5 us)
+    // Before the wait, the lengths as they are now (past L1) give the range this CTA will most
+    // likely have, if they all agree (a few instructions then).  Its first tiles are requested into
+    // L2, a hint: in a step the kernel before is a short one (the append), beside which the memory
+    // idled.  In a call of few tiles a CTA, bound by latency, the copies of its first segment are
+    // then issued right after the wait, beside the read of the lengths that count; if those give
+    // another range, the copies are dropped (the consumers pass over their stages).  What is read
+    // early decides only which rows are fetched first.  (GB300, layers one by one in a graph: 1
+    // sequence of 1024 rows 6.39 us, 6.06 with the L2 requests, 5.73 with the early copies; 8 of
+    // 4096 rows 25.7, 23.5 and, as longer calls gain nothing from them, 24.0.)
+    int guess_t[2], guess_tiles = 0, guess_row = 0, guess_off = 0;
+    TileGroup guess = g;  // the first segment's group; guess_tiles of its tiles, from guess_row on
     {
-      int t[2];
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int b = 2 * lane + k;
-        const int n = b < a.batch ? min(__ldcg(a.len + b), a.max_len) : 0;
-        t[k] = (max(n, 0) + kTile - 1) / kTile;
-      }
-      const int tiles = __shfl_sync(0xffffffffu, t[0], 0);
-      const bool same = (2 * lane >= a.batch || t[0] == tiles) &&
-                        (2 * lane + 1 >= a.batch || t[1] == tiles);
-      const int x = lane % (2 * P::kBoxes), i = lane / (2 * P::kBoxes);  // box, tile of this lane
-      if (__all_sync(0xffffffffu, same) && i < Cl::kStages) {
+      for (int k = 0; k < 2; ++k)
+        guess_t[k] = (max(min(early_n[k], a.max_len), 0) + kTile - 1) / kTile;
+      const int tiles = __shfl_sync(0xffffffffu, guess_t[0], 0);
+      const bool same = (2 * lane >= a.batch || guess_t[0] == tiles) &&
+                        (2 * lane + 1 >= a.batch || guess_t[1] == tiles);
+      if (__all_sync(0xffffffffu, same) && tiles > 0) {
         const int len = (gi1 - gi0) * tiles;
-        const int u = quick_div(len * rank, ctas) + i;
-        if (u < quick_div(len * (rank + 1), ctas)) {
-          const int skip = quick_div(u, tiles), gi = gi0 + skip;
-          TileGroup gp = g;
-          if (skip > 0) {
-            const int lb = quick_div(gi, a.H_kv);
-            gp.kvh = gi - lb * a.H_kv;
-            gp.lloc = quick_div(lb, a.batch);
-            gp.b = lb - gp.lloc * a.batch;
-          }
-          const int64_t row = stream_row(gp) + __ldcg(a.seq_off + gp.b) +
-                              (int64_t)(u - skip * tiles) * kTile;
-          if (row >= 0 && row < rows_total)
-            tma_prefetch_2d(x < P::kBoxes ? &tmK : &tmV, x % P::kBoxes * P::kBoxCols, (int)row);
+        const int u = quick_div(len * rank, ctas), end = quick_div(len * (rank + 1), ctas);
+        const int skip = quick_div(u, tiles);
+        if (skip > 0) {
+          const int gi = gi0 + skip, lb = quick_div(gi, a.H_kv);
+          guess.kvh = gi - lb * a.H_kv;
+          guess.lloc = quick_div(lb, a.batch);
+          guess.b = lb - guess.lloc * a.batch;
         }
+        const int off0 = __shfl_sync(0xffffffffu, early_off[0], guess.b >> 1);
+        const int off1 = __shfl_sync(0xffffffffu, early_off[1], guess.b >> 1);
+        guess_off = guess.b & 1 ? off1 : off0;
+        const int64_t row = (int64_t)stream_row(guess) + guess_off +
+                            (int64_t)(u - skip * tiles) * kTile;
+        int ahead = 0;
+        if (row >= 0 && row < rows_total) {
+          guess_row = (int)row;
+          ahead = min(min(end, (skip + 1) * tiles) - u, Cl::kStages);
+          if (end - u <= Cl::kStages) guess_tiles = ahead;
+        }
+        // box and tile of this lane
+        const int x = lane % (2 * P::kBoxes), i = lane / (2 * P::kBoxes);
+        if (i < ahead)
+          tma_prefetch_2d(x < P::kBoxes ? &tmK : &tmV, x % P::kBoxes * P::kBoxCols,
+                          guess_row + i * kTile);
       }
       __syncwarp();
     }
+    auto head_first = [&](const TileGroup &g) {
+      return ((int64_t)g.lloc * a.batch + g.b) * a.H_q + (int64_t)g.kvh * G;
+    };
+    const int64_t guess_head0 = head_first(guess);
+    auto copy_tile = [&](int st, int row, uint64_t policy) {
+      unsigned char *stage = smem + (size_t)st * Cl::kStageBytes;
+      mbar_arrive_expect_tx(&full_bar[st], Cl::kStageBytes);
+#pragma unroll
+      for (int h = 0; h < P::kBoxes; ++h) {
+        tma_load_2d(stage + h * Cl::kBoxBytes, &tmK, h * P::kBoxCols, row, &full_bar[st], policy);
+        tma_load_2d(stage + (P::kBoxes + h) * Cl::kBoxBytes, &tmV, h * P::kBoxCols, row,
+                    &full_bar[st], policy);
+      }
+    };
+    auto copy_q = [&](int qb, int64_t head0) {
+      mbar_arrive_expect_tx(&q_full[qb], Cl::kQBytes);
+      bulk_load(qbuf + qb * Cl::kQBytes, (const unsigned char *)a.q + head0 * D * Cl::kSize,
+                Cl::kQBytes, &q_full[qb]);
+    };
+    // K/V are streamed once; a call that fits beside the rest of the step stays in L2
+    auto tile_policy = [&](int total) {
+      return total * a.H_kv * a.n_layers <= kL2KeepBytes / Cl::kTileBytes ? evict_normal
+                                                                           : evict_first;
+    };
+    const uint64_t guess_policy = tile_policy(guess_t[0] * a.batch);
     pdl_enter();
-    // lengths and the tiles before each sequence, two sequences a lane
+    // lengths and the tiles before each sequence, two sequences a lane (requested before the early
+    // copies are issued, first used after)
     int n[2], t[2], any_empty = 0;
+    int64_t off[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const int b = 2 * lane + k;
       n[k] = b < a.batch ? a.len[b] : -1;
-      if (b < a.batch) s_off[b] = (int)a.seq_off[b];
+      off[k] = b < a.batch ? a.seq_off[b] : 0;
     }
-    const int bad = __shfl_sync(0xffffffffu, lane == 0 ? (int)status_bad(a.status) : 0, 0);
+    const int32_t status = lane == 0 && a.status ? *(volatile const int32_t *)a.status : 0;
+    if (lane == 0 && guess_tiles > 0) {
+      for (int i = 0; i < guess_tiles; ++i) copy_tile(i, guess_row + i * kTile, guess_policy);
+      copy_q(0, guess_head0);
+    }
+    __syncwarp();
+    const int bad = __shfl_sync(0xffffffffu, status, 0);
+    bool hit = guess_tiles > 0 && !bad;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
+      if (2 * lane + k < a.batch) s_off[2 * lane + k] = (int)off[k];
+      hit = hit && (int)off[k] == early_off[k];
       if (n[k] > a.max_len) {
         set_status(a.status, LG_ERR_CAPACITY);
         n[k] = -1;
+        hit = false;
       }
       any_empty |= n[k] == 0;
       n[k] = max(n[k], 0);
       t[k] = (n[k] + kTile - 1) / kTile;
+      hit = hit && (2 * lane + k >= a.batch || t[k] == guess_t[k]);
     }
+    hit = __all_sync(0xffffffffu, hit);
     const int t_first = __shfl_sync(0xffffffffu, t[0], 0);
     const bool same = (2 * lane >= a.batch || t[0] == t_first) &&
                       (2 * lane + 1 >= a.batch || t[1] == t_first);
@@ -389,53 +447,43 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
       s_c0 = c0;
       s_c1 = c1;
       s_empty = any_empty && !bad;
+      s_skip = hit ? 0 : guess_tiles;
     }
     __syncwarp();
     named_arrive<Cl::kThreads>(1);
     if (lane == 0 && u0 < u1) {
-      // K/V are streamed once; a call that fits beside the rest of the step stays in L2
-      const uint64_t policy = ts.total * a.H_kv * a.n_layers <= kL2KeepBytes / Cl::kTileBytes
-                                  ? evict_normal
-                                  : evict_first;
-      uint32_t it = 0, seg = 0;
+      const uint64_t policy = tile_policy(ts.total);
       auto timed_out = [&](uint64_t *bar, uint32_t parity) {
         if (mbar_wait(bar, parity)) return false;
         set_status(a.status, LG_ERR_TIMEOUT);
         return true;
       };
-      bool ok = true;
-      for (int t = u0; t < u1 && ok; ++seg) {
+      // stages used so far, segments begun so far (a dropped guess counts as one)
+      uint32_t it = guess_tiles, seg = guess_tiles > 0 && !hit;
+      bool ok = true, begun = hit;
+      for (int t = hit ? u0 + guess_tiles : u0; t < u1 && ok; ++seg) {
         const int end = min(g.start + g.tiles, u1);
         if (seg > 0 || g.kvh != first_kvh || g.lloc != first_lloc) row0 = stream_row(g);
         const int row = row0 + s_off[g.b] - g.start * kTile;
-        for (bool first = true; t < end; ++t, ++it, first = false) {
+        for (; t < end; ++t, ++it) {
           const int st = it % Cl::kStages;
           if (it >= (uint32_t)Cl::kStages &&
               timed_out(&empty_bar[st], ((it / Cl::kStages) - 1) & 1)) {
             ok = false;
             break;
           }
-          unsigned char *stage = smem + (size_t)st * Cl::kStageBytes;
-          mbar_arrive_expect_tx(&full_bar[st], Cl::kStageBytes);
-#pragma unroll
-          for (int h = 0; h < P::kBoxes; ++h) {
-            tma_load_2d(stage + h * Cl::kBoxBytes, &tmK, h * P::kBoxCols, row + t * kTile,
-                        &full_bar[st], policy);
-            tma_load_2d(stage + (P::kBoxes + h) * Cl::kBoxBytes, &tmV, h * P::kBoxCols,
-                        row + t * kTile, &full_bar[st], policy);
-          }
-          if (first) {
-            const int64_t head0 = ((int64_t)g.lloc * a.batch + g.b) * a.H_q + (int64_t)g.kvh * G;
+          copy_tile(st, row + t * kTile, policy);
+          if (!begun) {
             const int qb = seg & 1;
             if (seg >= 2 && timed_out(&q_empty[qb], ((seg >> 1) - 1) & 1)) {
               ok = false;
               break;
             }
-            mbar_arrive_expect_tx(&q_full[qb], Cl::kQBytes);
-            bulk_load(qbuf + qb * Cl::kQBytes, (const unsigned char *)a.q + head0 * D * Cl::kSize,
-                      Cl::kQBytes, &q_full[qb]);
+            copy_q(qb, head_first(g));
+            begun = true;
           }
         }
+        begun = false;
         if (ok && t < u1) ts.next(g);
       }
     }
@@ -511,6 +559,16 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     }
     return ok;
   };
+  if (s_skip > 0) {
+    // a dropped guess: its stages and queries pass unused
+    landed(&q_full[0], 0);
+    for (; it < (uint32_t)s_skip; ++it) {
+      landed(&full_bar[it], 0);
+      if (lane == 0) mbar_arrive(&empty_bar[it]);
+    }
+    if (lane == 0) mbar_arrive(&q_empty[0]);
+    seg = 1;
+  }
   for (int t = u0; t < u1; ++seg) {
     const int start = t, end = min(g.start + g.tiles, u1);
     const int n = s_len[g.b];

@@ -111,3 +111,48 @@ def test_cluster_pass(cuda, lens, H_kv, G, d, nl, dtype, h2o):
         # every non-empty sequence adds G to its kv-head's scores
         total, all_ = sc.double().sum(-1), float(G * sum(n > 0 for n in lens))
         assert torch.allclose(total, torch.full_like(total, all_), rtol=1e-5)
+
+
+@pytest.mark.parametrize("dtype,n0,b,H_kv,G,nl", [
+    ("bf16", 126, 1, 8, 2, 1), ("bf16", 254, 3, 2, 4, 2), ("bf16", 1022, 1, 8, 2, 1),
+    ("f32", 62, 2, 8, 2, 1), ("f32", 127, 1, 2, 8, 1), ("f32", 190, 1, 4, 3, 2)])
+def test_lengths_that_move_beside_the_call(cuda, dtype, n0, b, H_kv, G, nl):
+    """The pass looks at the lengths before its dependency wait and copies the tiles it then
+    expects; here lg_begin_step, still in flight beside it in a graph, moves the lengths past a
+    tile boundary, so that the expectation is dropped on one of the steps."""
+    steps, d = 5, 128
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    gen = torch.Generator(device=cuda)
+    gen.manual_seed(n0)
+    cap = n0 + steps + 1
+    k, v = (torch.randn((nl, H_kv, b * cap, d), generator=gen, device=cuda).to(tdt)
+            for _ in range(2))
+    q = torch.randn((nl, b, H_kv * G, d), generator=gen, device=cuda).to(tdt)
+    off = np.arange(b, dtype=np.int64) * cap
+    c = lg.Cache(nl, H_kv, d, dtype, off, [cap] * b, [n0] * b, cuda, k=k, v=v)
+    g = lg.Guard(c, H_kv * G, n_layers_per_call=nl)
+    out = torch.zeros((steps, nl, b, H_kv * G, d), dtype=tdt, device=cuda)
+    st = torch.zeros((steps, nl, b, H_kv * G, 4), device=cuda)
+
+    def run():
+        for s in range(steps):
+            lg.lg_begin_step(c)
+            lg.lg_decode_attend(c, 0, nl, q, H_kv * G, g.scale, out[s], st[s], 64, 0, cap, g.ws)
+
+    side = torch.cuda.Stream(device=cuda)
+    with torch.cuda.stream(side):
+        run()
+        side.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side, capture_error_mode="thread_local"):
+            run()
+        for _ in range(3):
+            out.zero_()
+            c.len.fill_(n0)
+            graph.replay()
+            side.synchronize()
+            assert lg.lg_read_device_status(c) == 0
+            for s in range(steps):
+                want, ws = _exact(k, v, q, [n0 + s + 1] * b, off, 0, nl, 64)
+                _close(out[s], want, *((2e-2, 1e-3) if dtype == "bf16" else (1e-4, 1e-5)), "out")
+                _close(st[s], ws, 1e-4, 1e-6, "stats")
