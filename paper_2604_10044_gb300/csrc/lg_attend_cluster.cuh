@@ -11,15 +11,17 @@
 // evenly over its CTAs, so every CTA streams one contiguous range of tiles through a ring of
 // tensor copies.  A group that lies within one CTA is finished there.  The (at most two) groups
 // a CTA shares with its neighbours are folded over its warps, and the folded pieces {M, l, u, sigma, o[32]} go straight into the
-// shared memory of the CTAs that own them (the sharing CTAs own a group's pieces in turn); after
-// one cluster barrier each owner merges what it received.  No counters, no workspace, no other
-// launch.  Uneven lengths cost little: a CTA with less to read leaves its bandwidth to the others
-// (one CTA streams up to 80 GB/s, 1.6 times its even share).
+// shared memory of the CTAs that own them (the sharing CTAs own a group's pieces in turn), each
+// store counting its bytes on the owner's barrier; the owner merges once all have arrived (a
+// cluster barrier in its place waits for the stores' acknowledgements first: 5.74 -> 5.58 us a layer at one
+// sequence of 1024 rows, 32 sequences of 128 9.70 -> 9.09).  No
+// counters, no workspace, no other launch.  Uneven lengths cost little: a CTA with less to read
+// leaves its bandwidth to the others (one CTA streams up to 90 GB/s, 1.8 times its even share).
 //
 // GB300, one layer of 28 (append and attention, called one by one in a graph), one sequence of
-// 1024 rows, 16/8 heads of 128: 12.0 -> 6.4 us.  Of a CTA's 4.4 us after its wait, 0.3 go to the
-// lengths, 0.5 to its range and first copy, 1.3 to that copy, 0.7 to the tile, 0.8 to the fold,
-// 0.4 to the barrier and 0.4 to the merge (clock64 at each phase).
+// 1024 rows, 16/8 heads of 128: 12.0 -> 5.6 us.  Of a CTA's 4.1 us after its wait, 1.6 go to its
+// first copies, 0.7 to the tile, 0.8 to the fold, 0.4 to the pieces' way and 0.4 to the merge
+// (clock64 at each phase).
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -109,13 +111,19 @@ __device__ __forceinline__ uint32_t peer_addr(const void *p, int rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
   return a;
 }
-__device__ __forceinline__ void peer_st(uint32_t addr, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+// (each counts its bytes on the barrier, which lies in the same CTA as the address)
+__device__ __forceinline__ void peer_st(uint32_t addr, float v, uint32_t bar) {
+  asm volatile(
+      "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(addr),
+      "f"(v), "r"(bar)
+      : "memory");
 }
-__device__ __forceinline__ void peer_st4(uint32_t addr, float4 v) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y),
-               "f"(v.z), "f"(v.w)
-               : "memory");
+__device__ __forceinline__ void peer_st4(uint32_t addr, float4 v, uint32_t bar) {
+  asm volatile(
+      "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, "
+      "[%5];" ::"r"(addr),
+      "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar)
+      : "memory");
 }
 
 template <int kThreads>
@@ -220,9 +228,10 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[Cl::kStages];
   __shared__ __align__(8) uint64_t empty_bar[Cl::kStages];
+  __shared__ __align__(8) uint64_t recv_bar[2];  // a slot's pieces have arrived
   __shared__ __align__(8) uint64_t q_full[2], q_empty[2];  // query rows of segment i in buffer i & 1
   __shared__ int s_len[kClusterSeqs], s_pre[kClusterSeqs], s_off[kClusterSeqs];
-  __shared__ int s_total, s_c0, s_c1, s_empty, s_skip;
+  __shared__ int s_total, s_c0, s_c1, s_empty, s_skip, s_bad;
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   unsigned char *qbuf = smem + Cl::kStages * Cl::kStageBytes;  // [2][G][D]
@@ -241,7 +250,6 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
         early_off[k] = (int)__ldcg(a.seq_off + 2 * lane + k);
       }
   }
-  cluster_arrive();  // waited for before the first store to a peer: every CTA has started then
   if (threadIdx.x == kWarps * 32) {
     for (int s = 0; s < Cl::kStages; ++s) {
       mbar_init(&full_bar[s], 1);
@@ -250,11 +258,15 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     for (int s = 0; s < 2; ++s) {
       mbar_init(&q_full[s], 1);
       mbar_init(&q_empty[s], kWarps);
+      mbar_init(&recv_bar[s], 1);
     }
     mbar_fence_init();
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmK)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
   }
+  __syncwarp();
+  // waited for before the first store to a peer: every CTA has started and set up its barriers
+  cluster_arrive();
   TileSpace ts;
   ts.len = s_len;
   ts.pre = s_pre;
@@ -405,10 +417,8 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
           s_len[2 * lane + k] = n[k];
           s_pre[2 * lane + k] = (2 * lane + k) * t_first;
         }
-      if (!bad) {
-        c0 = gi0 * t_first;
-        c1 = gi1 * t_first;
-      }
+      c0 = gi0 * t_first;
+      c1 = gi1 * t_first;
       u0 = c0 + quick_div((c1 - c0) * rank, ctas);
       u1 = c0 + quick_div((c1 - c0) * (rank + 1), ctas);
       g.tiles = t_first;
@@ -431,12 +441,10 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
       ts.total = __shfl_sync(0xffffffffu, upto, 31);
       __syncwarp();
       const int all = ts.total * a.H_kv * a.n_layers;
-      if (!bad) {
-        // this cluster's run of groups [c0, c1) (even lanes form its start, odd lanes its end)
-        const int x = run_bound(ts, all, cluster + (lane & 1), n_cl);
-        c0 = __shfl_sync(0xffffffffu, x, 0);
-        c1 = __shfl_sync(0xffffffffu, x, 1);
-      }
+      // this cluster's run of groups [c0, c1) (even lanes form its start, odd lanes its end)
+      const int x = run_bound(ts, all, cluster + (lane & 1), n_cl);
+      c0 = __shfl_sync(0xffffffffu, x, 0);
+      c1 = __shfl_sync(0xffffffffu, x, 1);
       u0 = c0 + quick_div((c1 - c0) * rank, ctas);
       u1 = c0 + quick_div((c1 - c0) * (rank + 1), ctas);
       if (u0 < u1) g = ts.find(u0);
@@ -448,10 +456,11 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
       s_c1 = c1;
       s_empty = any_empty && !bad;
       s_skip = hit ? 0 : guess_tiles;
+      s_bad = bad;
     }
     __syncwarp();
     named_arrive<Cl::kThreads>(1);
-    if (lane == 0 && u0 < u1) {
+    if (lane == 0 && u0 < u1 && !bad) {
       const uint64_t policy = tile_policy(ts.total);
       auto timed_out = [&](uint64_t *bar, uint32_t parity) {
         if (mbar_wait(bar, parity)) return false;
@@ -489,8 +498,6 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     }
     __syncwarp();
     cluster_wait();
-    cluster_arrive();
-    cluster_wait();
     return;
   }
 
@@ -519,13 +526,19 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     s.np = __popc(mask);
     return s;
   };
+  struct UnitAddr {
+    uint32_t data, bar;
+  };
   // where this CTA's partial of a group's unit goes: the owner, sharer number un % np, and its
   // slot of this group
   auto unit_addr = [&](const Sharers &sh, const TileGroup &g, int un) {
     const int j = quick_div(un, sh.np);
     const int owner = __ffs(__ballot_sync(0xffffffffu, sh.nth == un - j * sh.np)) - 1;
     const int slot = __shfl_sync(0xffffffffu, sh.lo, owner) >= g.start ? 0 : 1;
-    return peer_addr(recv + slot * Cl::kRecvFloats + (j * sh.np + sh.mine) * Cl::kUnit, owner);
+    UnitAddr u;
+    u.data = peer_addr(recv + slot * Cl::kRecvFloats + (j * sh.np + sh.mine) * Cl::kUnit, owner);
+    u.bar = peer_addr(&recv_bar[slot], owner);
+    return u;
   };
   const int u0 = first_tile(rank), u1 = first_tile(rank + 1);
   TileGroup g = {};
@@ -551,7 +564,10 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
   Slot slot0 = {}, slot1 = {};
   P pass;
   uint32_t it = 0, seg = 0;
-  bool ok = true;  // false once a copy did not land in time (the barriers below stay matched)
+  // With the status set nothing is read or written, but a CTA still passes its (meaningless)
+  // pieces on: the status may have been set by another CTA of this launch, and its peers wait.
+  const bool bad = s_bad;
+  bool ok = !bad;  // also false once a copy did not land in time
   auto landed = [&](uint64_t *bar, uint32_t parity) {
     if (ok && !mbar_wait(bar, parity)) {
       set_status(a.status, LG_ERR_TIMEOUT);
@@ -561,10 +577,14 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
   };
   if (s_skip > 0) {
     // a dropped guess: its stages and queries pass unused
-    landed(&q_full[0], 0);
+    bool in = mbar_wait(&q_full[0], 0);
     for (; it < (uint32_t)s_skip; ++it) {
-      landed(&full_bar[it], 0);
+      in = mbar_wait(&full_bar[it], 0) && in;
       if (lane == 0) mbar_arrive(&empty_bar[it]);
+    }
+    if (!in) {
+      set_status(a.status, LG_ERR_TIMEOUT);
+      ok = false;
     }
     if (lane == 0) mbar_arrive(&q_empty[0]);
     seg = 1;
@@ -580,9 +600,13 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     const bool whole = start == g.start && end == g.start + g.tiles;
     const int64_t head0 = ((int64_t)g.lloc * a.batch + g.b) * a.H_q + (int64_t)g.kvh * G;
     Sharers sh = {};
-    uint32_t dst0 = 0;
+    UnitAddr dst0 = {};
     if (!whole) {
       sh = sharers(g);
+      if (threadIdx.x == 0)  // the pieces of its units: np times (32 + 4) floats each
+        mbar_arrive_expect_tx(&recv_bar[start == u0 ? 0 : 1],
+                              quick_div(Cl::kUnits - sh.mine + sh.np - 1, sh.np) * sh.np *
+                                  Cl::kUnit * (int)sizeof(float));
       dst0 = unit_addr(sh, g, warp / G * Cl::kTaskUnits * G + warp % G);
     }
     if (landed(&q_full[qb], (seg >> 1) & 1)) pass.begin(qbuf + qb * Cl::kQBytes, a.qscale, lane);
@@ -630,25 +654,24 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
 #pragma unroll
         for (int w = 0; w < kWarps; ++w) o += f[w] * part[(w * G + h) * kRow + e];
         if (whole) {
-          finish<T, D>(a, head0 + h, e, slice == 0 && lane == 0, M, l, u, sg, o);
+          if (!bad) finish<T, D>(a, head0 + h, e, slice == 0 && lane == 0, M, l, u, sg, o);
         } else {
-          const uint32_t dst = k == 0 && task == warp ? dst0 : unit_addr(sh, g, un);
-          peer_st(dst + lane * 4, o);
-          if (lane == 0) peer_st4(dst + 32 * 4, make_float4(M, l, u, sg));
+          const UnitAddr dst = k == 0 && task == warp ? dst0 : unit_addr(sh, g, un);
+          peer_st(dst.data + lane * 4, o, dst.bar);
+          if (lane == 0) peer_st4(dst.data + 32 * 4, make_float4(M, l, u, sg), dst.bar);
         }
       }
     }
     if (!whole) (start == u0 ? slot0 : slot1) = Slot{sh.mine, sh.np, head0};
     if (t < u1) ts.next(g);
   }
-  __syncwarp();
-  cluster_arrive();
-  cluster_wait();  // every partial has arrived
 #pragma unroll 1
   for (int slot = 0; slot < 2; ++slot) {
     const int mine = slot ? slot1.mine : slot0.mine, np = slot ? slot1.np : slot0.np;
     const int64_t head0 = slot ? slot1.head0 : slot0.head0;
     if (np == 0) continue;
+    if (!mbar_wait_cluster(&recv_bar[slot], 0)) set_status(a.status, LG_ERR_TIMEOUT);
+    if (bad) continue;
 #pragma unroll 1
     for (int j = warp; j * np + mine < Cl::kUnits; j += kWarps) {
       const int un = j * np + mine;
