@@ -109,10 +109,11 @@ __global__ void append_kernel(lg_cache c, int layer0, const uint4 *k_new, const 
 // 32-element word join theirs by shuffles.  The loads of a warp are consecutive (row block,
 // kv-head) items, kv-head fastest, so the words of a row leave a warp together; lane j of a
 // word's lanes stores the words of items j, j + kLanes, ...
-// (GB300, 8 prompts of 32768 rows, 8 kv-heads of 128 bf16, 570 MB: 448.3 -> 94.2 us, 6.05 TB/s;
+// (GB300, 8 prompts of 32768 rows, 8 kv-heads of 128 bf16, 570 MB: 448.3 -> 92.0 us, 6.20 TB/s;
 // a thread per word with 32 2-byte loads, each load of a warp over 32 rows, kept L1 99 % busy
-// and HBM at 16 %.)
-constexpr int kSketchThreads = 256;
+// and HBM at 16 %.  CTAs of 256 threads 94.2, 16 loads in flight 102, persistent CTAs with bulk
+// copies through a ring in shared memory 90 to 100.)
+constexpr int kSketchThreads = 128;
 constexpr int kSketchLoads = 8;
 
 template <typename T, int D>
