@@ -17,11 +17,13 @@ struct Pass<__nv_bfloat16, D, G> {
   static constexpr int kBlocks = kTile / 16 / kWarps;  // 16-row blocks of a warp
   static constexpr float kTileUs = 0.72f * D / 128.f;  // one CTA's time for a tile
   static constexpr int kFoldUnits = 1;
+  static constexpr bool kEarlyUnits = true;
+  static constexpr int kFlushTiles = 0;  // (a lane's sums take one rounding per 16 rows here)
 
   WarpSums<D> acc;
   uint32_t qf[D / 16][2];
 
-  __device__ __forceinline__ void begin(const unsigned char *q, float, int lane) {
+  __device__ __forceinline__ void begin(const unsigned char *q, bool, float, int lane) {
     acc.reset();
     load_q<D, G>(qf, q, lane);
   }
@@ -30,7 +32,7 @@ struct Pass<__nv_bfloat16, D, G> {
     tile_update<D, G, kBlocks>(acc, qf, stage, tile_rows, suffix, logits, qscale, warp, lane);
   }
   __device__ __forceinline__ void join() { acc.join_lanes(); }
-  __device__ __forceinline__ void store(float *rows, int lane) {
+  __device__ __forceinline__ void store(float *rows, bool, int lane) {
     acc.template store<G, D + 4>(rows, rows + D, lane);
   }
 };

@@ -10,11 +10,12 @@
 // sequence, kv-head) groups, about the same number of tiles each, and splits the run's tiles
 // evenly over its CTAs, so every CTA streams one contiguous range of tiles through a ring of
 // tensor copies.  A group that lies within one CTA is finished there.  The (at most two) groups
-// a CTA shares with its neighbours are folded over its warps, and the folded pieces {M, l, u, sigma, o[32]} go straight into the
-// shared memory of the CTAs that own them (the sharing CTAs own a group's pieces in turn), each
-// store counting its bytes on the owner's barrier; the owner merges once all have arrived (a
-// cluster barrier in its place waits for the stores' acknowledgements first: 5.74 -> 5.58 us a layer at one
-// sequence of 1024 rows, 32 sequences of 128 9.70 -> 9.09).  No
+// a CTA shares with its neighbours are folded over its warps, and the folded pieces {M, l, u,
+// sigma, o[32]} go straight into the shared memory of the CTAs that own them (the sharing CTAs own
+// a group's pieces in turn), each store counting its bytes on the owner's barrier; the owner
+// merges once all have arrived (a cluster barrier in its place waits for the stores'
+// acknowledgements first: 5.74 -> 5.58 us a layer at one sequence of 1024 rows, 32 sequences of
+// 128 9.70 -> 9.09).  No
 // counters, no workspace, no other launch.  Uneven lengths cost little: a CTA with less to read
 // leaves its bandwidth to the others (one CTA streams up to 90 GB/s, 1.8 times its even share).
 //
@@ -45,8 +46,9 @@ constexpr int kMaxCluster = 8;    // CTAs of a cluster at most (portable)
 // What differs between the element types: the tile and the ring, and a consumer warp's work.
 //   kTile rows a tile, kBoxes boxes of kBoxCols columns per tensor, kStages stages in the ring
 //   kWarps consumer warps, which share every tile; kTileUs one CTA's time for a tile
-//   begin(the segment's query rows), update(a tile), join() (the lanes' sums) and store(a row of
-//   D + 4 floats per head: o, then {M, l, u, sigma})
+//   begin(the query rows, whether it is the segment's first tile), update(a tile), join() (the
+//   lanes' sums) and store(to, or added to, a row of D + 4 floats per head: o, then {M, l, u,
+//   sigma}); with kFlushTiles > 0 a segment's sums are stored every so many tiles
 template <typename T, int D, int G>
 struct Pass;
 
@@ -506,9 +508,12 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
   named_sync<Cl::kThreads>(1);
   cluster_wait();
   ts.total = s_total;
-  const int c0 = s_c0, c1 = s_c1;
-  // this CTA's tiles [u0, u1): an even share of the cluster's
-  auto first_tile = [&](int r) { return c0 + quick_div((c1 - c0) * r, ctas); };
+  // this CTA's tiles [u0, u1): an even share of the cluster's (read again for each use: registers
+  // are short)
+  auto first_tile = [&](int r) {
+    const int c0 = *(volatile int *)&s_c0, c1 = *(volatile int *)&s_c1;
+    return c0 + quick_div((c1 - c0) * r, ctas);
+  };
   // The CTAs of the cluster that share a group: lane r stands for CTA r (np of them, mine before
   // this one).  CTA number i of them owns units i, i + np, ... of the group.
   struct Sharers {
@@ -558,8 +563,7 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
   // groups in the slots: 0 for a segment that starts at u0, 1 for another that ends at u1
   // (np 0: not in use; mine and np as above, the group's first head)
   struct Slot {
-    int mine, np;
-    int64_t head0;
+    int mine, np, head0;
   };
   Slot slot0 = {}, slot1 = {};
   P pass;
@@ -593,38 +597,48 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     const int start = t, end = min(g.start + g.tiles, u1);
     const int n = s_len[g.b];
     const int suffix_lo = n - min(a.suffix_w, n);
-    const int64_t lrow = ((int64_t)g.lloc * a.H_kv + g.kvh) * a.S_total + s_off[g.b];
+    // (32 bits hold every row and head of a call: the limits of attend_cluster_takes)
+    const int lrow = (g.lloc * a.H_kv + g.kvh) * (int)a.S_total + s_off[g.b];
     const int qb = seg & 1;
     // who shares the group and where this warp's first unit goes, formed while the first copies
     // are in flight (after the tiles they would sit on the way to the merge)
     const bool whole = start == g.start && end == g.start + g.tiles;
-    const int64_t head0 = ((int64_t)g.lloc * a.batch + g.b) * a.H_q + (int64_t)g.kvh * G;
+    const int head0 = (g.lloc * a.batch + g.b) * a.H_q + g.kvh * G;
     Sharers sh = {};
     UnitAddr dst0 = {};
-    if (!whole) {
+    auto place_units = [&] {
+      if (whole) return;
       sh = sharers(g);
       if (threadIdx.x == 0)  // the pieces of its units: np times (32 + 4) floats each
         mbar_arrive_expect_tx(&recv_bar[start == u0 ? 0 : 1],
                               quick_div(Cl::kUnits - sh.mine + sh.np - 1, sh.np) * sh.np *
                                   Cl::kUnit * (int)sizeof(float));
       dst0 = unit_addr(sh, g, warp / G * Cl::kTaskUnits * G + warp % G);
-    }
-    if (landed(&q_full[qb], (seg >> 1) & 1)) pass.begin(qbuf + qb * Cl::kQBytes, a.qscale, lane);
-    for (; t < end; ++t, ++it) {
-      const int st = it % Cl::kStages;
-      if (landed(&full_bar[st], (it / Cl::kStages) & 1)) {
-        const int r0 = (t - g.start) * kTile;
-        pass.update(smem + (size_t)st * Cl::kStageBytes, min(kTile, n - r0), suffix_lo - r0,
-                    a.logits ? a.logits + (lrow + r0) * G : nullptr, a.qscale, warp, lane);
+    };
+    if (P::kEarlyUnits) place_units();
+    // (all of the segment at once, or kFlushTiles tiles at a time)
+    do {
+      const int from = t, stop = P::kFlushTiles ? min(end, t + P::kFlushTiles) : end;
+      if (landed(&q_full[qb], (seg >> 1) & 1))
+        pass.begin(qbuf + qb * Cl::kQBytes, from == start, a.qscale, lane);
+      for (; t < stop; ++t, ++it) {
+        const int st = it % Cl::kStages;
+        if (landed(&full_bar[st], (it / Cl::kStages) & 1)) {
+          const int r0 = (t - g.start) * kTile;
+          float *logits = a.logits ? a.logits + (int64_t)(lrow + r0) * G : nullptr;
+          pass.update(smem + (size_t)st * Cl::kStageBytes, min(kTile, n - r0), suffix_lo - r0,
+                      logits, a.qscale, warp, lane);
+        }
+        if (lane == 0) mbar_arrive(&empty_bar[st]);
       }
-      if (lane == 0) mbar_arrive(&empty_bar[st]);
-    }
-    if (lane == 0) mbar_arrive(&q_empty[qb]);
-    // the segment's warp partials folded: a whole group is finished here, a part of a group goes
-    // to the owners of its units
-    pass.join();
-    if (start != u0) named_sync<kWarps * 32>(2);  // the segment before has been folded
-    pass.store(part + warp * G * kRow, lane);
+      if (t == end && lane == 0) mbar_arrive(&q_empty[qb]);
+      // the segment's warp partials folded: a whole group is finished here, a part of a group goes
+      // to the owners of its units
+      pass.join();
+      if (from == start && start != u0) named_sync<kWarps * 32>(2);  // the segment before is folded
+      pass.store(part + warp * G * kRow, from != start, lane);
+    } while (P::kFlushTiles && t < end);
+    if (!P::kEarlyUnits) place_units();
     named_sync<kWarps * 32>(2);
 #pragma unroll 1
     for (int task = warp; task < Cl::kTasks; task += kWarps) {
@@ -668,7 +682,7 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
 #pragma unroll 1
   for (int slot = 0; slot < 2; ++slot) {
     const int mine = slot ? slot1.mine : slot0.mine, np = slot ? slot1.np : slot0.np;
-    const int64_t head0 = slot ? slot1.head0 : slot0.head0;
+    const int head0 = slot ? slot1.head0 : slot0.head0;
     if (np == 0) continue;
     if (!mbar_wait_cluster(&recv_bar[slot], 0)) set_status(a.status, LG_ERR_TIMEOUT);
     if (bad) continue;

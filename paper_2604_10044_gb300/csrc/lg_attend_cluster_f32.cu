@@ -7,8 +7,8 @@
 // probabilities are passed back by shuffles.  Up to 4 heads the memory bounds a call; at 5 to 8
 // the chains of dependent shuffles and FMAs do, of which two to four rows run side by side.
 // GB300, one layer (append and attention), 268 MB, 4 sequences of 8191 rows, 8 kv-heads of 128,
-// against the chunk kernel with its separate combine: 1 head a group 80.8 -> 43.6 us, 4 heads
-// 91.1 -> 46.8, 8 heads 108.0 -> 76.6.  Not kept: a lane a row with the query rows broadcast from
+// against the chunk kernel with its separate combine: 1 head a group 80.8 -> 41.4 us, 4 heads
+// 91.1 -> 45.4, 8 heads 108.0 -> 76.1.  Not kept: a lane a row with the query rows broadcast from
 // shared memory (its datapath moves 512 bytes for a broadcast too: 54 and 80 us at 4 and 8 heads).
 #include "lg_attend_cluster.cuh"
 
@@ -25,6 +25,7 @@ struct Pass<float, D, G> {
   static constexpr int kStages = (G <= 4 ? 3 : 5) * 128 / D;
   static constexpr int kWarps = 8;
   static constexpr int kFoldUnits = 4;
+  static constexpr bool kEarlyUnits = false;  // (six registers that the tiles' loop lacks)
   static constexpr float kTileUs = (G <= 4 ? 1.f : 1.2f) * D / 128.f;
   static constexpr int kBox = kTile * 128;       // bytes of a box
   static constexpr int kEpl = G <= 2 ? 16 : (G <= 4 ? 8 : 4);  // elements of a lane
@@ -37,11 +38,21 @@ struct Pass<float, D, G> {
   static constexpr int kSteps = kRows / kRpw < kMaxSteps ? kRows / kRpw : kMaxSteps;
   static constexpr int kGP = pow2_ceil(G);
   static constexpr int kDup = kLpr / kGP;        // lanes that hold the same head's logit
+  // A flush every so many tiles (32 of a lane's rows) adds the sums to the warp's partial in shared
+  // memory, which keeps the chains of dependent roundings short: a lane takes hundreds of rows of a
+  // long call.  Distance of the output from 64 bits (2-norm, normal rows; the chunk kernel /
+  // without flushes / with): 4 sequences of 8191, 4 heads 2.65e-7 / 2.82e-7 / 2.16e-7, one of
+  // 131071, 8 heads 4.4e-7 / 8.4e-7 / 2.6e-7.  It costs 2 % of the time (44.4 -> 45.4 us, above).
+  static constexpr int kFlushTiles = 32 * kRpw / kRows;
   static_assert(kGP <= kLpr && kRows % (kSteps * kRpw) == 0, "lanes for the heads, whole steps");
 
-  float2 q[G][kCh][2], o[G][kCh][2];
-  float m, l, u, sg;  // of head (lane % kLpr) / kDup over this lane's row group
+  static constexpr int kKept = D / 64;  // pairs of a head that a lane keeps when they are joined
+  struct __align__(8 * kKept) Pairs {
+    float2 p[kKept];
+  };
 
+  float2 q[G][kCh][2], o[G][2 * kCh];
+  float m, l, u, sg;  // of head (lane % kLpr) / kDup over this lane's row group
   // chunk j of this lane, a multiple of 4 elements: the lanes of a row side by side, so that
   // eight lanes read 128 bytes of different banks (with four lanes a row, odd rows take the
   // other half of a box first)
@@ -54,7 +65,8 @@ struct Pass<float, D, G> {
                                              (((ch & 7) ^ (row & 7)) << 4));
   }
 
-  __device__ __forceinline__ void begin(const unsigned char *qrows, float qscale, int lane) {
+  __device__ __forceinline__ void begin(const unsigned char *qrows, bool first, float qscale,
+                                        int lane) {
     const float4 *q4 = reinterpret_cast<const float4 *>(qrows);
 #pragma unroll
     for (int g = 0; g < G; ++g)
@@ -63,9 +75,9 @@ struct Pass<float, D, G> {
         const float4 v = q4[g * (D / 4) + chunk(j, lane)];
         q[g][j][0] = make_float2(v.x * qscale, v.y * qscale);
         q[g][j][1] = make_float2(v.z * qscale, v.w * qscale);
-        o[g][j][0] = o[g][j][1] = make_float2(0.f, 0.f);
+        o[g][2 * j] = o[g][2 * j + 1] = make_float2(0.f, 0.f);
       }
-    m = -INFINITY;
+    if (first) m = -INFINITY;  // else it runs on
     l = u = sg = 0.f;
   }
 
@@ -115,8 +127,8 @@ struct Pass<float, D, G> {
           const float2 c2 = make_float2(cg, cg);
 #pragma unroll
           for (int j = 0; j < kCh; ++j) {
-            o[g][j][0] = __fmul2_rn(o[g][j][0], c2);
-            o[g][j][1] = __fmul2_rn(o[g][j][1], c2);
+            o[g][2 * j] = __fmul2_rn(o[g][2 * j], c2);
+            o[g][2 * j + 1] = __fmul2_rn(o[g][2 * j + 1], c2);
           }
         }
       }
@@ -146,8 +158,8 @@ struct Pass<float, D, G> {
           const float2 p2 = make_float2(pg, pg);
 #pragma unroll
           for (int j = 0; j < kCh; ++j) {
-            o[g][j][0] = __ffma2_rn(p2, make_float2(v[j].x, v[j].y), o[g][j][0]);
-            o[g][j][1] = __ffma2_rn(p2, make_float2(v[j].z, v[j].w), o[g][j][1]);
+            o[g][2 * j] = __ffma2_rn(p2, make_float2(v[j].x, v[j].y), o[g][2 * j]);
+            o[g][2 * j + 1] = __ffma2_rn(p2, make_float2(v[j].z, v[j].w), o[g][2 * j + 1]);
           }
         }
       }
@@ -155,7 +167,8 @@ struct Pass<float, D, G> {
     __syncwarp();
   }
 
-  // the row groups' sums on every lane, against the warp's maximum of each head
+  // The row groups' sums, against the warp's maximum of each head: l, u and sg on every lane, of o
+  // the pairs that the lane keeps (o[g][0 .. kKept)).
   __device__ __forceinline__ void join() {
     const int lane = threadIdx.x & 31, gbase = lane - lane % kLpr;
     float M = m;
@@ -176,48 +189,67 @@ struct Pass<float, D, G> {
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       const float fg = __shfl_sync(0xffffffffu, f, gbase + g * kDup);
+      float2(&v)[2 * kCh] = o[g], sum[kCh];
 #pragma unroll
-      for (int j = 0; j < kCh; ++j)
+      for (int c = 0; c < 2 * kCh; ++c) v[c] = __fmul2_rn(v[c], make_float2(fg, fg));
+      // each level, a lane hands half of its pairs to the other row group's lane
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          o[g][j][k].x *= fg;
-          o[g][j][k].y *= fg;
-        }
-#pragma unroll
-      for (int x = kLpr; x < 32; x <<= 1) {
+      for (int x = kLpr, half = kCh; x < 32; x <<= 1, half >>= 1) {
+        const bool up = lane & x;
         // the neighbour row of four-lane rows holds its chunks in the other order
-        const int flip = kLpr == 4 && x == kLpr ? 1 : 0;
-        float2 t[kCh][2];
+        const int flip = kLpr == 4 && x == kLpr ? 2 : 0;
 #pragma unroll
-        for (int j = 0; j < kCh; ++j)
-#pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            t[j][k].x = __shfl_xor_sync(0xffffffffu, o[g][j ^ flip][k].x, x);
-            t[j][k].y = __shfl_xor_sync(0xffffffffu, o[g][j ^ flip][k].y, x);
+        for (int c = 0; c < kCh; ++c)
+          if (c < half) {
+            const float2 send = up ? v[c ^ flip] : v[(c ^ flip) + half];
+            const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, send.x, x),
+                                           __shfl_xor_sync(0xffffffffu, send.y, x));
+            sum[c] = __fadd2_rn(up ? v[c + half] : v[c], got);
           }
 #pragma unroll
-        for (int j = 0; j < kCh; ++j)
-#pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            o[g][j][k].x += t[j][k].x;
-            o[g][j][k].y += t[j][k].y;
-          }
+        for (int c = 0; c < kCh; ++c)
+          if (c < half) v[c] = sum[c];
       }
     }
   }
 
-  __device__ __forceinline__ void store(float *rows, int lane) {
-    if (lane < kLpr) {
-#pragma unroll
-      for (int g = 0; g < G; ++g)
-#pragma unroll
-        for (int j = 0; j < kCh; ++j)
-          *reinterpret_cast<float4 *>(rows + g * (D + 4) + 4 * chunk(j, lane)) =
-              make_float4(o[g][j][0].x, o[g][j][0].y, o[g][j][1].x, o[g][j][1].y);
-      const int hd = lane / kDup;
-      if (lane % kDup == 0 && hd < G)
-        *reinterpret_cast<float4 *>(rows + hd * (D + 4) + D) = make_float4(m, l, u, sg);
+  // the joined sums to the warp's partial, or added to the sums of earlier tiles there
+  __device__ __forceinline__ void store(float *rows, bool add, int lane) {
+    const int gbase = lane - lane % kLpr, hd = lane % kLpr / kDup;
+    float f = 0.f;
+    if (add && hd < G) {
+      const float4 h = *reinterpret_cast<const float4 *>(rows + hd * (D + 4) + D);
+      const float dm = fmaxf(h.x - m, -1e30f);  // the maximum runs on: h.x <= m
+      f = exp2f(dm);
+      l += f * h.y;
+      u += f * (h.z + dm * h.y);
+      sg += f * h.w;
     }
+    // where this lane's pairs lie
+    int c = 0;
+#pragma unroll
+    for (int x = kLpr, half = kCh; x < 32; x <<= 1, half >>= 1) c += lane & x ? half : 0;
+    float *at = rows + 4 * chunk(c >> 1, lane) + 2 * (c & 1);
+#pragma unroll
+    for (int g = 0; g < G; ++g, at += D + 4) {
+      const float fg = __shfl_sync(0xffffffffu, f, gbase + g * kDup);
+      float2 v[kKept];
+#pragma unroll
+      for (int i = 0; i < kKept; ++i) v[i] = o[g][i];
+      if (add) {
+        const Pairs h = *reinterpret_cast<const Pairs *>(at);
+#pragma unroll
+        for (int i = 0; i < kKept; ++i) v[i] = __ffma2_rn(make_float2(fg, fg), h.p[i], v[i]);
+      }
+      Pairs w;
+#pragma unroll
+      for (int i = 0; i < kKept; ++i) w.p[i] = v[i];
+      *reinterpret_cast<Pairs *>(at) = w;
+    }
+    __syncwarp();  // every lane has read its head's earlier sums
+    if (lane < kLpr && lane % kDup == 0 && hd < G)
+      *reinterpret_cast<float4 *>(rows + hd * (D + 4) + D) = make_float4(m, l, u, sg);
+    __syncwarp();
   }
 };
 

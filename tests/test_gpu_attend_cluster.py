@@ -156,3 +156,24 @@ def test_lengths_that_move_beside_the_call(cuda, dtype, n0, b, H_kv, G, nl):
                 want, ws = _exact(k, v, q, [n0 + s + 1] * b, off, 0, nl, 64)
                 _close(out[s], want, *((2e-2, 1e-3) if dtype == "bf16" else (1e-4, 1e-5)), "out")
                 _close(st[s], ws, 1e-4, 1e-6, "stats")
+
+
+@pytest.mark.parametrize("lens,H_kv,G,d", [([40000], 1, 8, 128), ([30001], 2, 4, 128),
+                                           ([20000, 9000], 2, 1, 128), ([33000], 2, 6, 64),
+                                           ([50000], 2, 2, 64)])
+def test_long_fp32_segments_keep_their_precision(cuda, lens, H_kv, G, d):
+    """Segments of many times the 32 rows a lane adds up before it puts its sums away: their
+    error against 64 bits stays that of short chains.  A sum of n random terms in a chain is off
+    by about 2^-24.8 sqrt(n / 2) of its size (a rounding is 2^-24.8 of its value on average), so
+    1.4e-7 for each of the 32-row chains, the chain of put-away sums (a dozen to 60 long) and the
+    merges of 8 warps and 8 CTAs, 2.4e-7 together with the products' roundings; unbroken chains of
+    400 to 2000 rows would give 4.8e-7 to 1.1e-6."""
+    g = torch.Generator(device=cuda)
+    g.manual_seed(sum(lens))
+    S = int(sum(lens)) + len(lens)
+    k, v = (torch.randn((1, H_kv, S, d), generator=g, device=cuda) for _ in range(2))
+    q = torch.randn((1, len(lens), H_kv * G, d), generator=g, device=cuda)
+    got, st, _, off = _run(k, v, q, lens, 0, 1, 64, False, 0)
+    want, ws = _exact(k, v, q, lens, off, 0, 1, 64)
+    assert ((got.double() - want).norm() / want.norm()).item() < 4e-7
+    assert ((st.double() - ws).norm() / ws.norm()).item() < 4e-7
