@@ -2,16 +2,17 @@
 // (LoopGuard Sec. 3.1, Eq. 1; statistics read by Sec. 5.2), plus the H2O score accumulation
 // of the comparator policy (Sec. 2.2, Sec. 6.1), and the choice of a call's pass.
 //
-// The chunk kernel here serves fp32 caches past the cluster pass's limits (lg_attend_cluster.cuh:
-// more than 64 sequences, the longest calls).  One CTA streams CH consecutive rows of one (layer,
-// sequence, kv-head) and serves all g query heads of that kv-head, so every K/V byte is read from
-// HBM once per step.  A producer warp moves 8 KB K and V tiles into a 4-stage shared-memory ring
-// with 1-D bulk copies (TMA) completing on mbarriers; four consumer warps compute.  A row is split over LPR lanes
-// (16 B each): the lanes form partial dot products for all heads with packed fp32 FMAs, a
-// transposed butterfly leaves each lane with the full logit of one head, that lane runs the
-// online softmax for its head (in log2 units) and the probabilities are broadcast back for
-// the P.V update.  The CTA writes one partial {M, l, u, sigma, o[d]} per head; a second kernel
-// merges the partials of a head and emits out and the statistics {m, l, H, S}.
+// The chunk kernel here serves the fp32 calls that the cluster pass (lg_attend_cluster.cuh) does
+// not take: more than 64 sequences, the longest calls, and those that its rule finds faster here.
+// One CTA streams CH consecutive rows of one (layer, sequence, kv-head) and serves all g query
+// heads of that kv-head, so every K/V byte is read from HBM once per step.  A producer warp moves
+// 8 KB K and V tiles into a 4-stage shared-memory ring with 1-D bulk copies (TMA) completing on
+// mbarriers; four consumer warps compute.  A row is split over LPR lanes (16 B each): the lanes
+// form partial dot products for all heads with packed fp32 FMAs, a transposed butterfly leaves each
+// lane with the full logit of one head, that lane runs the online softmax for its head (in log2
+// units) and the probabilities are broadcast back for the P.V update.  The CTA writes one partial
+// {M, l, u, sigma, o[d]} per head; a second kernel merges the partials of a head and emits out and
+// the statistics {m, l, H, S}.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -391,16 +392,16 @@ template <typename T, int D, int G>
 static cudaError_t launch_typed(const AttendArgs &a, int64_t rows_total, void *out, float *stats,
                                 float *final_ml, float *h2o, cudaStream_t s) {
   using C = AttendCfg<T, D, G>;
-  cudaError_t e;
-  if (Elem<T>::kDtype == LG_BF16) {
-    // tensor-core passes (lg_attend_cluster.cu, lg_attend_mma.cu), which merge their partials
-    e = attend_cluster_takes(a, mma_tile_rows(), rows_total)
-            ? launch_attend_cluster(a, D, G, rows_total, s)
-            : launch_attend_mma_partial(a, D, G, rows_total, s);
-    if (e != cudaSuccess) return e;
-  } else if (attend_cluster_takes(a, cluster_f32_tile_rows(), rows_total)) {
-    LG_TRY(launch_attend_cluster_f32(a, D, G, rows_total, s));
-  } else {
+  cudaError_t e = cudaSuccess;
+  constexpr bool kBf16 = Elem<T>::kDtype == LG_BF16;
+  bool general =
+      !attend_cluster_takes(a, kBf16 ? mma_tile_rows() : cluster_f32_tile_rows(), rows_total);
+  if (!general)
+    LG_TRY((kBf16 ? launch_attend_cluster : launch_attend_cluster_f32)(a, D, G, rows_total,
+                                                                      &general, s));
+  if (general && kBf16) {
+    LG_TRY(launch_attend_mma_partial(a, D, G, rows_total, s));  // merges its partials
+  } else if (general) {
     auto kp = attend_partial_kernel<T, D, G>;
     e = cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
     if (e != cudaSuccess) return e;

@@ -43,9 +43,20 @@ namespace {
 constexpr int kClusterSeqs = 64;  // batch at most (two sequences a lane in the prologue's scan)
 constexpr int kMaxCluster = 8;    // CTAs of a cluster at most (portable)
 
+// a call as the choice of its pass sees it (cluster_shape below)
+struct CallShape {
+  int groups, tiles;          // (layer, sequence, kv-head) groups; tiles of a longest one
+  float tile_bytes, tile_us;  // a tile's bytes, one CTA's time for it
+  float seg_us;               // a segment's fold
+  // a CTA's last segments: where it has several tiles of a group, of which it shares some
+  float ends_us(int c) const { return tiles < 8 ? 0.f : seg_us * (c > 1 ? 2.f : 1.f); }
+  float mem_us(float n_tiles) const { return n_tiles * tile_bytes / 7.3e6f; }
+};
+
 // What differs between the element types: the tile and the ring, and a consumer warp's work.
 //   kTile rows a tile, kBoxes boxes of kBoxCols columns per tensor, kStages stages in the ring
-//   kWarps consumer warps, which share every tile; kTileUs one CTA's time for a tile
+//   kWarps consumer warps, which share every tile; kTileUs one CTA's time for a tile, kSegmentUs
+//   for a segment's fold; general_us(call, its shape, mean length): the general pass's time
 //   begin(the query rows, whether it is the segment's first tile), update(a tile), join() (the
 //   lanes' sums) and store(to, or added to, a row of D + 4 floats per head: o, then {M, l, u,
 //   sigma}); with kFlushTiles > 0 a segment's sums are stored every so many tiles
@@ -763,59 +774,94 @@ cudaError_t resident_clusters(int (&n)[kNumSizes]) {
   return cudaSuccess;
 }
 
-// Cluster size and count for `groups` groups of at most `tiles` tiles: the size whose estimated
-// time is least.  With K clusters, each takes groups / K groups and then groups mod K of them one
-// more; either phase is bound by the memory (kTilesPerUs tiles a microsecond over all CTAs) or by
-// the CTAs (kTileUs a tile, kSegmentUs a segment end).  Of a batch the host knows the longest
-// length it may have, not the others, so a ragged one (lengths kRagged of the longest on average,
-// as log-uniform ones are) counts as much: its clusters' runs are even but for half of a longest
-// group on one cluster.  Smaller clusters fill the GPU better
-// (152 SMs hold 15, 23, 36, 76, 152 clusters of 8, 6, 4, 2, 1), larger ones split a group further
-// and stream a little better (about a percent per halving on passes of half a millisecond).
-// Measured per call (append and attention, layers called one by one in a graph, us, sizes 8 / 6 /
-// 4 / 2 / 1; 8 kv-heads of 128): 1 sequence of 1024 rows 7.3 / 7.9 / 7.9 / 9.1 / 10.9; 8 of 4096
-// 30.2 / 26.6 / 26.8 / 26.6 / 29.4; 2 of 131071, 8 heads a group, 238 / 157 / 207 / 397 / 780; 16
-// of 32768, 8 heads a group, 309 / 302 / 303 / 302 / 296.
+// What a call is estimated to take (us), by cluster size and by the general pass.  Only max_len is
+// known of the lengths, and how many rows the cache has for them: `fill` = S_total / (batch *
+// max_len) at most 1.  A batch with fill above 0.9 may have equal lengths or any others, so it is
+// judged as equal ones and, half as much, as ragged ones of 0.35 of the longest on average (as
+// log-uniform ones are); below, as ragged ones of fill on average.
+constexpr float kRagged = 0.35f, kFull = 0.9f, kCallUs = 5.f;
+
+// K clusters of c CTAs.  Equal lengths: each takes groups / K groups and then groups mod K of them
+// one more; either phase is bound by the memory or by the CTAs.  Ragged ones: the clusters' runs
+// are even but for a part of a longest group on one cluster, and no group has more than c CTAs.
+// Larger clusters stream a little better (about a percent per halving on passes of half a
+// millisecond).
+inline float equal_us(const CallShape &s, int c, int k) {
+  const int q = s.groups / k, r = s.groups % k;
+  const float cta = (float)s.tiles / (float)c * s.tile_us;  // a group's tiles on one of its CTAs
+  float us = fmaxf(s.mem_us((float)k * (float)q * (float)s.tiles),
+                   (float)q * cta + s.seg_us * (float)(q - 1) / (float)c);
+  if (r) us += fmaxf(s.mem_us((float)r * (float)s.tiles), cta + s.seg_us / (float)c);
+  return us + s.ends_us(c);
+}
+inline float ragged_us(const CallShape &s, int c, int k, float mean) {
+  const float cta = (float)s.tiles / (float)c * s.tile_us;
+  const float total = mean * (float)s.groups * (float)s.tiles;
+  const float even = (total * s.tile_us + (float)s.groups * s.seg_us) / (float)(k * c);
+  return fmaxf(fmaxf(s.mem_us(total), even) + 0.35f * cta, cta) + s.ends_us(c);
+}
+
+// Cluster size and count, and whether the general pass (general(mean): its estimate for lengths of
+// that mean share of the longest) is expected to be faster: with few long groups, which have at
+// most 8 CTAs each here and the whole GPU there, and, of fp32 calls, with 5 to 8 heads a group,
+// bound by a CTA's arithmetic.  Smaller clusters fill the GPU better (152 SMs hold 15, 23, 36, 76,
+// 152 clusters of 8, 6, 4, 2, 1), larger ones split a group further.
+// Measured per call (append and attention, one layer, us, 128 elements; sizes 8 / 6 / 4 / 2 / 1,
+// general): bf16, equal lengths, 1 sequence of 131071 rows, 2 kv-heads, 1 head a group 74 / 97 /
+// 142 / 277 / 540, 45; the same with 8 heads 102 / 132 / 192 / 374 / 727, 136; 2 of 66791, 8 kv-heads
+// 107 / 80 / 91 / 150 / 284, 90; ragged, 8 up to 124643, 2 kv-heads 84 / 101 / 140 / 264 / 522, 73;
+// the same with 7 heads 103 / 132 / 189 / 367 / 717, 109; 48 up to 17000, 4 kv-heads 87 / 88 / 91 /
+// 99 / 106, 99.  fp32, 6 of 9036, 8 kv-heads, 4 heads 88 / 93 / 93 / 88 / 165, 109; the same with 8
+// heads 158 / 158 / 159 / 158 / 307, 134; ragged, 11 up to 88235, 2 kv-heads, 1 head 134 / 158 / 211
+// / 394 / 773, 173; the same with 7 heads 380 / 505 / 751 / 1488 / 2965, 232.  Over 130 such calls
+// the choice is 2 % off the best one's time on average; over 240 random ones none is slower than
+// the general pass.
 struct ClusterShape {
   int ctas, clusters;
+  bool general;
 };
-inline ClusterShape cluster_shape(int groups, int batch, int tiles, int tile_bytes, float kTileUs,
-                                  const int (&resident)[kNumSizes]) {
-  const float kTilesPerUs = 7.3e6f / (float)tile_bytes;
-  constexpr float kSegmentUs = 1.f, kRagged = 0.35f;
-  ClusterShape best = {1, 1};
+template <typename General>
+ClusterShape cluster_shape(const CallShape &s, int batch, float fill, General general,
+                           const int (&resident)[kNumSizes]) {
+  const float w_equal = batch == 1 || fill > kFull ? 1.f : 0.f;
+  const float w_ragged = batch == 1 ? 0.f : (w_equal > 0.f ? 0.5f : 1.f);
+  const float mean = w_equal > 0.f ? kRagged : fill;
+  ClusterShape best = {1, 1, false};
   float best_us = 0.f;
   for (int i = 0; i < kNumSizes; ++i) {
-    const int c = kSizes[i], k = resident[i] < groups ? resident[i] : groups;
-    const int q = groups / k, r = groups % k;
-    const float cta = (float)tiles / (float)c * kTileUs;  // a group's tiles on one of its CTAs
-    float us = fmaxf((float)k * (float)q * (float)tiles / kTilesPerUs,
-                     (float)q * cta + kSegmentUs * (1.f + (float)(q - 1) / (float)c));
-    if (r) us += fmaxf((float)r * (float)tiles / kTilesPerUs, cta + kSegmentUs / (float)c);
-    us *= 1.f + 0.0125f * log2f((float)kMaxCluster / (float)c);
-    if (batch > 1)
-      us += fmaxf(kRagged * (float)groups * (float)tiles / kTilesPerUs,
-                  kRagged * (float)groups * (float)tiles / (float)(k * c) * kTileUs) + 0.5f * cta;
+    const int c = kSizes[i], k = resident[i] < s.groups ? resident[i] : s.groups;
+    const float wide = 1.f + 0.0125f * log2f((float)kMaxCluster / (float)c);
+    const float us = w_equal * (kCallUs + wide * equal_us(s, c, k)) +
+                     w_ragged * (kCallUs + wide * ragged_us(s, c, k, mean));
     if (best_us == 0.f || us < best_us) {
       best_us = us;
-      best = {c, k};
+      best = {c, k, false};
     }
   }
+  best.general = w_equal * general(1.f) + w_ragged * general(mean) < 1.05f * best_us;
   return best;
 }
 
 template <typename T, int D, int G>
-cudaError_t launch_cluster_typed(const AttendArgs &a, int64_t rows_total, cudaStream_t s) {
+cudaError_t launch_cluster_typed(const AttendArgs &a, int64_t rows_total, bool *general,
+                                 cudaStream_t s) {
+  using P = Pass<T, D, G>;
   int resident[kNumSizes];
   LG_TRY((resident_clusters<T, D, G>(resident)));
-  constexpr int rows = Pass<T, D, G>::kTile;
+  constexpr int rows = P::kTile;
+  const int tiles = (a.max_len + rows - 1) / rows;
+  const CallShape shape = {a.n_layers * a.batch * a.H_kv, tiles,
+                           (float)ClusterCfg<T, D, G>::kTileBytes, P::kTileUs,
+                           tiles < 8 ? 1.f : P::kSegmentUs};
+  const float fill = fminf(1.f, (float)a.S_total / ((float)a.batch * (float)a.max_len));
+  const ClusterShape sh = cluster_shape(
+      shape, a.batch, fill, [&](float mean) { return P::general_us(a, shape, mean); }, resident);
+  *general = sh.general;
+  if (sh.general) return cudaSuccess;
   CUtensorMap mk, mv;
   if (!make_kv_map(&mk, a.K, Elem<T>::kDtype, D, rows_total, rows) ||
       !make_kv_map(&mv, a.V, Elem<T>::kDtype, D, rows_total, rows))
     return cudaErrorInvalidValue;
-  const ClusterShape sh =
-      cluster_shape(a.n_layers * a.batch * a.H_kv, a.batch, (a.max_len + rows - 1) / rows,
-                    ClusterCfg<T, D, G>::kTileBytes, Pass<T, D, G>::kTileUs, resident);
   auto kern = attend_cluster_kernel<T, D, G>;
   LG_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               ClusterCfg<T, D, G>::kSmem));
@@ -824,25 +870,27 @@ cudaError_t launch_cluster_typed(const AttendArgs &a, int64_t rows_total, cudaSt
 }
 
 template <typename T, int D>
-cudaError_t launch_cluster_d(const AttendArgs &a, int g, int64_t rows_total, cudaStream_t s) {
+cudaError_t launch_cluster_d(const AttendArgs &a, int g, int64_t rows_total, bool *general,
+                             cudaStream_t s) {
   switch (g) {
-    case 1: return launch_cluster_typed<T, D, 1>(a, rows_total, s);
-    case 2: return launch_cluster_typed<T, D, 2>(a, rows_total, s);
-    case 3: return launch_cluster_typed<T, D, 3>(a, rows_total, s);
-    case 4: return launch_cluster_typed<T, D, 4>(a, rows_total, s);
-    case 5: return launch_cluster_typed<T, D, 5>(a, rows_total, s);
-    case 6: return launch_cluster_typed<T, D, 6>(a, rows_total, s);
-    case 7: return launch_cluster_typed<T, D, 7>(a, rows_total, s);
-    case 8: return launch_cluster_typed<T, D, 8>(a, rows_total, s);
+    case 1: return launch_cluster_typed<T, D, 1>(a, rows_total, general, s);
+    case 2: return launch_cluster_typed<T, D, 2>(a, rows_total, general, s);
+    case 3: return launch_cluster_typed<T, D, 3>(a, rows_total, general, s);
+    case 4: return launch_cluster_typed<T, D, 4>(a, rows_total, general, s);
+    case 5: return launch_cluster_typed<T, D, 5>(a, rows_total, general, s);
+    case 6: return launch_cluster_typed<T, D, 6>(a, rows_total, general, s);
+    case 7: return launch_cluster_typed<T, D, 7>(a, rows_total, general, s);
+    case 8: return launch_cluster_typed<T, D, 8>(a, rows_total, general, s);
   }
   return cudaErrorInvalidValue;
 }
 
-// the pass over a cache of rows_total rows of T
+// the pass over a cache of rows_total rows of T, or *general set and nothing launched
 template <typename T>
-cudaError_t launch_cluster(const AttendArgs &a, int d, int g, int64_t rows_total, cudaStream_t s) {
-  if (d == 128) return launch_cluster_d<T, 128>(a, g, rows_total, s);
-  if (d == 64) return launch_cluster_d<T, 64>(a, g, rows_total, s);
+cudaError_t launch_cluster(const AttendArgs &a, int d, int g, int64_t rows_total, bool *general,
+                           cudaStream_t s) {
+  if (d == 128) return launch_cluster_d<T, 128>(a, g, rows_total, general, s);
+  if (d == 64) return launch_cluster_d<T, 64>(a, g, rows_total, general, s);
   return cudaErrorInvalidValue;
 }
 

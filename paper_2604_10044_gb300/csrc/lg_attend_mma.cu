@@ -1,6 +1,7 @@
 // Decode attention over a bf16 KV cache fused with the guard's per-head statistics (LoopGuard
 // Sec. 3.1, Eq. 1; statistics read by Sec. 5.2), on tensor cores: the pass for batches of more than
-// 64 sequences and the longest calls (lg_attend_cluster.cu takes the others).
+// 64 sequences, the longest calls, and those of few long groups that the cluster pass's rule leaves
+// here (lg_attend_cluster.cuh takes the others).
 //
 // Persistent CTAs (one per SM) start on chunks blockIdx.x and blockIdx.x + gridDim.x and take
 // further chunks from a shared counter, each a run of consecutive rows of one (layer,

@@ -37,13 +37,14 @@ int mma_tile_rows();
 cudaError_t launch_attend_mma_partial(const AttendArgs &a, int d, int g, int64_t rows_total,
                                       cudaStream_t s);
 
-// the cluster pass (lg_attend_cluster.cuh): whether it takes a call, and the call
+// the cluster pass (lg_attend_cluster.cuh): whether it can take a call, and the call (*general set
+// and nothing launched where the pass past its limits is expected to be faster)
 bool attend_cluster_takes(const AttendArgs &a, int tile_rows, int64_t rows_total);
 cudaError_t launch_attend_cluster(const AttendArgs &a, int d, int g, int64_t rows_total,
-                                  cudaStream_t s);
+                                  bool *general, cudaStream_t s);
 int cluster_f32_tile_rows();
 cudaError_t launch_attend_cluster_f32(const AttendArgs &a, int d, int g, int64_t rows_total,
-                                      cudaStream_t s);
+                                      bool *general, cudaStream_t s);
 
 // guard kernels (lg_guard.cu)
 cudaError_t launch_begin_step(const lg_cache &c, cudaStream_t s);

@@ -177,3 +177,27 @@ def test_long_fp32_segments_keep_their_precision(cuda, lens, H_kv, G, d):
     want, ws = _exact(k, v, q, lens, off, 0, 1, 64)
     assert ((got.double() - want).norm() / want.norm()).item() < 4e-7
     assert ((st.double() - ws).norm() / ws.norm()).item() < 4e-7
+
+
+@pytest.mark.parametrize("lens,H_kv,G,d,dtype,h2o", [
+    # few long groups, with 8 CTAs each in the cluster pass: the general pass is the faster
+    ([131071], 2, 1, 128, "bf16", False), ([60000, 500, 800, 3], 2, 1, 128, "bf16", True),
+    # a CTA's arithmetic bounds the cluster pass over fp32 rows with many heads a group
+    ([9036] * 6, 8, 6, 64, "f32", False), ([20000, 700, 0, 5000], 2, 8, 128, "f32", True),
+    # beside them, calls that the cluster pass keeps
+    ([9036] * 6, 8, 6, 64, "bf16", False), ([20000, 700, 0, 5000], 2, 1, 128, "f32", True)])
+def test_either_side_of_the_choice(cuda, lens, H_kv, G, d, dtype, h2o):
+    g = torch.Generator(device=cuda)
+    g.manual_seed(sum(lens) + G)
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    S = int(sum(lens)) + len(lens)
+    k, v = (torch.randn((1, H_kv, S, d), generator=g, device=cuda).to(tdt) for _ in range(2))
+    q = torch.randn((1, len(lens), H_kv * G, d), generator=g, device=cuda).to(tdt)
+    got, st, sc, off = _run(k, v, q, lens, 0, 1, 64, h2o, 0)
+    want, ws = _exact(k, v, q, lens, off, 0, 1, 64)
+    # the parity tests' bounds: bf16 output rounding, fp32 sums
+    _close(got, want, *((2e-2, 1e-3) if dtype == "bf16" else (1e-4, 1e-5)), "out")
+    _close(st, ws, 1e-4, 1e-6, "stats")
+    if h2o:
+        total, all_ = sc.double().sum(-1), float(G * sum(n > 0 for n in lens))
+        assert torch.allclose(total, torch.full_like(total, all_), rtol=1e-5)
