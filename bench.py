@@ -449,8 +449,10 @@ class GpuBench:
     # launches of this repository's kernels per step (harness + path)
     def launches_per_step(self):
         calls = math.ceil(self.w.L / self.nl)
-        # per call on the tensor-core path: the counter reset and the pass (it merges its own
-        # partials); a partial pass and a merge on the fp32 path; H2O adds the score update
+        # per call past the cluster pass's limits: the counter reset and the persistent pass, or on
+        # an fp32 cache a partial pass and a merge; H2O adds the score update.  A call that the
+        # cluster pass takes is one kernel instead of two (attend_cluster_takes in
+        # csrc/lg_attend_cluster.cu): there this is an upper bound, which the line says.
         attend = 2 + (1 if self.policy == "h2o" else 0)
         path = 1 + 1 + attend * calls               # begin, append (+sketch), attend
         harness = 1                                 # the step's inputs
@@ -781,7 +783,11 @@ def run_gpu(args, ws, rank, local):
             "guard_ms_per_step": round(sum(guard_ms) / len(sampled), 4)},
         "eager_ms_per_step": round(eager_ms / K, 4) if eager_ms is not None else None,
         "gpu_launches": (path_l + harness_l) * K,
-        "gpu_launches_detail": {"path_per_step": path_l, "harness_per_step": harness_l},
+        "gpu_launches_detail": {
+            "path_per_step": path_l, "harness_per_step": harness_l,
+            "note": "two kernels an attention call, as past the cluster pass's limits (more than "
+                    "64 sequences, or 2^20 tiles as the bandwidth sweep's); a call within them is "
+                    "one kernel, so that the steps launched are fewer by their attention calls"},
         "clocks": clk,
     }
     if e2e:
