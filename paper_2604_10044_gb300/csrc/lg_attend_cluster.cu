@@ -28,7 +28,10 @@ struct Pass<__nv_bfloat16, D, G> {
   }
   static constexpr int kFoldUnits = 1;
   static constexpr bool kEarlyUnits = true;
-  static constexpr int kFlushTiles = 0;  // (a lane's sums take one rounding per 16 rows here)
+  // No flush: o takes one rounded addition per 16 rows (kFresh in lg_mma_tile.cuh), l, u and sigma
+  // one per row of a lane (two rows a block and head), so that 2 sequences of 131071 rows have l
+  // 2.2e-7 off its 64-bit value where the persistent pass has 3.0e-7.
+  static constexpr int kFlushTiles = 0;
 
   WarpSums<D> acc;
   uint32_t qf[D / 16][2];
@@ -39,7 +42,7 @@ struct Pass<__nv_bfloat16, D, G> {
   }
   __device__ __forceinline__ void update(unsigned char *stage, int tile_rows, int suffix,
                                          float *logits, float qscale, int warp, int lane) {
-    tile_update<D, G, kBlocks>(acc, qf, stage, tile_rows, suffix, logits, qscale, warp, lane);
+    tile_update<D, G, kBlocks, true>(acc, qf, stage, tile_rows, suffix, logits, qscale, warp, lane);
   }
   __device__ __forceinline__ void join() { acc.join_lanes(); }
   __device__ __forceinline__ void store(float *rows, bool, int lane) {

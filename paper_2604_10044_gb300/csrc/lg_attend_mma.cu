@@ -547,7 +547,7 @@ attend_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
       load_q<D, G>(qf, qbuf + st * C::kQBytes, lane);
       acc.reset();
     }
-    tile_update<D, G, 2>(acc, qf, smem + (size_t)st * C::kStageBytes,
+    tile_update<D, G, 2, false>(acc, qf, smem + (size_t)st * C::kStageBytes,
                          min(kTile, rows - t * kTile), suffix_lo - row0 - t * kTile,
                          a.logits ? a.logits + (lrow0 + t * kTile) * G : nullptr, a.qscale, warp,
                          lane);

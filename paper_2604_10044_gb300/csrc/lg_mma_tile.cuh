@@ -74,6 +74,15 @@ __device__ __forceinline__ void mma_bf16(float *d, uint32_t a0, uint32_t a1, uin
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// the same into fresh sums
+__device__ __forceinline__ void mma_bf16_zero(float *d, uint32_t a0, uint32_t a1, uint32_t a2,
+                                              uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, "
+      "{%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+}
+
 __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
   uint32_t d;
   asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
@@ -158,7 +167,16 @@ __device__ __forceinline__ void load_q(uint32_t (&qf)[D / 16][2], const unsigned
 // One consumer warp's MB blocks of 16 rows of a tile in `stage` (K boxes, then V boxes): logits,
 // online softmax, sums and o^T.  tile_rows: rows of the tile in use; rows from `suffix` on (tile row
 // numbers) count toward the suffix mass; logits: nullable, the tile's first row [rows][G].
-template <int D, int G, int MB>
+// kFresh: a block's products go into sums of their own, which are then added to o.  The matrix
+// unit truncates where an addition rounds, so a chain of its additions falls short in proportion
+// to its length: with a segment's 342 blocks in one chain (2 sequences of 131071 rows, 8 heads a
+// group, clusters of 6) the output was 1.28e-5 of its norm off the 64-bit value before its rounding
+// to bf16, with this 2.36e-6; the persistent pass, whose chunks of 8 tiles keep the chains short,
+// has 2.40e-6 there (most of it P's two bf16 parts).  It costs nothing at one tile a CTA, 0 to 1 %
+// of most calls and 3.5 % where a CTA's own work bounds the call (1 sequence of 16384 rows, 4 heads:
+// 17.9 -> 18.5 us); flushes to shared memory every 16 blocks cost more (the long call above 157.0
+// -> 159.5 us, against 156.9).
+template <int D, int G, int MB, bool kFresh>
 __device__ __forceinline__ void tile_update(WarpSums<D> &acc, const uint32_t (&qf)[D / 16][2],
                                             unsigned char *stage, int tile_rows, int suffix,
                                             float *logits, float qscale, int warp, int lane) {
@@ -298,12 +316,23 @@ __device__ __forceinline__ void tile_update(WarpSums<D> &acc, const uint32_t (&q
       for (int j = 0; j < 4; ++j)
         ldsm_x4_trans(vbase + (e0 >> 2) * kBoxBytes + swz(r, j * 2 + (msel & 1)), va[j][0],
                       va[j][1], va[j][2], va[j][3]);
+      float fresh[4][4];
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        mma_bf16(o[e0 + j], va[j][0], va[j][1], va[j][2], va[j][3], pb[mb][0], pb[mb][1]);
+        if (kFresh)
+          mma_bf16_zero(fresh[j], va[j][0], va[j][1], va[j][2], va[j][3], pb[mb][0], pb[mb][1]);
+        else
+          mma_bf16(o[e0 + j], va[j][0], va[j][1], va[j][2], va[j][3], pb[mb][0], pb[mb][1]);
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        mma_bf16(o[e0 + j], va[j][0], va[j][1], va[j][2], va[j][3], pl[mb][0], pl[mb][1]);
+        mma_bf16(kFresh ? fresh[j] : o[e0 + j], va[j][0], va[j][1], va[j][2], va[j][3], pl[mb][0],
+                 pl[mb][1]);
+      if (kFresh) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) o[e0 + j][k] += fresh[j][k];
+      }
     }
   }
   __syncwarp();
