@@ -244,7 +244,8 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
   __shared__ __align__(8) uint64_t recv_bar[2];  // a slot's pieces have arrived
   __shared__ __align__(8) uint64_t q_full[2], q_empty[2];  // query rows of segment i in buffer i & 1
   __shared__ int s_len[kClusterSeqs], s_pre[kClusterSeqs], s_off[kClusterSeqs];
-  __shared__ int s_total, s_c0, s_c1, s_empty, s_skip, s_bad;
+  __shared__ int s_total, s_c0, s_c1, s_empty, s_skip;
+  __shared__ int s_stop;  // bit 0: the status was set before this call, bit 1: a wait ran out
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   unsigned char *qbuf = smem + Cl::kStages * Cl::kStageBytes;  // [2][G][D]
@@ -280,6 +281,7 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
   __syncwarp();
   // waited for before the first store to a peer: every CTA has started and set up its barriers
   cluster_arrive();
+  auto stopped = [&] { return *(volatile int *)&s_stop; };
   TileSpace ts;
   ts.len = s_len;
   ts.pre = s_pre;
@@ -469,7 +471,7 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
       s_c1 = c1;
       s_empty = any_empty && !bad;
       s_skip = hit ? 0 : guess_tiles;
-      s_bad = bad;
+      s_stop = bad != 0;
     }
     __syncwarp();
     named_arrive<Cl::kThreads>(1);
@@ -489,15 +491,17 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
         const int row = row0 + s_off[g.b] - g.start * kTile;
         for (; t < end; ++t, ++it) {
           const int st = it % Cl::kStages;
+          // (a stage whose copy was late is handed back with s_stop set, and not used again)
           if (it >= (uint32_t)Cl::kStages &&
-              timed_out(&empty_bar[st], ((it / Cl::kStages) - 1) & 1)) {
+              (timed_out(&empty_bar[st], ((it / Cl::kStages) - 1) & 1) || stopped())) {
             ok = false;
             break;
           }
           copy_tile(st, row + t * kTile, policy);
           if (!begun) {
             const int qb = seg & 1;
-            if (seg >= 2 && timed_out(&q_empty[qb], ((seg >> 1) - 1) & 1)) {
+            if (seg >= 2 &&
+                (timed_out(&q_empty[qb], ((seg >> 1) - 1) & 1) || stopped())) {
               ok = false;
               break;
             }
@@ -581,25 +585,24 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
   uint32_t it = 0, seg = 0;
   // With the status set nothing is read or written, but a CTA still passes its (meaningless)
   // pieces on: the status may have been set by another CTA of this launch, and its peers wait.
-  const bool bad = s_bad;
-  bool ok = !bad;  // also false once a copy did not land in time
+  const bool bad = stopped() & 1;
+  // The waits of one lane: at the limit a warp's lanes may see a barrier differently, and what
+  // follows has shuffles and matrix instructions of all lanes, so nothing branches on them.  After
+  // the first that runs out no copy is waited for; what is late is worked on as it is.
+  auto ran_out = [&] {
+    set_status(a.status, LG_ERR_TIMEOUT);
+    atomicOr(&s_stop, 2);
+  };
   auto landed = [&](uint64_t *bar, uint32_t parity) {
-    if (ok && !mbar_wait(bar, parity)) {
-      set_status(a.status, LG_ERR_TIMEOUT);
-      ok = false;
-    }
-    return ok;
+    if (!mbar_try_wait(bar, parity) && !stopped() && !mbar_wait(bar, parity)) ran_out();
   };
   if (s_skip > 0) {
     // a dropped guess: its stages and queries pass unused
     bool in = mbar_wait(&q_full[0], 0);
     for (; it < (uint32_t)s_skip; ++it) {
-      in = mbar_wait(&full_bar[it], 0) && in;
+      in = in && mbar_wait(&full_bar[it], 0);
+      if (!in) ran_out();
       if (lane == 0) mbar_arrive(&empty_bar[it]);
-    }
-    if (!in) {
-      set_status(a.status, LG_ERR_TIMEOUT);
-      ok = false;
     }
     if (lane == 0) mbar_arrive(&q_empty[0]);
     seg = 1;
@@ -630,16 +633,15 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     // (all of the segment at once, or kFlushTiles tiles at a time)
     do {
       const int from = t, stop = P::kFlushTiles ? min(end, t + P::kFlushTiles) : end;
-      if (landed(&q_full[qb], (seg >> 1) & 1))
-        pass.begin(qbuf + qb * Cl::kQBytes, from == start, a.qscale, lane);
+      landed(&q_full[qb], (seg >> 1) & 1);
+      pass.begin(qbuf + qb * Cl::kQBytes, from == start, a.qscale, lane);
       for (; t < stop; ++t, ++it) {
         const int st = it % Cl::kStages;
-        if (landed(&full_bar[st], (it / Cl::kStages) & 1)) {
-          const int r0 = (t - g.start) * kTile;
-          float *logits = a.logits ? a.logits + (int64_t)(lrow + r0) * G : nullptr;
-          pass.update(smem + (size_t)st * Cl::kStageBytes, min(kTile, n - r0), suffix_lo - r0,
-                      logits, a.qscale, warp, lane);
-        }
+        landed(&full_bar[st], (it / Cl::kStages) & 1);
+        const int r0 = (t - g.start) * kTile;
+        float *logits = a.logits && !bad ? a.logits + (int64_t)(lrow + r0) * G : nullptr;
+        pass.update(smem + (size_t)st * Cl::kStageBytes, min(kTile, n - r0), suffix_lo - r0, logits,
+                    a.qscale, warp, lane);
         if (lane == 0) mbar_arrive(&empty_bar[st]);
       }
       if (t == end && lane == 0) mbar_arrive(&q_empty[qb]);

@@ -111,3 +111,33 @@ def test_cluster_bookkeeping():
         subprocess.run(["g++", "-O2", "-std=c++17", cpp, "-o", exe], check=True)
         r = subprocess.run([exe], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout
+
+
+def _kernel():
+    """the cluster pass's producer and consumers, without comments"""
+    text = open(SRC).read()
+    body = re.sub(r"//[^\n]*", "", text[text.index("attend_cluster_kernel(const"):])
+    body = body[:body.index("\n}\n") + 2]  # to the kernel's own closing brace
+    at = body.index("pdl_enter();\n  named_sync")
+    return body[:at], body[at:]
+
+
+def test_nothing_of_a_warp_branches_on_a_lanes_wait():
+    """What follows a wait uses shuffles and matrix instructions of all lanes, and at the time limit a
+    warp's lanes may see the barrier differently: so a wait that ran out sets a flag of the CTA and
+    the warp goes on together.  After that no copy is waited for, and the producer, which sees the
+    flag with any stage or query buffer handed back after it, arms none of their barriers again."""
+    producer, code = _kernel()
+    landed = re.search(r"auto landed = [^{]*\{(.*?)\n  \};", code, re.S).group(1)
+    assert re.sub(r"\s+", " ", landed).strip() == \
+        "if (!mbar_try_wait(bar, parity) && !stopped() && !mbar_wait(bar, parity)) ran_out();"
+    assert "s_stop, 2" in re.search(r"auto ran_out = [^{]*\{(.*?)\n  \};", code, re.S).group(1)
+    for use in re.finditer(r"[^;{}]*(pass\.begin|pass\.update|landed)\(&?[^;]*;", code):
+        assert "if (" not in use.group(0) or "P::" in use.group(0), use.group(0)
+    skip = code[code.index("if (s_skip > 0)"):code.index("for (int t = u0;")]
+    assert "in = in && mbar_wait(&full_bar[it], 0);" in skip and "if (!in) ran_out();" in skip
+    # (those two, the one in landed() and the one of the pieces)
+    assert len(re.findall(r"\bmbar_wait(?:_cluster)?\(", code)) == 4
+    for bar in ("empty_bar", "q_empty"):
+        wait = re.search(r"timed_out\(&%s\[[^;{]*\{" % bar, producer).group(0)
+        assert "|| stopped()" in wait, wait
