@@ -697,7 +697,7 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     const int mine = slot ? slot1.mine : slot0.mine, np = slot ? slot1.np : slot0.np;
     const int head0 = slot ? slot1.head0 : slot0.head0;
     if (np == 0) continue;
-    if (!mbar_wait_cluster(&recv_bar[slot], 0)) set_status(a.status, LG_ERR_TIMEOUT);
+    if (!mbar_wait_cluster(&recv_bar[slot], 0)) ran_out();
     if (bad) continue;
 #pragma unroll 1
     for (int j = warp; j * np + mine < Cl::kUnits; j += kWarps) {
@@ -725,6 +725,14 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
       }
       finish<T, D>(a, head0 + un % G, un / G * 32 + lane, un < G && lane == 0, M, l, u, sg, o);
     }
+  }
+  __syncwarp();
+  if (stopped() & 2) {
+    // A peer may still be about to send pieces into this CTA's shared memory (every CTA sends
+    // them, late or not): it stays until every thread of the cluster has ended or come here.
+    cluster_arrive();
+    cluster_wait();
+    linger();
   }
 }
 

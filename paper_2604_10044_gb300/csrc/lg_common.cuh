@@ -158,6 +158,13 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity
   }
 }
 
+// After a wait that ran out, before the CTA's shared memory goes to another: as long again, for
+// copies into it that are still in flight.
+__device__ __forceinline__ void linger() {
+  const uint64_t t0 = global_ns();
+  while (global_ns() - t0 < kWaitLimitNs) __nanosleep(1000);
+}
+
 // ------------------------------------------------------------------ bulk copies
 
 // 1-D bulk copy global -> shared, completion counted in bytes on `bar`.  Both addresses

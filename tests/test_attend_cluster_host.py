@@ -141,3 +141,20 @@ def test_nothing_of_a_warp_branches_on_a_lanes_wait():
     for bar in ("empty_bar", "q_empty"):
         wait = re.search(r"timed_out\(&%s\[[^;{]*\{" % bar, producer).group(0)
         assert "|| stopped()" in wait, wait
+
+
+def test_a_cta_outlives_what_is_sent_to_it():
+    """A CTA leaves when the pieces for it have arrived, or, once a wait ran out, when every thread
+    of the cluster has ended or met it at a barrier and what is in flight has had time to land.
+    Every CTA reaches its sends whatever became of its own copies, so that the barrier is met."""
+    _, code = _kernel()
+    assert re.search(r"__syncwarp\(\);\s*if \(stopped\(\) & 2\) \{\s*cluster_arrive\(\);\s*"
+                     r"cluster_wait\(\);\s*linger\(\);\s*\}\s*\}$", code), code[-300:]
+    lambdas = re.sub(r"auto \w+ = \[&\].*?\n  \};", "", code, flags=re.S)
+    assert not re.search(r"\breturn\b", re.sub(r"if \(whole\) return;", "", lambdas))
+    sends = code[code.index("for (int task = warp;"):code.index("slot0 : slot1) = Slot")]
+    whole, shared = sends.split("} else {")
+    assert "if (!bad) finish" in whole and "peer_st(" in shared and "if (lane == 0) peer_st4" in shared
+    # a CTA that owns units waits for their pieces with the status set, too
+    merge = code[code.index("for (int slot = 0;"):]
+    assert "if (!mbar_wait_cluster(&recv_bar[slot], 0)) ran_out();" in merge[:merge.index("if (bad")]
