@@ -54,6 +54,7 @@ attend_partial_kernel(AttendArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t full_bar[C::kStages];
   __shared__ __align__(8) uint64_t empty_bar[C::kStages];
+  __shared__ int s_late;  // a wait ran out: no other copy is waited for, issued or used
 
   const int chunk = blockIdx.x, kvh = blockIdx.y;
   const int b = blockIdx.z % a.batch, lloc = blockIdx.z / a.batch;
@@ -79,17 +80,22 @@ attend_partial_kernel(AttendArgs a) {
       mbar_init(&empty_bar[s], C::kWarps);
     }
     mbar_fence_init();
+    s_late = 0;
   }
   __syncthreads();
+  auto stopped = [&] { return *(volatile int *)&s_late; };
 
   if (warp == C::kWarps) {
     // producer: one thread issues the bulk copies of every tile of the chunk
     if (lane == 0) {
       for (int t = 0; t < ntiles; ++t) {
         const int st = t % C::kStages;
-        if (t >= C::kStages && !mbar_wait(&empty_bar[st], ((t / C::kStages) - 1) & 1)) {
-          set_status(a.status, LG_ERR_TIMEOUT);
-          break;
+        if (t >= C::kStages) {
+          if (!mbar_wait(&empty_bar[st], ((t / C::kStages) - 1) & 1)) {
+            set_status(a.status, LG_ERR_TIMEOUT);
+            break;
+          }
+          if (stopped()) break;
         }
         const int rt = min(C::kTile, rows - t * C::kTile);
         const uint32_t bytes = (uint32_t)rt * C::kRowBytes;
@@ -134,14 +140,15 @@ attend_partial_kernel(AttendArgs a) {
   const int suffix_lo = n - min(a.suffix_w, n);
   float *logits = a.logits;
   const int64_t lrow0 = ((int64_t)lloc * a.H_kv + kvh) * a.S_total + a.seq_off[b] + row0;
-  bool ok = true;
 
-  for (int t = 0; t < ntiles && ok; ++t) {
+  for (int t = 0; t < ntiles; ++t) {
     const int st = t % C::kStages;
-    if (!mbar_wait(&full_bar[st], (t / C::kStages) & 1)) {
+    // (at the limit a warp's lanes may see the barrier differently: they go on together all the
+    // same, as what follows has shuffles of all lanes)
+    const uint32_t parity = (t / C::kStages) & 1;
+    if (!mbar_try_wait(&full_bar[st], parity) && !stopped() && !mbar_wait(&full_bar[st], parity)) {
       set_status(a.status, LG_ERR_TIMEOUT);
-      ok = false;
-      break;
+      *(volatile int *)&s_late = 1;
     }
     const unsigned char *ks = smem + (size_t)st * 2 * C::kTileBytes;
     const unsigned char *vs = ks + C::kTileBytes;
@@ -211,9 +218,13 @@ attend_partial_kernel(AttendArgs a) {
   }
 
   // ---------------------------------------------------------------- CTA merge of row groups
-  // all copies have landed (every tile was waited on), so the ring is free for scratch
+  // all copies have landed (every tile was waited on) unless a wait ran out, so the ring is free for
+  // scratch
   asm volatile("bar.sync 1, %0;" ::"n"(C::kWarps * 32) : "memory");
-  if (!ok) return;
+  if (stopped()) {  // the same for every warp: none sets it after the barrier
+    linger();
+    return;
+  }
   float *so = reinterpret_cast<float *>(smem);            // [kGroups][G][D]
   float *ss = so + C::kGroups * G * D;                    // [kGroups][GP][4]
 #pragma unroll

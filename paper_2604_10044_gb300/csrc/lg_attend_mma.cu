@@ -355,7 +355,7 @@ attend_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
     // chunk partial of the group.
     for (uint32_t tk = warp - kMergerWarp0;; tk += kMergers) {
       const int slot = tk % kTickets;
-      if (!mbar_wait(&tfull[slot], (tk / kTickets) & 1)) {
+      if (!mbar_wait_warp(&tfull[slot], (tk / kTickets) & 1)) {
         set_status(a.status, LG_ERR_TIMEOUT);
         return;
       }
@@ -528,8 +528,9 @@ attend_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
   bool handoff = true;    // false once a buffer or ticket slot was not released in time
   for (uint32_t it = 0;; ++it) {
     const int st = it % C::kStages;
-    if (!mbar_wait(&full_bar[st], (it / C::kStages) & 1)) {
+    if (!mbar_wait_warp(&full_bar[st], (it / C::kStages) & 1)) {
       set_status(a.status, LG_ERR_TIMEOUT);
+      linger();
       return;
     }
     const int c = stage_chunk[st];

@@ -158,6 +158,13 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity
   }
 }
 
+// Bounded wait of a whole warp (every lane calls it, converged): one answer for all lanes, as the
+// lanes may see the barrier differently at the limit and the warp goes on to shuffles and matrix
+// instructions of all of them.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+}
+
 // After a wait that ran out, before the CTA's shared memory goes to another: as long again, for
 // copies into it that are still in flight.
 __device__ __forceinline__ void linger() {

@@ -158,3 +158,22 @@ def test_a_cta_outlives_what_is_sent_to_it():
     # a CTA that owns units waits for their pieces with the status set, too
     merge = code[code.index("for (int slot = 0;"):]
     assert "if (!mbar_wait_cluster(&recv_bar[slot], 0)) ran_out();" in merge[:merge.index("if (bad")]
+
+
+def test_the_general_passes_waits_have_one_answer_a_warp():
+    """The same in the persistent pass, whose consumer and merger warps end together after a wait that
+    ran out, and in the chunk kernel, whose warps go on and all end after the CTA's next barrier
+    (a warp that left before it would leave the others waiting at the one after)."""
+    src = os.path.dirname(SRC)
+    mma = re.sub(r"//[^\n]*", "", open(os.path.join(src, "lg_attend_mma.cu")).read())
+    for bar in ("full_bar", "tfull"):
+        waits = re.findall(r"(mbar_wait\w*)\(&%s\[" % bar, mma)
+        assert waits == ["mbar_wait_warp"], (bar, waits)
+    assert re.search(r"mbar_wait_warp\(&full_bar[^{]*\{[^}]*linger\(\);\s*return;", mma)
+    common = open(os.path.join(src, "lg_common.cuh")).read()
+    assert "return __all_sync(0xffffffffu, mbar_wait(bar, parity));" in common
+    chunk = re.sub(r"//[^\n]*", "", open(os.path.join(src, "lg_attend.cu")).read())
+    chunk = chunk[chunk.index("attend_partial_kernel(AttendArgs a)"):chunk.index("attend_combine_kernel")]
+    loop, rest = chunk[chunk.index("const int suffix_lo"):].split("bar.sync 1", 1)
+    assert "break" not in loop and "ok" not in re.findall(r"\b\w+\b", loop)
+    assert re.search(r"^[^}]*?if \(stopped\(\)\) \{\s*linger\(\);\s*return;\s*\}", rest)
