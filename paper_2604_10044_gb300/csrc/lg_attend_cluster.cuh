@@ -409,7 +409,10 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
     for (int k = 0; k < 2; ++k) {
       if (2 * lane + k < a.batch) s_off[2 * lane + k] = (int)off[k];
       hit = hit && (int)off[k] == early_off[k];
-      if (n[k] > a.max_len) {
+      // (a negative length is an error over fp32 rows and reads as none over bf16 ones, as in the
+      // general passes)
+      if (n[k] > a.max_len ||
+          (Elem<T>::kDtype == LG_F32 && n[k] < 0 && 2 * lane + k < a.batch)) {
         set_status(a.status, LG_ERR_CAPACITY);
         n[k] = -1;
         hit = false;

@@ -43,6 +43,19 @@ def test_max_len_below_a_length_sets_status(cuda):
     assert lg.lg_read_device_status(cache) == 4
 
 
+@pytest.mark.parametrize("batch", [2, 65])  # the cluster pass, the chunk kernel (past 64 sequences)
+def test_negative_length_over_fp32_rows_sets_status(cuda, batch):
+    """both fp32 passes check a length against zero before they use it"""
+    H_kv, H_q, d, n = 2, 4, 64, 100
+    cache = lg.Cache(1, H_kv, d, "f32", np.arange(batch) * (n + 1), [n + 1] * batch, [n] * batch,
+                     cuda)
+    g = lg.Guard(cache, H_q)
+    cache.len[batch - 1] = -3
+    q = torch.zeros((1, batch, H_q, d), device=cuda)
+    lg.lg_decode_attend(cache, 0, 1, q, H_q, 0.1, g.out, g.stats, 64, 0, g.max_len, g.ws)
+    assert lg.lg_read_device_status(cache) == 4
+
+
 def test_budget_without_room_sets_status(cuda):
     w, cache = _small(cuda)
     g = lg.Guard(cache, w.H_q)
