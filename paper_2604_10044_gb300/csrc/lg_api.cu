@@ -216,6 +216,8 @@ lg_status lg_decode_attend(const lg_cache *c, int layer0, int n_layers, const vo
   a.max_len = max_len;
   a.suffix_w = suffix_w;
   a.qscale = scale * 1.4426950408889634f;
+  a.gate = nullptr;
+  a.sms = 0;
   const int64_t rows_total = (int64_t)c->L * c->H_kv * c->S_total;
   if (c->dtype == LG_BF16 && rows_total >= ((int64_t)1 << 31)) return LG_ERR_UNSUPPORTED;
   return cuda_status(lg::launch_attend(a, c->dtype, c->d, g, rows_total, out, stats, final_ml,

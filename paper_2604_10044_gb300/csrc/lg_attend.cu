@@ -50,6 +50,7 @@ template <typename T, int D, int G>
 __global__ void __launch_bounds__(AttendCfg<T, D, G>::kThreads)
 attend_partial_kernel(AttendArgs a) {
   pdl_enter();
+  if (a.gate && *a.gate < 0) return;  // the cluster pass has done the call
   using C = AttendCfg<T, D, G>;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t full_bar[C::kStages];
@@ -281,6 +282,7 @@ __global__ void attend_combine_kernel(AttendArgs a, void *out, float *stats, flo
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t head = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   if (head >= (int64_t)a.n_layers * a.batch * a.H_q) return;
+  if (a.gate && *a.gate < 0) return;
   if (status_bad(a.status)) return;
   const int b = (int)((head / a.H_q) % a.batch);
   const int n = a.len[b];
@@ -400,7 +402,7 @@ __global__ void __launch_bounds__(256) h2o_accumulate_kernel(AttendArgs a, float
 // ------------------------------------------------------------------ launch
 
 template <typename T, int D, int G>
-static cudaError_t launch_typed(const AttendArgs &a, int64_t rows_total, void *out, float *stats,
+static cudaError_t launch_typed(AttendArgs a, int64_t rows_total, void *out, float *stats,
                                 float *final_ml, float *h2o, cudaStream_t s) {
   using C = AttendCfg<T, D, G>;
   cudaError_t e = cudaSuccess;

@@ -15,17 +15,6 @@ struct Pass<__nv_bfloat16, D, G> {
   // shared memory for eight partials)
   static constexpr int kWarps = G <= 4 ? 8 : 4;
   static constexpr int kBlocks = kTile / 16 / kWarps;  // 16-row blocks of a warp
-  static constexpr float kTileUs = D == 128 ? (G <= 4 ? 0.66f : 0.76f) : (G <= 4 ? 0.47f : 0.63f);
-  static constexpr float kSegmentUs = 0.4f + 0.35f * G;
-  // the persistent pass: its chunks are about an eighth of a CTA's share, 3 to 16 a CTA; one warp
-  // merges a group's, head by head, and those past a group's length are claimed all the same
-  static float general_us(const AttendArgs &, const CallShape &s, float mean) {
-    const float total = mean * (float)s.groups * (float)s.tiles, share = total / 152.f;
-    const float chunk = fmaxf(share / fminf(16.f, fmaxf(3.f, share / 8.f)), 1.f);
-    const float per_group = (float)s.tiles / chunk;
-    return 12.f + 1.03f * s.mem_us(total) + 0.07f * (float)G * per_group +
-           0.7f / 152.f * (1.f - mean) * (float)s.groups * per_group;
-  }
   static constexpr int kFoldUnits = 1;
   static constexpr bool kEarlyUnits = true;
   // No flush: o takes one rounded addition per 16 rows (kFresh in lg_mma_tile.cuh), l, u and sigma
@@ -54,10 +43,8 @@ struct Pass<__nv_bfloat16, D, G> {
 
 // The limits of its tables and integers: the batch (two sequences a lane), the groups (a group
 // number times a cluster number in a float's 24 bits) and the tiles (a cluster's tiles times a CTA
-// number in 24 bits).  Within them cluster_shape compares its time with the persistent pass's.
-// Both, same box, us: 1 sequence of 1024 rows 7.3, 12.0; 1 of 131072, 8 heads a group, 109, 170; 2
-// of 131071 157, 200; 8 of 4096 26.6, 34.3; 64 ragged up to 16384 220, 245; 32 layers of 8 x 4096
-// at once 590, 594; 8 layers of 16 x 32704 2310, 2324.
+// number in 24 bits).  Within them attend_choose (lg_attend_rule.cuh) compares it with the general
+// pass.
 bool attend_cluster_takes(const AttendArgs &a, int tile_rows, int64_t rows_total) {
   const int64_t groups = (int64_t)a.n_layers * a.batch * a.H_kv;
   const int64_t tiles = groups * ((a.max_len + tile_rows - 1) / tile_rows);
@@ -65,7 +52,7 @@ bool attend_cluster_takes(const AttendArgs &a, int tile_rows, int64_t rows_total
          rows_total < (int64_t)1 << 31;
 }
 
-cudaError_t launch_attend_cluster(const AttendArgs &a, int d, int g, int64_t rows_total,
+cudaError_t launch_attend_cluster(AttendArgs &a, int d, int g, int64_t rows_total,
                                   bool *general, cudaStream_t s) {
   return launch_cluster<__nv_bfloat16>(a, d, g, rows_total, general, s);
 }

@@ -32,6 +32,7 @@
 
 #include <atomic>
 
+#include "lg_attend_rule.cuh"
 #include "lg_common.cuh"
 #include "lg_internal.h"
 #include "lg_mma_tile.cuh"
@@ -41,22 +42,10 @@ namespace lg {
 namespace {
 
 constexpr int kClusterSeqs = 64;  // batch at most (two sequences a lane in the prologue's scan)
-constexpr int kMaxCluster = 8;    // CTAs of a cluster at most (portable)
-
-// a call as the choice of its pass sees it (cluster_shape below)
-struct CallShape {
-  int groups, tiles;          // (layer, sequence, kv-head) groups; tiles of a longest one
-  float tile_bytes, tile_us;  // a tile's bytes, one CTA's time for it
-  float seg_us;               // a segment's fold
-  // a CTA's last segments: where it has several tiles of a group, of which it shares some
-  float ends_us(int c) const { return tiles < 8 ? 0.f : seg_us * (c > 1 ? 2.f : 1.f); }
-  float mem_us(float n_tiles) const { return n_tiles * tile_bytes / 7.3e6f; }
-};
 
 // What differs between the element types: the tile and the ring, and a consumer warp's work.
 //   kTile rows a tile, kBoxes boxes of kBoxCols columns per tensor, kStages stages in the ring
-//   kWarps consumer warps, which share every tile; kTileUs one CTA's time for a tile, kSegmentUs
-//   for a segment's fold; general_us(call, its shape, mean length): the general pass's time
+//   kWarps consumer warps, which share every tile
 //   begin(the query rows, whether it is the segment's first tile), update(a tile), join() (the
 //   lanes' sums) and store(to, or added to, a row of D + 4 floats per head: o, then {M, l, u,
 //   sigma}); with kFlushTiles > 0 a segment's sums are stored every so many tiles
@@ -228,6 +217,18 @@ __device__ __forceinline__ void finish(const AttendArgs &a, int64_t head, int e,
   }
 }
 
+// whether the general pass is the faster for a call's lengths: the longest of each lane's two
+// sequences, tiles of all of them (not inlined: few calls ask, and the others' way to their first
+// copies stays as short as it was)
+template <typename T, int D, int G>
+__device__ __noinline__ bool leave_to_general(int groups, int rows, int batch, int total,
+                                              int chunk_rows, int max_chunks, int sms, int ctas,
+                                              int n_cl) {
+  const CallShape s = call_shape({Elem<T>::kDtype == LG_BF16, D, G, Pass<T, D, G>::kTile}, groups,
+                                 __reduce_max_sync(0xffffffffu, rows), chunk_rows, max_chunks, sms);
+  return general_gains_us(s, batch, total, total == s.tiles * batch, ctas, n_cl) > 0.f;
+}
+
 }  // namespace
 
 template <typename T, int D, int G>
@@ -244,7 +245,8 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
   __shared__ __align__(8) uint64_t recv_bar[2];  // a slot's pieces have arrived
   __shared__ __align__(8) uint64_t q_full[2], q_empty[2];  // query rows of segment i in buffer i & 1
   __shared__ int s_len[kClusterSeqs], s_pre[kClusterSeqs], s_off[kClusterSeqs];
-  __shared__ int s_total, s_c0, s_c1, s_empty, s_skip;
+  __shared__ int s_total, s_c0, s_c1, s_skip;
+  __shared__ int s_todo;  // besides the tiles: 1 empty sequences, 2 the general pass's counters
   __shared__ int s_stop;  // bit 0: the status was set before this call, bit 1: a wait ran out
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -468,11 +470,22 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
       if (u0 < u1) g = ts.find(u0);
     }
     any_empty = __any_sync(0xffffffffu, any_empty);
+    bool general = false;
+    if (a.gate) {
+      // the general pass follows: one of the two runs, by the lengths (the same in every CTA)
+      general = leave_to_general<T, D, G>(groups, max(n[0], n[1]), a.batch, ts.total, a.chunk_rows,
+                                          a.max_chunks, a.sms, ctas, n_cl);
+      if (!general && blockIdx.x == 0 && lane == 0) *a.gate = -1;
+      if (general) {
+        c0 = c1 = u0 = u1 = 0;
+        hit = false;
+      }
+    }
     if (lane == 0) {
       s_total = ts.total;
       s_c0 = c0;
       s_c1 = c1;
-      s_empty = any_empty && !bad;
+      s_todo = bad ? 0 : general ? 2 : any_empty;
       s_skip = hit ? 0 : guess_tiles;
       s_stop = bad != 0;
     }
@@ -566,7 +579,13 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
   const int u0 = first_tile(rank), u1 = first_tile(rank + 1);
   TileGroup g = {};
   if (u0 < u1) g = ts.find(u0);
-  if (s_empty) {
+  if (s_todo == 2) {
+    // the call is left to the general pass: its counters (the gate is their first) to zero and the
+    // direction word flipped, as zero_counters_kernel does
+    const int words = 1 + a.n_layers * a.batch * a.H_kv;
+    for (int i = blockIdx.x * kWarps * 32 + threadIdx.x; i <= words; i += gridDim.x * kWarps * 32)
+      a.counter[i] = i < words ? 0 : a.counter[i] ^ 1;
+  } else if (s_todo == 1) {
     // empty sequences: zero output, m = -inf, l = H = S = 0
     for (int i = blockIdx.x; i < a.n_layers * a.batch * a.H_kv; i += gridDim.x) {
       const int lb = i / a.H_kv;
@@ -742,9 +761,6 @@ attend_cluster_kernel(const __grid_constant__ CUtensorMap tmK,
 namespace {
 
 constexpr int kMaxDev = 64;
-constexpr int kSizes[] = {8, 6, 4, 2, 1};  // cluster sizes used (5 and 7 fit no better than 4 and 6
-                                           // beside the GPU's clusters of SMs)
-constexpr int kNumSizes = sizeof(kSizes) / sizeof(kSizes[0]);
 
 template <typename T, int D, int G>
 struct ClusterLaunch {
@@ -787,103 +803,37 @@ cudaError_t resident_clusters(int (&n)[kNumSizes]) {
   return cudaSuccess;
 }
 
-// What a call is estimated to take (us), by cluster size and by the general pass.  Only max_len is
-// known of the lengths, and how many rows the cache has for them: `fill` = S_total / (batch *
-// max_len) at most 1.  A batch with fill above 0.9 may have equal lengths or any others, so it is
-// judged as equal ones and, half as much, as ragged ones of 0.35 of the longest on average (as
-// log-uniform ones are); below, as ragged ones of fill on average.
-constexpr float kRagged = 0.35f, kFull = 0.9f, kCallUs = 5.f;
-
-// K clusters of c CTAs.  Equal lengths: each takes groups / K groups and then groups mod K of them
-// one more; either phase is bound by the memory or by the CTAs.  Ragged ones: the clusters' runs
-// are even but for a part of a longest group on one cluster, and no group has more than c CTAs.
-// Larger clusters stream a little better (about a percent per halving on passes of half a
-// millisecond).
-inline float equal_us(const CallShape &s, int c, int k) {
-  const int q = s.groups / k, r = s.groups % k;
-  const float cta = (float)s.tiles / (float)c * s.tile_us;  // a group's tiles on one of its CTAs
-  float us = fmaxf(s.mem_us((float)k * (float)q * (float)s.tiles),
-                   (float)q * cta + s.seg_us * (float)(q - 1) / (float)c);
-  if (r) us += fmaxf(s.mem_us((float)r * (float)s.tiles), cta + s.seg_us / (float)c);
-  return us + s.ends_us(c);
-}
-inline float ragged_us(const CallShape &s, int c, int k, float mean) {
-  const float cta = (float)s.tiles / (float)c * s.tile_us;
-  const float total = mean * (float)s.groups * (float)s.tiles;
-  const float even = (total * s.tile_us + (float)s.groups * s.seg_us) / (float)(k * c);
-  return fmaxf(fmaxf(s.mem_us(total), even) + 0.35f * cta, cta) + s.ends_us(c);
-}
-
-// Cluster size and count, and whether the general pass (general(mean): its estimate for lengths of
-// that mean share of the longest) is expected to be faster: with few long groups, which have at
-// most 8 CTAs each here and the whole GPU there, and, of fp32 calls, with 5 to 8 heads a group,
-// bound by a CTA's arithmetic.  Smaller clusters fill the GPU better (152 SMs hold 15, 23, 36, 76,
-// 152 clusters of 8, 6, 4, 2, 1), larger ones split a group further.
-// Measured per call (append and attention, one layer, us, 128 elements; sizes 8 / 6 / 4 / 2 / 1,
-// general): bf16, equal lengths, 1 sequence of 131071 rows, 2 kv-heads, 1 head a group 74 / 97 /
-// 142 / 277 / 540, 45; the same with 8 heads 102 / 132 / 192 / 374 / 727, 136; 2 of 66791, 8 kv-heads
-// 107 / 80 / 91 / 150 / 284, 90; ragged, 8 up to 124643, 2 kv-heads 84 / 101 / 140 / 264 / 522, 73;
-// the same with 7 heads 103 / 132 / 189 / 367 / 717, 109; 48 up to 17000, 4 kv-heads 87 / 88 / 91 /
-// 99 / 106, 99.  fp32, 6 of 9036, 8 kv-heads, 4 heads 88 / 93 / 93 / 88 / 165, 109; the same with 8
-// heads 158 / 158 / 159 / 158 / 307, 134; ragged, 11 up to 88235, 2 kv-heads, 1 head 134 / 158 / 211
-// / 394 / 773, 173; the same with 7 heads 380 / 505 / 751 / 1488 / 2965, 232.  Over 130 such calls
-// the choice is 2 % off the best one's time on average; over 240 random ones none is slower than
-// the general pass.
-struct ClusterShape {
-  int ctas, clusters;
-  bool general;
-};
-template <typename General>
-ClusterShape cluster_shape(const CallShape &s, int batch, float fill, General general,
-                           const int (&resident)[kNumSizes]) {
-  const float w_equal = batch == 1 || fill > kFull ? 1.f : 0.f;
-  const float w_ragged = batch == 1 ? 0.f : (w_equal > 0.f ? 0.5f : 1.f);
-  const float mean = w_equal > 0.f ? kRagged : fill;
-  ClusterShape best = {1, 1, false};
-  float best_us = 0.f;
-  for (int i = 0; i < kNumSizes; ++i) {
-    const int c = kSizes[i], k = resident[i] < s.groups ? resident[i] : s.groups;
-    const float wide = 1.f + 0.0125f * log2f((float)kMaxCluster / (float)c);
-    const float us = w_equal * (kCallUs + wide * equal_us(s, c, k)) +
-                     w_ragged * (kCallUs + wide * ragged_us(s, c, k, mean));
-    if (best_us == 0.f || us < best_us) {
-      best_us = us;
-      best = {c, k, false};
-    }
-  }
-  best.general = w_equal * general(1.f) + w_ragged * general(mean) < 1.05f * best_us;
-  return best;
+template <typename T, int D, int G>
+constexpr PassKind pass_kind() {
+  return {Elem<T>::kDtype == LG_BF16, D, G, Pass<T, D, G>::kTile};
 }
 
 template <typename T, int D, int G>
-cudaError_t launch_cluster_typed(const AttendArgs &a, int64_t rows_total, bool *general,
+cudaError_t launch_cluster_typed(AttendArgs &a, int64_t rows_total, bool *general,
                                  cudaStream_t s) {
-  using P = Pass<T, D, G>;
   int resident[kNumSizes];
   LG_TRY((resident_clusters<T, D, G>(resident)));
-  constexpr int rows = P::kTile;
-  const int tiles = (a.max_len + rows - 1) / rows;
-  const CallShape shape = {a.n_layers * a.batch * a.H_kv, tiles,
-                           (float)ClusterCfg<T, D, G>::kTileBytes, P::kTileUs,
-                           tiles < 8 ? 1.f : P::kSegmentUs};
-  const float fill = fminf(1.f, (float)a.S_total / ((float)a.batch * (float)a.max_len));
-  const ClusterShape sh = cluster_shape(
-      shape, a.batch, fill, [&](float mean) { return P::general_us(a, shape, mean); }, resident);
-  *general = sh.general;
-  if (sh.general) return cudaSuccess;
+  a.sms = resident[kNumSizes - 1];  // one CTA an SM
+  const CallShape shape = call_shape(pass_kind<T, D, G>(), a.n_layers * a.batch * a.H_kv, a.max_len,
+                                     a.chunk_rows, a.max_chunks, a.sms);
+  const AttendChoice ch = attend_choose(
+      shape, a.batch, fminf(1.f, (float)a.S_total / ((float)a.batch * (float)a.max_len)), resident);
+  *general = ch.pass != kClusterPass;
+  if (ch.pass == kGeneralPass) return cudaSuccess;
+  if (ch.pass == kEitherPass) a.gate = a.counter;
   CUtensorMap mk, mv;
-  if (!make_kv_map(&mk, a.K, Elem<T>::kDtype, D, rows_total, rows) ||
-      !make_kv_map(&mv, a.V, Elem<T>::kDtype, D, rows_total, rows))
+  if (!make_kv_map(&mk, a.K, Elem<T>::kDtype, D, rows_total, Pass<T, D, G>::kTile) ||
+      !make_kv_map(&mv, a.V, Elem<T>::kDtype, D, rows_total, Pass<T, D, G>::kTile))
     return cudaErrorInvalidValue;
   auto kern = attend_cluster_kernel<T, D, G>;
   LG_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               ClusterCfg<T, D, G>::kSmem));
-  ClusterLaunch<T, D, G> l(sh.clusters, sh.ctas, s);
-  return cudaLaunchKernelEx(&l.cfg, kern, mk, mv, a, sh.ctas, sh.clusters, (int)rows_total);
+  ClusterLaunch<T, D, G> l(ch.clusters, ch.ctas, s);
+  return cudaLaunchKernelEx(&l.cfg, kern, mk, mv, a, ch.ctas, ch.clusters, (int)rows_total);
 }
 
 template <typename T, int D>
-cudaError_t launch_cluster_d(const AttendArgs &a, int g, int64_t rows_total, bool *general,
+cudaError_t launch_cluster_d(AttendArgs &a, int g, int64_t rows_total, bool *general,
                              cudaStream_t s) {
   switch (g) {
     case 1: return launch_cluster_typed<T, D, 1>(a, rows_total, general, s);
@@ -898,9 +848,10 @@ cudaError_t launch_cluster_d(const AttendArgs &a, int g, int64_t rows_total, boo
   return cudaErrorInvalidValue;
 }
 
-// the pass over a cache of rows_total rows of T, or *general set and nothing launched
+// the pass over a cache of rows_total rows of T; *general set: the general pass is to be launched,
+// alone, or after it with a.gate set
 template <typename T>
-cudaError_t launch_cluster(const AttendArgs &a, int d, int g, int64_t rows_total, bool *general,
+cudaError_t launch_cluster(AttendArgs &a, int d, int g, int64_t rows_total, bool *general,
                            cudaStream_t s) {
   if (d == 128) return launch_cluster_d<T, 128>(a, g, rows_total, general, s);
   if (d == 64) return launch_cluster_d<T, 64>(a, g, rows_total, general, s);

@@ -26,16 +26,6 @@ struct Pass<float, D, G> {
   static constexpr int kWarps = 8;
   static constexpr int kFoldUnits = 4;
   static constexpr bool kEarlyUnits = false;  // (six registers that the tiles' loop lacks)
-  static constexpr float kTileUs = D == 128 ? (G <= 2 ? 0.66f : G <= 4 ? 1.13f : 1.07f)
-                                            : (G <= 2 ? 0.38f : G <= 4 ? 0.62f : 0.69f);
-  static constexpr float kSegmentUs = 1.f;
-  // the chunk kernel (more arithmetic the more heads) and its combine, which walks a group's
-  // chunks one by one (their partials still in L2 after a short pass)
-  static float general_us(const AttendArgs &a, const CallShape &s, float mean) {
-    const float mem = s.mem_us(mean * (float)s.groups * (float)s.tiles);
-    return 12.f + (8.f + 3.f * G) * fminf(1.f, mem / 30.f) + (1.03f + 0.045f * G) * mem +
-           (mem < 15.f ? 0.23f : 0.42f) * (float)a.max_len / (float)a.chunk_rows;
-  }
   static constexpr int kBox = kTile * 128;       // bytes of a box
   static constexpr int kEpl = G <= 2 ? 16 : (G <= 4 ? 8 : 4);  // elements of a lane
   static constexpr int kCh = kEpl / 4;           // 16-byte chunks of a lane
@@ -266,7 +256,7 @@ struct Pass<float, D, G> {
 
 int cluster_f32_tile_rows() { return kF32TileMin; }
 
-cudaError_t launch_attend_cluster_f32(const AttendArgs &a, int d, int g, int64_t rows_total,
+cudaError_t launch_attend_cluster_f32(AttendArgs &a, int d, int g, int64_t rows_total,
                                       bool *general, cudaStream_t s) {
   return launch_cluster<float>(a, d, g, rows_total, general, s);
 }

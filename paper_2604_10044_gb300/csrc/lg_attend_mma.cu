@@ -295,6 +295,7 @@ attend_mma_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
   }
   pdl_enter();  // the tensormap prefetch above reads only the kernel's parameters
+  if (a.gate && *(volatile int *)a.gate < 0) return;  // the cluster pass has done the call
   if (threadIdx.x == 0) {
     s_bad = status_bad(a.status);
     s_rev = a.counter[1 + a.n_layers * a.batch * a.H_kv] & 1;
@@ -695,9 +696,8 @@ cudaError_t launch_attend_mma_partial(const AttendArgs &a, int d, int g, int64_t
   const int total = a.n_layers * a.batch * a.H_kv * a.max_chunks;
   const int grid = total < sms ? total : sms;
   if (!a.counter) return cudaErrorInvalidValue;
-  const size_t counters = (size_t)(1 + (int64_t)a.n_layers * a.batch * a.H_kv) * sizeof(int);
-  {
-    const int n = (int)(counters / sizeof(int));
+  if (!a.gate) {  // (the cluster pass in front of this one clears them itself)
+    const int n = 1 + a.n_layers * a.batch * a.H_kv;
     const int blocks = (n + 255) / 256 < sms ? (n + 255) / 256 : sms;
     if ((e = launch_pdl(zero_counters_kernel, blocks, 256, 0, s, a.counter, n)) != cudaSuccess)
       return e;

@@ -27,6 +27,10 @@ struct AttendArgs {
   int max_len;
   int suffix_w;
   float qscale;            // softmax scale * log2(e)
+  int *gate;               // nullable, else `counter`: both passes are launched, and the cluster
+                           // pass leaves -1 in its first word when it has done the call, or clears
+                           // the counters for the general pass after it
+  int sms;                 // of the GPU (cluster pass)
 };
 
 int attend_tile_rows(int dtype, int d);
@@ -37,13 +41,13 @@ int mma_tile_rows();
 cudaError_t launch_attend_mma_partial(const AttendArgs &a, int d, int g, int64_t rows_total,
                                       cudaStream_t s);
 
-// the cluster pass (lg_attend_cluster.cuh): whether it can take a call, and the call (*general set
-// and nothing launched where the pass past its limits is expected to be faster)
+// the cluster pass (lg_attend_cluster.cuh): whether it can take a call, and the call (*general set:
+// the general pass is to be launched, instead or, with a.gate set, after it)
 bool attend_cluster_takes(const AttendArgs &a, int tile_rows, int64_t rows_total);
-cudaError_t launch_attend_cluster(const AttendArgs &a, int d, int g, int64_t rows_total,
+cudaError_t launch_attend_cluster(AttendArgs &a, int d, int g, int64_t rows_total,
                                   bool *general, cudaStream_t s);
 int cluster_f32_tile_rows();
-cudaError_t launch_attend_cluster_f32(const AttendArgs &a, int d, int g, int64_t rows_total,
+cudaError_t launch_attend_cluster_f32(AttendArgs &a, int d, int g, int64_t rows_total,
                                       bool *general, cudaStream_t s);
 
 // guard kernels (lg_guard.cu)

@@ -100,7 +100,8 @@ def test_cluster_bookkeeping():
     if shutil.which("g++") is None:
         pytest.skip("needs g++")
     text = open(SRC).read()
-    assert re.search(r"kClusterSeqs = 64;", text) and re.search(r"kMaxCluster = 8;", text)
+    assert re.search(r"kClusterSeqs = 64;", text)
+    assert "kMaxCluster = 8;" in open(SRC.replace("cluster", "rule")).read()
     assert "groups <= 1 << 16 && tiles < 1 << 20" in open(SRC[:-1]).read()  # the ranges checked here
     code = "\n".join([_block(text, r"^__device__ __forceinline__ int quick_div\("),
                       _block(text, r"^struct TileGroup \{"), _block(text, r"^struct TileSpace \{"),

@@ -17,9 +17,9 @@ pytestmark = pytest.mark.gpu
 LIMIT = 64  # kClusterSeqs in csrc/lg_attend_cluster.cuh
 
 
-def _run(k, v, q, lens, layer0, n_layers, suffix_w, h2o, pad):
+def _run(k, v, q, lens, layer0, n_layers, suffix_w, h2o, pad, ran="cluster"):
     """out, stats (and scores) of layers [layer0, layer0 + n_layers) over cache rows k, v
-    [L][H_kv][S][d]; pad: empty sequences after the real ones"""
+    [L][H_kv][S][d]; pad: empty sequences after the real ones; ran: the pass that the call is to run"""
     L, H_kv, S, d = k.shape
     b, H_q = len(lens), q.shape[2]
     cap = np.concatenate([np.asarray(lens) + 1, np.ones(pad, np.int64)]).astype(np.int32)
@@ -34,11 +34,31 @@ def _run(k, v, q, lens, layer0, n_layers, suffix_w, h2o, pad):
     qq = torch.cat([q, torch.ones((n_layers, pad, H_q, d), dtype=q.dtype, device=q.device)], 1)
     out = torch.full((n_layers, b + pad, H_q, d), 7.0, dtype=k.dtype, device=k.device)
     st = torch.full((n_layers, b + pad, H_q, 4), 7.0, dtype=torch.float32, device=k.device)
+    ws = _Workspace(c, H_q, n_layers, int(cap.max()), g.ws)
     lg.lg_decode_attend(c, layer0, n_layers, qq.contiguous(), H_q, g.scale, out, st, suffix_w,
                         1 if h2o else 0, int(cap.max()), g.ws)
     assert lg.lg_read_device_status(c) == 0
+    if sum(lens):
+        assert ws.ran() == ran
     sc = c.h2o[layer0:layer0 + n_layers, :, :S].clone() if h2o else None
     return out[:, :b], st[:, :b], sc, off
+
+
+class _Workspace:
+    """Which pass a call ran, from what it left in its workspace: the general passes write split-K
+    partials, its first part, the cluster pass none."""
+
+    MARK = -12345
+
+    def __init__(self, cache, H_q, n_layers, max_len, ws):
+        counters = (2 + n_layers * cache.batch * cache.H_kv) * 4
+        self.partials = lg.lg_workspace_size(cache, H_q, n_layers, max_len) - -(-counters // 256) * 256
+        self.ws = ws.view(torch.int32)
+        self.ws.fill_(self.MARK)
+
+    def ran(self):
+        part = self.ws[:self.partials // 4]
+        return "cluster" if bool((part == self.MARK).all()) else "general"
 
 
 def _exact(k, v, q, lens, off, layer0, n_layers, suffix_w):
@@ -102,7 +122,7 @@ def test_cluster_pass(cuda, lens, H_kv, G, d, nl, dtype, h2o):
     # the parity tests' bounds: bf16 output rounding, fp32 sums
     _close(got, want, *((2e-2, 1e-3) if dtype == "bf16" else (1e-4, 1e-5)), "out")
     _close(st, ws, 1e-4, 1e-6, "stats")
-    gen, gst, gsc, _ = _run(k, v, q, lens, 1, nl, 50, h2o, LIMIT + 1 - len(lens))
+    gen, gst, gsc, _ = _run(k, v, q, lens, 1, nl, 50, h2o, LIMIT + 1 - len(lens), "general")
     # bf16: both within 2^-8 of the same value, so they differ by one step at most
     _close(got, gen, 2.0 ** -7 if dtype == "bf16" else 2e-5, 1e-5, "out against the general pass")
     _close(st, gst, 2e-5, 1e-6, "stats against the general pass")
@@ -201,21 +221,24 @@ def test_long_bf16_segments_keep_their_precision(cuda, lens, H_kv, G, d):
         assert ((st[..., i].double() - ws[..., i]).norm() / ws[..., i].norm()).item() < 6.5e-7, i
 
 
-@pytest.mark.parametrize("lens,H_kv,G,d,dtype,h2o", [
+@pytest.mark.parametrize("lens,H_kv,G,d,dtype,h2o,ran", [
     # few long groups, with 8 CTAs each in the cluster pass: the general pass is the faster
-    ([131071], 2, 1, 128, "bf16", False), ([60000, 500, 800, 3], 2, 1, 128, "bf16", True),
+    ([131071], 2, 1, 128, "bf16", False, "general"),
+    ([60000, 500, 800, 3], 2, 1, 128, "bf16", True, "general"),
     # a CTA's arithmetic bounds the cluster pass over fp32 rows with many heads a group
-    ([9036] * 6, 8, 6, 64, "f32", False), ([20000, 700, 0, 5000], 2, 8, 128, "f32", True),
+    ([9036] * 6, 8, 6, 64, "f32", False, "general"),
+    ([20000, 700, 0, 5000], 2, 8, 128, "f32", True, "general"),
     # beside them, calls that the cluster pass keeps
-    ([9036] * 6, 8, 6, 64, "bf16", False), ([20000, 700, 0, 5000], 2, 1, 128, "f32", True)])
-def test_either_side_of_the_choice(cuda, lens, H_kv, G, d, dtype, h2o):
+    ([9036] * 6, 8, 6, 64, "bf16", False, "cluster"),
+    ([20000, 700, 0, 5000], 2, 1, 128, "f32", True, "cluster")])
+def test_either_side_of_the_choice(cuda, lens, H_kv, G, d, dtype, h2o, ran):
     g = torch.Generator(device=cuda)
     g.manual_seed(sum(lens) + G)
     tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
     S = int(sum(lens)) + len(lens)
     k, v = (torch.randn((1, H_kv, S, d), generator=g, device=cuda).to(tdt) for _ in range(2))
     q = torch.randn((1, len(lens), H_kv * G, d), generator=g, device=cuda).to(tdt)
-    got, st, sc, off = _run(k, v, q, lens, 0, 1, 64, h2o, 0)
+    got, st, sc, off = _run(k, v, q, lens, 0, 1, 64, h2o, 0, ran)
     want, ws = _exact(k, v, q, lens, off, 0, 1, 64)
     # the parity tests' bounds: bf16 output rounding, fp32 sums
     _close(got, want, *((2e-2, 1e-3) if dtype == "bf16" else (1e-4, 1e-5)), "out")
@@ -223,3 +246,58 @@ def test_either_side_of_the_choice(cuda, lens, H_kv, G, d, dtype, h2o):
     if h2o:
         total, all_ = sc.double().sum(-1), float(G * sum(n > 0 for n in lens))
         assert torch.allclose(total, torch.full_like(total, all_), rtol=1e-5)
+
+
+@pytest.mark.parametrize("h2o", [False, True])
+@pytest.mark.parametrize("dtype,b,slot,H_kv,G,d,nl", [
+    ("bf16", 8, 36000, 4, 6, 64, 1), ("bf16", 8, 46500, 2, 1, 128, 1), ("f32", 4, 15000, 2, 6, 64, 2),
+    ("f32", 4, 30001, 1, 5, 128, 1)])
+def test_lengths_in_equal_slots_choose_the_pass(cuda, dtype, b, slot, H_kv, G, d, nl, h2o):
+    """Few long groups in equal slots: the call gets both passes, of which the one that is the
+    faster for the lengths runs, here in one graph whose lengths change from replay to replay (one
+    workspace, so that each pass finds what the other left)."""
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    gen = torch.Generator(device=cuda)
+    gen.manual_seed(slot)
+    off = np.arange(b, dtype=np.int64) * slot
+    k, v = (torch.randn((nl, H_kv, b * slot, d), generator=gen, device=cuda).to(tdt)
+            for _ in range(2))
+    q = torch.randn((nl, b, H_kv * G, d), generator=gen, device=cuda).to(tdt)
+    c = lg.Cache(nl, H_kv, d, dtype, off, [slot] * b, [slot - 1] * b, cuda,
+                 "h2o" if h2o else "loopguard", k, v)
+    g = lg.Guard(c, H_kv * G, policy="h2o" if h2o else "loopguard", n_layers_per_call=nl)
+    out = torch.zeros((nl, b, H_kv * G, d), dtype=tdt, device=cuda)
+    st = torch.zeros((nl, b, H_kv * G, 4), device=cuda)
+    side = torch.cuda.Stream(device=cuda)
+    ws = _Workspace(c, H_kv * G, nl, slot, g.ws)
+
+    def run():
+        lg.lg_decode_attend(c, 0, nl, q, H_kv * G, g.scale, out, st, 64, int(h2o), slot, g.ws)
+
+    with torch.cuda.stream(side):
+        run()
+        side.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side, capture_error_mode="thread_local"):
+            run()
+        for lens, ran in [([slot - 1] * b, "cluster"), ([slot - 1] + [100] * (b - 1), "general"),
+                          ([0, 1] + [100] * (b - 3) + [slot - 1], "general"),
+                          ([slot // 2] * b, "cluster"), ([0, slot] + [3] * (b - 2), "general"),
+                          ([0] * b, "none"), ([100] * (b - 1) + [slot], "general")]:
+            ws.ws[:ws.partials // 4].fill_(ws.MARK)
+            out.fill_(7.0)
+            st.fill_(7.0)
+            c.len.copy_(torch.as_tensor(np.asarray(lens, np.int32), device=cuda))
+            if h2o:
+                c.h2o.zero_()
+            graph.replay()
+            side.synchronize()
+            assert lg.lg_read_device_status(c) == 0
+            if ran != "none":
+                assert ws.ran() == ran, lens
+            want, wst = _exact(k, v, q, lens, off, 0, nl, 64)
+            _close(out, want, *((2e-2, 1e-3) if dtype == "bf16" else (1e-4, 1e-5)), "out")
+            _close(st, wst, 1e-4, 1e-6, "stats")
+            if h2o:
+                total, all_ = c.h2o.double().sum(-1), float(G * sum(n > 0 for n in lens))
+                assert torch.allclose(total, torch.full_like(total, all_), rtol=1e-5)
