@@ -184,11 +184,14 @@ LG_API lg_status lg_sketch_build(const lg_cache *c, const lg_guard_params *p, in
    stats: device [n_layers][batch][H_q][4] fp32.  Query head h reads kv-head h / (H_q/H_kv).
    accumulate_h2o: also add sum over the GQA group of a_i to h2o[l][kvh][slot] (c->h2o).
    max_len: host bound on every len[b] (sizes the grid; a longer sequence is an error).
-   ws: device workspace of at least lg_workspace_size(...) bytes, 256-byte aligned.  Batches of up
-   to 64 sequences use only its logits and {M, l} part (accumulate_h2o); bf16 calls with more
-   walk the cache in alternating directions from call to call (one word of ws keeps the
-   direction), so that a call starts on the rows the previous call read last, which may still be
-   in L2; no result depends on the direction. */
+   ws: device workspace of at least lg_workspace_size(...) bytes, 256-byte aligned, with any
+   contents.  A call may write all of it: which kernels it runs, and what they keep in ws (split-K
+   partials, counters, the logits of accumulate_h2o), is the library's choice by the call's sizes
+   and lengths and by the GPU.  So calls that may overlap on the GPU need a workspace each, and
+   nothing else survives in one.  Calls one after another may share one; those that run the
+   persistent bf16 kernel then walk the cache in alternating directions (one word of ws keeps the
+   direction), so that a call starts on the rows the previous one read last, which may still be in
+   L2; no result depends on the direction. */
 LG_API lg_status lg_decode_attend(const lg_cache *c, int layer0, int n_layers, const void *q, int H_q,
                            float scale, void *out, float *stats, int suffix_w,
                            int accumulate_h2o, int max_len, void *ws, size_t ws_bytes,

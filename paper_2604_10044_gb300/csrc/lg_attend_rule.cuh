@@ -4,8 +4,11 @@
 //
 // The host sees sizes only: max_len bounds the lengths, and S_total says how many rows the cache
 // has for them.  Sequences kept in equal slots look like equal lengths, whatever they are.  Most
-// calls are no slower by clusters for any lengths; for the others the host launches both, and the
-// cluster pass, which reads the lengths anyway, decides (attend_choose below).
+// calls lose little by clusters for any lengths; for the others the host launches both, and the
+// cluster pass, which reads the lengths anyway, decides (attend_choose below).  Eight slots of
+// 131072 rows, 2 kv-heads, 4 heads a group, bf16, us a call (the general pass alone / clusters alone
+// / both): all full 177 / 153 / 157, one full and seven of 300 rows 57 / 121 / 60; 16 slots of 56396
+// rows, 1 head, fp32, the same 303 / 254 / 260 and 76 / 138 / 83.
 #pragma once
 #include <math.h>
 
