@@ -446,23 +446,11 @@ class GpuBench:
         if ev:
             ev[3].record(self.stream)
 
-    # launches of this repository's kernels per step (harness + path)
     def launches_per_step(self):
-        calls = math.ceil(self.w.L / self.nl)
-        # per call past the cluster pass's limits: the counter reset and the persistent pass, or on
-        # an fp32 cache a partial pass and a merge; H2O adds the score update.  A call that the
-        # cluster pass takes is one kernel instead of two (attend_cluster_takes in
-        # csrc/lg_attend_cluster.cu): there this is an upper bound, which the line says.
-        attend = 2 + (1 if self.policy == "h2o" else 0)
-        path = 1 + 1 + attend * calls               # begin, append (+sketch), attend
-        harness = 1                                 # the step's inputs
-        if self.policy in ("h2o", "streaming"):     # evict, lengths
-            path += 2
-        elif self.policy == "loopguard" and self.detector == "token":
-            path += 2                               # token monitor + keep, compact
-        elif self.policy == "loopguard":
-            path += 2                               # detect + keep, compact
-        return path, harness
+        """kernels of one step, counted in a capture of it (an attention call launches one to three,
+        by the pass it takes; everything a step launches is this repository's): (path, harness)"""
+        harness = kernels_launched(self.stream, lambda: self.select_inputs(0))
+        return kernels_launched(self.stream, lambda: self.step(0)) - harness, harness
 
     def replay_log(self, K, fresh=False):
         """replay the timed trajectory (the decisions are deterministic, so they are the
@@ -555,6 +543,33 @@ def code_only(src):
             out.append(c)
             i += 1
     return " ".join("".join(out).split())
+
+
+def kernels_launched(stream, call):
+    """kernels that call() launches on the stream: it is captured, not run"""
+    import ctypes
+    cu = ctypes.CDLL("libcuda.so.1")
+
+    def ok(rc):
+        if rc != 0:
+            raise RuntimeError("CUDA driver error %d while counting launches" % rc)
+
+    st, graph, n = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t(0)
+    ok(cu.cuStreamBeginCapture_v2(st, 1))             # of this thread's calls
+    try:
+        call()
+    finally:
+        rc = cu.cuStreamEndCapture(st, ctypes.byref(graph))
+    ok(rc)
+    ok(cu.cuGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    ok(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    kernels, kind = 0, ctypes.c_int(0)
+    for node in nodes:
+        ok(cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
+        kernels += kind.value == 0                    # CU_GRAPH_NODE_TYPE_KERNEL
+    ok(cu.cuGraphDestroy(graph))
+    return kernels
 
 
 def source_hash():
@@ -783,11 +798,7 @@ def run_gpu(args, ws, rank, local):
             "guard_ms_per_step": round(sum(guard_ms) / len(sampled), 4)},
         "eager_ms_per_step": round(eager_ms / K, 4) if eager_ms is not None else None,
         "gpu_launches": (path_l + harness_l) * K,
-        "gpu_launches_detail": {
-            "path_per_step": path_l, "harness_per_step": harness_l,
-            "note": "two kernels an attention call, as past the cluster pass's limits (more than "
-                    "64 sequences, or 2^20 tiles as the bandwidth sweep's); a call within them is "
-                    "one kernel, so that the steps launched are fewer by their attention calls"},
+        "gpu_launches_detail": {"path_per_step": path_l, "harness_per_step": harness_l},
         "clocks": clk,
     }
     if e2e:

@@ -43,8 +43,22 @@ def test_bench_line_keeps_the_contract():
     assert e["value"] > 0 and e["h2d_bytes_per_step"] > 0 and e["d2h_bytes_per_step"] > 0
     c = d["clocks"]
     assert c["sm_mhz"] > 0 and c["sm_max_mhz"] > 0 and isinstance(c["reasons"], list)
-    # six library launches and one harness launch a step on this path
-    assert d["gpu_launches"] == 7 * 6
+    # five library launches (begin, append, the attention of all layers by the cluster pass, the
+    # loop-onset test, the compaction) and one harness launch a step
+    assert d["gpu_launches"] == 6 * 6
+    assert d["gpu_launches_detail"] == {"path_per_step": 5, "harness_per_step": 1}
+
+
+@pytest.mark.parametrize("extra,path", [
+    (["--layers-per-call", "10"], 4 + 4),               # 32 layers in calls of 10, 10, 10 and 2
+    (["--policy", "h2o"], 4 + 2),                       # attention and the score update
+    (["--workload", "1"], 4 + 1)])                      # fp32
+def test_launches_are_those_of_the_pass_taken(extra, path):
+    args = ["--workload", "2", "--batch", "2", "--steps", "4", "--warmup", "3", "--no-e2e",
+            "--no-cpu-baseline", *extra]
+    d = _line(*args)
+    assert d["gpu_launches_detail"]["path_per_step"] == path
+    assert d["gpu_launches"] == (path + 1) * 4
 
 
 @pytest.mark.parametrize("extra", [["--detector", "kv"], ["--detector", "token"],
