@@ -59,30 +59,44 @@ def test_attend_empty_and_boundary_lengths(cuda, dtype):
                 assert_close(st[layer, b, hs], s_ref, *STAT_TOL, what=tag + " stats")
 
 
-def test_pass_direction_changes_no_result(cuda):
-    """successive lg_decode_attend calls with one workspace walk the cache in opposite
-    directions; the same inputs give bit-identical outputs and statistics, with the H2O score
-    accumulation both off and on (ragged lengths, several chunks per group)"""
+@pytest.mark.parametrize("pad", [0, 60])  # the cluster pass, which has no direction; the persistent
+def test_pass_direction_changes_no_result(cuda, pad):
+    """successive lg_decode_attend calls with one workspace walk the cache in opposite directions
+    where they run the persistent pass (here past 64 sequences, by empty ones); the same inputs
+    give bit-identical outputs and statistics, with the H2O score accumulation both off and on
+    (ragged lengths, several chunks per group)"""
     w = synth.make_workload(4, L=2, batch=5, len_range=(40, 5000), budget_max=8192, steps=1,
                             onset_max=1, periods=(4, 8))
     K, V = synth.host_cache(w)
+    batch = w.batch + pad
+    rows = np.zeros(K.shape[:2] + (pad,) + K.shape[3:], K.dtype)
+    k, v = (lg.host_to_device(np.concatenate([x, rows], 2), cuda, w.dtype) for x in (K, V))
+    off = np.concatenate([w.seq_off, K.shape[2] + np.arange(pad)])
+    cap = np.concatenate([w.cap, np.ones(pad, w.cap.dtype)])
+    n0 = np.concatenate([w.n0, np.zeros(pad, w.n0.dtype)])
     for h2o in (0, 1):
-        cache = lg.Cache.from_host(w, K, V, cuda, policy="h2o" if h2o else "loopguard")
+        cache = lg.Cache(w.L, w.H_kv, w.d, w.dtype, off, cap, n0, cuda,
+                         "h2o" if h2o else "loopguard", k, v)
         max_len = int(w.n0.max())
-        if h2o:
-            lg.lg_h2o_reset(cache, max_len)
+        cache.prepare(max_len)
         q, _, _ = synth.host_step(w, w.n0.astype(np.int64))
+        q = np.concatenate([q, np.zeros((w.L, pad) + q.shape[2:], q.dtype)], 1)
         qd = lg.host_to_device(q, cuda, "bf16")
-        ws = torch.empty(lg.lg_workspace_size(cache, w.H_q, w.L, max_len, h2o) // 4 + 64,
-                         dtype=torch.float32, device=cuda)
-        runs = []
+        size = lg.lg_workspace_size(cache, w.H_q, w.L, max_len, h2o)
+        ws = torch.empty(size // 4 + 64, dtype=torch.float32, device=cuda)
+        # the counters end the workspace: the chunk counter, one per group, the direction
+        counters = (2 + w.L * batch * w.H_kv) * 4
+        direction = ws.view(torch.int32)[(size - -(-counters // 256) * 256 + counters) // 4 - 1]
+        runs, ways = [], []
         for _ in range(2):
-            out = torch.zeros((w.L, w.batch, w.H_q, w.d), dtype=torch.bfloat16, device=cuda)
-            stats = torch.zeros((w.L, w.batch, w.H_q, 4), dtype=torch.float32, device=cuda)
+            out = torch.zeros((w.L, batch, w.H_q, w.d), dtype=torch.bfloat16, device=cuda)
+            stats = torch.zeros((w.L, batch, w.H_q, 4), dtype=torch.float32, device=cuda)
             lg.lg_decode_attend(cache, 0, w.L, qd, w.H_q, 1.0 / np.sqrt(w.d), out, stats, 64,
                                 h2o, max_len, ws)
             torch.cuda.synchronize()
             assert lg.lg_read_device_status(cache) == 0
             runs.append((out.cpu(), stats.cpu()))
+            ways.append(int(direction) & 1)
+        assert (ways[0] != ways[1]) == (pad > 0), ways
         assert torch.equal(runs[0][0], runs[1][0]), h2o
         assert torch.equal(runs[0][1], runs[1][1]), h2o

@@ -39,11 +39,17 @@ def _valid_rows(x, w, lens):
     return torch.cat(parts)
 
 
+# a batch that the cluster pass takes, and one past its 64 sequences: the persistent pass, whose
+# counter reset, chunk counters and direction word are then part of every step
+SMALL = dict(batch=4, n=1200, budget=768, tail=(300, 500), periods=(8, 40))
+LARGE = dict(batch=66, n=300, budget=256, tail=(80, 120), periods=(8, 24))
+
+
+@pytest.mark.parametrize("size", [SMALL, LARGE], ids=["batch4", "batch66"])
 @pytest.mark.parametrize("policy,detector", [("loopguard", "kv"), ("loopguard", "token"),
                                              ("h2o", "kv"), ("streaming", "kv")])
-def test_graph_replay_matches_eager(cuda, policy, detector):
-    w = synth.make_workload(2, L=2, batch=4, n=1200, budget=768, steps=40, tail=(300, 500),
-                            periods=(8, 40))
+def test_graph_replay_matches_eager(cuda, policy, detector, size):
+    w = synth.make_workload(2, L=2, steps=40, **size)
     K = 24
     side = torch.cuda.Stream(device=cuda)
     with torch.cuda.stream(side):

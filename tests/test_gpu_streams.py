@@ -2,8 +2,9 @@
 state, stepped concurrently on two CUDA streams with their launches interleaved: each must
 match its own oracle at every step (attention outputs and statistics within the parity
 tolerances; flags, spans, lengths, kept lists and compacted rows exactly).  The library keeps no
-state between calls outside the caller's buffers (the pass direction and the chunk counters
-live in each call's workspace), so neither batch may see the other."""
+state between calls outside the caller's buffers (the persistent pass, which batches of more than 64
+sequences run, keeps its direction and its chunk counters in each call's workspace), so neither
+batch may see the other."""
 import numpy as np
 import pytest
 import torch
@@ -18,10 +19,17 @@ pytestmark = pytest.mark.gpu
 STEPS = 10
 
 
-def test_two_batches_on_two_streams(cuda):
-    ws = [synth.make_workload(2, L=2, batch=3, n=700, budget=512, steps=STEPS, tail=(200, 300),
-                              periods=(6, 20)),
-          synth.make_workload(3, L=2, batch=4, n=900, budget=384, steps=STEPS, periods=(8, 16))]
+# two batches for the cluster pass, two for the persistent pass, one of each
+SMALL = [(2, dict(L=2, batch=3, n=700, budget=512, tail=(200, 300), periods=(6, 20))),
+         (3, dict(L=2, batch=4, n=900, budget=384, periods=(8, 16)))]
+LARGE = [(2, dict(L=1, batch=66, n=150, budget=128, tail=(50, 70), periods=(5, 12))),
+         (3, dict(L=2, batch=70, n=160, budget=96, periods=(4, 8)))]
+
+
+@pytest.mark.parametrize("pair", [SMALL, LARGE, [SMALL[1], LARGE[0]]],
+                         ids=["cluster", "persistent", "one of each"])
+def test_two_batches_on_two_streams(cuda, pair):
+    ws = [synth.make_workload(number, steps=STEPS, **over) for number, over in pair]
     streams = [torch.cuda.Stream(device=cuda), torch.cuda.Stream(device=cuda)]
     prm_o, prm_g = oracle.params(), lg.lg_default_params()
     refs, caches, guards, budgets = [], [], [], []

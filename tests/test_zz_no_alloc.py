@@ -5,8 +5,10 @@ take cudaMalloc's implicit synchronisation).  Its scratch is a static array of t
 Checked through the C ABI on two calls in a row (the second reuses the array the first left
 behind), within the parity tests' tolerances, against both the CPU oracle (attention, Eq. 1,
 with its statistics) and lg_decode_attend with a caller workspace:
-  - the bf16 tensor-core path (GQA 4, three layers in one call);
-  - the fp32 path at head_dim 64 (a partial kernel and a merge kernel, both on the array);
+  - the bf16 tensor-core path (GQA 4, three layers in one call) by the cluster pass, and past 64
+    sequences by the persistent pass, with its counters and partials on the array;
+  - the fp32 path by the cluster pass (head_dim 64), and past 64 sequences by a partial kernel and a
+    merge kernel, both on the array;
   - the H2O accumulation (the logits kept in the array between the pass and the score
     update): accumulated scores within 1e-4 relative of the oracle's after each call.
 This file is collected last so that a run stopping at the first failure has run every other
@@ -80,6 +82,15 @@ def test_noalloc_bf16_twice(cuda):
 
 def test_noalloc_fp32_head_dim_64_twice(cuda):
     w = synth.make_workload(1, n=700, loop_len=192, budget=512)
+    _two_calls(w, cuda, "loopguard", 0)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_noalloc_past_64_sequences_twice(cuda, dtype):
+    w = synth.make_workload(2, L=1, batch=66, n=300, budget=256, steps=2, tail=(60, 90),
+                            periods=(10, 30), H_kv=2, H_q=8)
+    w.dtype = dtype
+    w.__post_init__()
     _two_calls(w, cuda, "loopguard", 0)
 
 
