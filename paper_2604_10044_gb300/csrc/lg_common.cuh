@@ -18,9 +18,10 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;
 // kernel before it in the stream is still running.  Each kernel therefore starts with
 // pdl_enter(): griddepcontrol.wait returns once the kernels it depends on have completed and
 // their memory is visible (at once when there is no such kernel), so nothing of the kernel
-// touches global memory before its predecessor is done; launch_dependents then lets the
-// next kernel be scheduled early in turn, and it waits the same way.  Completion is
-// transitive: the predecessor itself passed its wait only after its own predecessor was done.
+// touches global memory before its predecessor is done (two early readers apart: the loop-onset
+// test and the cluster pass, below); launch_dependents then lets the next kernel be scheduled
+// early in turn, and it waits the same way.  Completion is transitive: the predecessor itself
+// passed its wait only after its own predecessor was done.
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -29,10 +30,13 @@ __device__ __forceinline__ void pdl_enter() {
 // The same for a short kernel in front of a long one's launch (the slot reservation, the append,
 // the counter reset): the next kernel may be scheduled before this one's own wait is over, so
 // that its launch and prologue overlap the kernel before this one too.  The next kernel still
-// touches memory only once this kernel is complete, which it is only after its own wait.  The
-// one early reader, the loop-onset test, re-checks the length, the synced length and the newest
-// row after its wait, which covers the slot reservation and the append; every other kernel that
-// may change what it reads early triggers only after its own wait.
+// touches memory only once this kernel is complete, which it is only after its own wait.  Two
+// kernels read before their wait, and past L1.  The loop-onset test re-checks the length, the synced
+// length and the newest row after it, which covers the slot reservation and the append; every other
+// kernel that may change what it reads early triggers only after its own wait.  The attention's
+// cluster pass takes the lengths and offsets it finds as hints alone, for prefetches into L2 and for
+// which rows it copies first after its wait; it reads them again then, and drops what they do not
+// confirm.
 // (GB300, layers called one by one in a graph, one sequence of 1024 rows, append and attention:
 // 12.3 -> 11.5 us a layer with the persistent pass, 7.30 -> 7.16 us with the cluster pass.)
 __device__ __forceinline__ void pdl_enter_early() {

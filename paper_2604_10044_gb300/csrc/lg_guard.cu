@@ -967,7 +967,7 @@ struct EvictStream {
   float *sc;             // scores of the stream's slots
   int32_t *ps;           // their positions
   unsigned char *K, *V;  // their rows
-  int n, B;              // rows in use, budget
+  int n;                 // rows in use
   int32_t thrp;          // recent: position above this one
   int n_sink;
   template <int kMode>
@@ -1210,7 +1210,6 @@ __global__ void __launch_bounds__(kH2OThreads, 4) evict_kernel(lg_cache c, const
   e.K = (unsigned char *)c.k + o * rb;
   e.V = (unsigned char *)c.v + o * rb;
   e.n = n;
-  e.B = B;
   // recent: pos > thrp (H2O: the newest B/2 positions; streaming: the newest B - n_sink)
   e.thrp = now - (kMode == kEvictH2O ? B / 2 : B - n_sink);
   e.n_sink = n_sink;
