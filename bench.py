@@ -67,6 +67,10 @@ def parse():
     ap.add_argument("--no-clocks", action="store_true")
     ap.add_argument("--batch", type=int, default=0,
                     help="override the workload's batch (smaller cases for profiling)")
+    ap.add_argument("--layers", type=int, default=0,
+                    help="override the workload's layers (--profile-steps: smaller cases)")
+    ap.add_argument("--rows", type=int, default=0,
+                    help="override the rows of each sequence (--profile-steps: smaller cases)")
     ap.add_argument("--policy", default="loopguard",
                     choices=["loopguard", "h2o", "streaming", "full"],
                     help="cache policy of the timed steps: LoopGuard, or a comparator on the "
@@ -591,6 +595,11 @@ def gpu_workload(args, rank=0):
         over["seed"] = 1000 + rank
     if args.batch:
         over["batch"] = args.batch
+    if args.profile_steps and args.layers:
+        over["L"] = args.layers
+    if args.profile_steps and args.rows:
+        over["n"] = args.rows
+        over["tail"] = args.rows // 8                 # of the bandwidth sweep's loops
     return synth.make_workload(args.workload, **over)
 
 
@@ -614,7 +623,7 @@ def run_gpu(args, ws, rank, local):
         torch.cuda.synchronize()
         torch.cuda.nvtx.range_pop()
         # K/V rows each step's attention launch reads (for the DRAM-traffic summary)
-        print(json.dumps({"workload": args.workload, "batch": w.batch,
+        print(json.dumps({"workload": args.workload, "batch": w.batch, "layers": w.L,
                           "attend_rows_per_launch": rows,
                           "attend_alg_bytes_per_launch": [
                               attend_bytes(w, np.full(w.batch, 0)) + 2 * w.d * w.esize * r
@@ -742,19 +751,17 @@ def run_gpu(args, ws, rank, local):
     value = sum_over_ranks(K, ws) / (ms * 1e-3)
     step_read = sum(a_bytes) / max(1, len(a_bytes))
     path_l, harness_l = bench.launches_per_step()
-    # DRAM bytes of one attention launch of the sampled steps, from the committed capture of
-    # this workload on the current kernel code (scaled by the rows a launch reads: the sampled
-    # steps' lengths differ from the captured launch's by a few rows); else null
+    # DRAM bytes of one attention launch of the sampled steps: its algorithmic bytes times what the
+    # committed capture of a smaller call of the same kernel has per algorithmic byte; else null
     prof = traffic_from_profile(source_hash())
-    traffic, traffic_note = None, "no DRAM capture of this workload on the current kernel code"
-    sampled_rows = [w.L * w.H_kv * int(np.sum(lens[t].cpu().numpy() + 1)) for t in sampled]
-    if (prof and bench.nl == w.L and prof.get("workload") == args.workload
-            and prof.get("batch") == w.batch and args.policy == "loopguard"):
-        rows = sum(sampled_rows) / len(sampled_rows)
-        traffic = int(prof["dram_bytes"] * rows / prof["rows"])
-        traffic_note = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the attention launch "
-                        "of %s (profiles/attend_mma_traffic.txt), scaled by %.6f for the rows "
-                        "of the sampled steps" % (prof["launch"], rows / prof["rows"]))
+    alg = sum(a_bytes[t] for t in sampled) / len(sampled)
+    traffic, traffic_note = None, "no DRAM capture of this kernel on its current code"
+    if prof and bench.nl == w.L and prof.get("workload") == args.workload \
+            and not args.batch and args.policy == "loopguard":
+        traffic = int(alg * prof["dram_bytes"] / prof["alg_bytes"])
+        traffic_note = ("the launch's algorithmic bytes times %.4f, the DRAM bytes per algorithmic "
+                        "byte of %s (profiles/attend_mma_traffic.txt)"
+                        % (prof["dram_bytes"] / prof["alg_bytes"], prof["launch"]))
     line = {
         "metric": METRIC, "value": round(value, 3), "unit": UNIT, "n_gpus": ws, "steps": K,
         "warmup": W, "ms_per_step": round(ms / K, 4), "higher_is_better": True,
@@ -767,7 +774,7 @@ def run_gpu(args, ws, rank, local):
         "roofline": {"bound": "hbm", "achieved": round(attend_gbs, 1), "peak": hbm_peak,
                      "unit": "GB/s", "frac": round(attend_gbs / hbm_peak, 4),
                      "traffic": traffic, "traffic_note": traffic_note,
-                     "alg_bytes_per_launch": int(sum(a_bytes[t] for t in sampled) / len(sampled)),
+                     "alg_bytes_per_launch": int(alg),
                      "kernel": "lg_decode_attend (tensor-core pass with its split-K merge), all "
                                "%d layers per call" % w.L if bench.nl == w.L
                                else "lg_decode_attend",
