@@ -3,7 +3,8 @@
 // of the comparator policy (Sec. 2.2, Sec. 6.1), and the choice of a call's pass.
 //
 // The chunk kernel here serves the fp32 calls that the cluster pass (lg_attend_cluster.cuh) does
-// not take: more than 64 sequences, the longest calls, and those that its rule finds faster here.
+// not take: more than 64 sequences, the longest calls, and those that are the faster here by their
+// sizes or lengths (lg_attend_rule.cuh).
 // One CTA streams CH consecutive rows of one (layer, sequence, kv-head) and serves all g query
 // heads of that kv-head, so every K/V byte is read from HBM once per step.  A producer warp moves
 // 8 KB K and V tiles into a 4-stage shared-memory ring with 1-D bulk copies (TMA) completing on

@@ -15,9 +15,10 @@
 // a group's pieces in turn), each store counting its bytes on the owner's barrier; the owner
 // merges once all have arrived (a cluster barrier in its place waits for the stores'
 // acknowledgements first: 5.74 -> 5.58 us a layer at one sequence of 1024 rows, 32 sequences of
-// 128 9.70 -> 9.09).  No
-// counters, no workspace, no other launch.  Uneven lengths cost little: a CTA with less to read
-// leaves its bandwidth to the others (one CTA streams up to 90 GB/s, 1.8 times its even share).
+// 128 9.70 -> 9.09).  No counters, no partials in memory, no other launch.  Uneven lengths cost
+// little while groups outnumber the clusters: a CTA with less to read leaves its bandwidth to the
+// others (one CTA streams up to 90 GB/s, 1.8 times its even share).  A few long groups, which have
+// at most 8 CTAs each, are the general passes' (lg_attend_rule.cuh).
 //
 // GB300, one layer of 28 (append and attention, called one by one in a graph), one sequence of
 // 1024 rows, 16/8 heads of 128: 12.0 -> 5.6 us.  Of a CTA's 4.1 us after its wait, 1.6 go to its

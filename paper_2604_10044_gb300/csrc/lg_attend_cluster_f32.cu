@@ -7,8 +7,9 @@
 // probabilities are passed back by shuffles.  Up to 4 heads the memory bounds a call; at 5 to 8
 // the chains of dependent shuffles and FMAs do, of which two to four rows run side by side.
 // GB300, one layer (append and attention), 268 MB, 4 sequences of 8191 rows, 8 kv-heads of 128,
-// against the chunk kernel with its separate combine: 1 head a group 80.8 -> 41.4 us, 4 heads
-// 91.1 -> 45.4, 8 heads 108.0 -> 76.1.  Not kept: a lane a row with the query rows broadcast from
+// against the chunk kernel with its separate combine: 1 head a group 80.8 -> 41.5 us, 4 heads
+// 91.1 -> 44.9, 8 heads 108.0 -> 72.5 (77.7 with the chunk kernel launched after it, as lengths in
+// such slots can make that the faster).  Not kept: a lane a row with the query rows broadcast from
 // shared memory (its datapath moves 512 bytes for a broadcast too: 54 and 80 us at 4 and 8 heads).
 #include "lg_attend_cluster.cuh"
 
@@ -41,7 +42,7 @@ struct Pass<float, D, G> {
   // memory, which keeps the chains of dependent roundings short: a lane takes hundreds of rows of a
   // long call.  Distance of the output from 64 bits (2-norm, normal rows; the chunk kernel /
   // without flushes / with): 4 sequences of 8191, 4 heads 2.65e-7 / 2.82e-7 / 2.16e-7, one of
-  // 131071, 8 heads 4.4e-7 / 8.4e-7 / 2.6e-7.  It costs 2 % of the time (44.4 -> 45.4 us, above).
+  // 131071, 8 heads 4.4e-7 / 8.4e-7 / 2.6e-7.  It cost 2 % of the time when it came (44.4 -> 45.4 us, above).
   static constexpr int kFlushTiles = 32 * kRpw / kRows;
   static_assert(kGP <= kLpr && kRows % (kSteps * kRpw) == 0, "lanes for the heads, whole steps");
 
