@@ -172,10 +172,11 @@ __device__ __forceinline__ void load_q(uint32_t (&qf)[D / 16][2], const unsigned
 // to its length: with a segment's 342 blocks in one chain (2 sequences of 131071 rows, 8 heads a
 // group, clusters of 6) the output was 1.28e-5 of its norm off the 64-bit value before its rounding
 // to bf16, with this 2.36e-6; the persistent pass, whose chunks of 8 tiles keep the chains short,
-// has 2.40e-6 there (most of it P's two bf16 parts).  It costs nothing at one tile a CTA, 0 to 1 %
-// of most calls and 3.5 % where a CTA's own work bounds the call (1 sequence of 16384 rows, 4 heads:
-// 17.9 -> 18.5 us); flushes to shared memory every 16 blocks cost more (the long call above 157.0
-// -> 159.5 us, against 156.9).
+// has 2.40e-6 there (most of it P's two bf16 parts).  The additions follow all of a block's products,
+// so that none waits for its own (added after every four fragments: 18.6 us below).  It costs nothing
+// at one tile a CTA, 0 to 1.5 % of most calls and 2.5 % where a CTA's own work bounds the call (1
+// sequence of 16384 rows, 4 heads: 17.9 -> 18.3 us); flushes to shared memory every 16 blocks cost
+// more (the long call above 157.0 -> 159.5 us, against 156.9).
 template <int D, int G, int MB, bool kFresh>
 __device__ __forceinline__ void tile_update(WarpSums<D> &acc, const uint32_t (&qf)[D / 16][2],
                                             unsigned char *stage, int tile_rows, int suffix,
@@ -309,6 +310,7 @@ __device__ __forceinline__ void tile_update(WarpSums<D> &acc, const uint32_t (&q
 #pragma unroll
   for (int mb = 0; mb < MB; ++mb) {
     const int r = r_w + mb * 16 + (msel >> 1) * 8 + mrow;
+    float fresh[C::kKSteps][4];
 #pragma unroll
     for (int e0 = 0; e0 < C::kKSteps; e0 += 4) {
       uint32_t va[4][4];
@@ -316,23 +318,22 @@ __device__ __forceinline__ void tile_update(WarpSums<D> &acc, const uint32_t (&q
       for (int j = 0; j < 4; ++j)
         ldsm_x4_trans(vbase + (e0 >> 2) * kBoxBytes + swz(r, j * 2 + (msel & 1)), va[j][0],
                       va[j][1], va[j][2], va[j][3]);
-      float fresh[4][4];
 #pragma unroll
       for (int j = 0; j < 4; ++j)
         if (kFresh)
-          mma_bf16_zero(fresh[j], va[j][0], va[j][1], va[j][2], va[j][3], pb[mb][0], pb[mb][1]);
+          mma_bf16_zero(fresh[e0 + j], va[j][0], va[j][1], va[j][2], va[j][3], pb[mb][0], pb[mb][1]);
         else
           mma_bf16(o[e0 + j], va[j][0], va[j][1], va[j][2], va[j][3], pb[mb][0], pb[mb][1]);
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        mma_bf16(kFresh ? fresh[j] : o[e0 + j], va[j][0], va[j][1], va[j][2], va[j][3], pl[mb][0],
-                 pl[mb][1]);
-      if (kFresh) {
+        mma_bf16(kFresh ? fresh[e0 + j] : o[e0 + j], va[j][0], va[j][1], va[j][2], va[j][3],
+                 pl[mb][0], pl[mb][1]);
+    }
+    if (kFresh) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+      for (int eb = 0; eb < C::kKSteps; ++eb)
 #pragma unroll
-          for (int k = 0; k < 4; ++k) o[e0 + j][k] += fresh[j][k];
-      }
+        for (int k = 0; k < 4; ++k) o[eb][k] += fresh[eb][k];
     }
   }
   __syncwarp();
