@@ -126,22 +126,32 @@ def _kernel():
 def test_nothing_of_a_warp_branches_on_a_lanes_wait():
     """What follows a wait uses shuffles and matrix instructions of all lanes, and at the time limit a
     warp's lanes may see the barrier differently: so a wait that ran out sets a flag of the CTA and
-    the warp goes on together.  After that no copy is waited for, and the producer, which sees the
-    flag with any stage or query buffer handed back after it, arms none of their barriers again."""
+    the warp goes on together.  After that no copy is waited for, and the barriers that hand stages and
+    query buffers back are held before the warp arrives on them, so that the producer arms none again."""
     producer, code = _kernel()
     landed = re.search(r"auto landed = [^{]*\{(.*?)\n  \};", code, re.S).group(1)
     assert re.sub(r"\s+", " ", landed).strip() == \
         "if (!mbar_try_wait(bar, parity) && !stopped() && !mbar_wait(bar, parity)) ran_out();"
-    assert "s_stop, 2" in re.search(r"auto ran_out = [^{]*\{(.*?)\n  \};", code, re.S).group(1)
+    ran_out = re.search(r"auto ran_out = [^{]*\{(.*?)\n  \};", code, re.S).group(1)
+    assert "s_stop, 2" in ran_out
+    assert "s < Cl::kStages; ++s) mbar_hold(&empty_bar[s])" in ran_out
+    assert "s < 2; ++s) mbar_hold(&q_empty[s])" in ran_out
     for use in re.finditer(r"[^;{}]*(pass\.begin|pass\.update|landed)\(&?[^;]*;", code):
         assert "if (" not in use.group(0) or "P::" in use.group(0), use.group(0)
     skip = code[code.index("if (s_skip > 0)"):code.index("for (int t = u0;")]
     assert "in = in && mbar_wait(&full_bar[it], 0);" in skip and "if (!in) ran_out();" in skip
     # (those two, the one in landed() and the one of the pieces)
     assert len(re.findall(r"\bmbar_wait(?:_cluster)?\(", code)) == 4
+    # the wait for a stage's copy, then its work, then the arrival that hands it back
+    tile = code[code.index("for (; t < stop;"):]
+    assert tile.index("landed(&full_bar[st]") < tile.index("pass.update(") < \
+        tile.index("mbar_arrive(&empty_bar[st])")
+    assert skip.index("ran_out();") < skip.index("mbar_arrive(&empty_bar[it])")
     for bar in ("empty_bar", "q_empty"):
-        wait = re.search(r"timed_out\(&%s\[[^;{]*\{" % bar, producer).group(0)
-        assert "|| stopped()" in wait, wait
+        assert re.search(r"timed_out\(&%s\[" % bar, producer)
+    text = open(SRC).read()
+    hold = text[text.index("void mbar_hold("):]
+    assert "mbarrier.expect_tx" in hold[:hold.index("}")]
 
 
 def test_a_cta_outlives_what_is_sent_to_it():
